@@ -20,7 +20,13 @@
 // factored block by block (16 x 16 Cholesky factors L_k, L_k^-1 E_k) and the border is taken
 // through its Schur complement. The dynamics' Jacobian per grid point comes from forward-mode
 // differentiation (value and one derivative per pass, 16 passes). Everything is FP64: a
-// cluster of two CTAs of 512 threads per trajectory.
+// cluster of two, four or eight CTAs of 512 threads per trajectory.
+//
+// What bounds it: the FP64 pipe, where a warp instruction holds an SM for about 19 cycles, so
+// the work is laid out to issue few of them. Rows 0-9 of df/dw are constant (the rates and the
+// inputs), so only rows 10 and 11 are stored and every sum over the 12 rows takes the terms
+// that are not zero; the quotients by rho and 2N are formed once per entry; the block factor
+// carries the right-hand sides as further rows on the lanes that a 16-row factor leaves idle.
 #include <cmath>
 #include <new>
 
@@ -39,10 +45,11 @@ namespace cp {
 namespace {
 
 constexpr int kTrajThreads = 512;
-constexpr int kTrajCtas = 2;      // CTAs (one thread-block cluster) per trajectory
+constexpr int kSumCtas = 2;       // CTAs of a cluster that take the team sums (see Team)
 constexpr int kRedDoubles = 64;   // block reductions: [0, 32) and [32, 64) (one slot per warp)
-constexpr int kWarpScratch = 2 * 12 * 16;   // doubles of shared memory per warp (block factor, F_k pair)
 constexpr int NX = 12, NU = 4, NW = 16;
+constexpr int NF = 2;             // dense rows of df/dw (rows NX - NF .. NX - 1)
+constexpr int kWarpScratch = 3 * NW * NW;   // doubles of shared memory per warp (three blocks)
 constexpr double kGravity = 9.81;
 
 // A value and one derivative (forward mode).
@@ -163,13 +170,17 @@ __device__ void traj_f(const TrajDev &td, const T *x, const T *u, T *out, const 
 // Per-trajectory device workspace (doubles), laid out by the launcher.
 struct TrajWs {
     double *f;     // [N+1][12]
-    double *Fj;    // [N+1][12][16] df/dw
+    double *Fj;    // [N+1][2][16] rows 10 and 11 of df/dw (row r < 10: 1 at column r + 6)
     double *D;     // [N+1][16][16] diagonal blocks, then their Cholesky factors
     double *E;     // [N][16][16] off-diagonal blocks, then L_k^-1 E_k
     double *bb;    // [N+1][16] border column, then the forward/back solves
     double *g;     // [N+1][16] gradient, then the forward/back solves
     double *P;     // [N+1][16][16] L_k^-1 T[k][left neighbour] of the eliminated blocks
     double *trig;  // [N+1][10] cosines and sines of the dynamics at the grid points of z
+    double *er;    // [N][12] d(defect)/dt_F
+    double *dr;    // [N][12] defect + lambda / rho
+    double *b0;    // [N+1][16] border column as assembled
+    double *lr;    // [N+2][12] lambda / rho
 };
 
 __device__ __forceinline__ TrajWs ws_of(double *base, int N)
@@ -177,32 +188,44 @@ __device__ __forceinline__ TrajWs ws_of(double *base, int N)
     TrajWs w;
     w.f = base;
     w.Fj = w.f + (size_t)(N + 1) * NX;
-    w.D = w.Fj + (size_t)(N + 1) * NX * NW;
+    w.D = w.Fj + (size_t)(N + 1) * NF * NW;
     w.E = w.D + (size_t)(N + 1) * NW * NW;
     w.bb = w.E + (size_t)N * NW * NW;
     w.g = w.bb + (size_t)(N + 1) * NW;
     w.P = w.g + (size_t)(N + 1) * NW;
     w.trig = w.P + (size_t)(N + 1) * NW * NW;
+    w.er = w.trig + (size_t)(N + 1) * 10;
+    w.dr = w.er + (size_t)N * NX;
+    w.b0 = w.dr + (size_t)N * NX;
+    w.lr = w.b0 + (size_t)(N + 1) * NW;
     return w;
 }
 
-// The CTAs of one trajectory: a cluster of kTrajCtas CTAs on neighbouring SMs. Grid points,
+// The CTAs of one trajectory: a cluster of 2, 4 or 8 CTAs on neighbouring SMs. Grid points,
 // entries and blocks are split over the team-wide thread or warp index. Data one CTA writes to
 // the trajectory's global workspace is read by the other only after team_sync(), a cluster
 // barrier with release / acquire semantics. Every thread of both CTAs passes the same
 // sequence of them: no barrier sits under a branch whose condition the CTAs could see
-// differently (the sums below give both the same values).
+// differently (the sums below give all the same values). Sums over the trajectory are taken by
+// the first kSumCtas CTAs alone, whatever the cluster's size, so that their order, and with it
+// every bit of the solution, does not depend on how many trajectories share the GPU; they are
+// under 2% of the work.
 struct Team {
     int rank;   // this CTA's rank in the cluster
+    int ctas;   // CTAs in the cluster
     __device__ int tid() const { return rank * (int)blockDim.x + (int)threadIdx.x; }
-    __device__ int nthreads() const { return kTrajCtas * (int)blockDim.x; }
+    __device__ int nthreads() const { return ctas * (int)blockDim.x; }
     __device__ int warp() const { return tid() >> 5; }
     __device__ int nwarps() const { return nthreads() >> 5; }
+    // this thread's first term and the stride of a team sum (no term on the other CTAs)
+    __device__ int sum_first(int n) const { return rank < kSumCtas ? tid() : n; }
+    __device__ int sum_stride() const { return kSumCtas * (int)blockDim.x; }
 };
 
 __device__ __forceinline__ Team team_of_block()
 {
-    return Team{(int)cooperative_groups::this_cluster().block_rank()};
+    const cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    return Team{(int)cl.block_rank(), (int)cl.num_blocks()};
 }
 
 __device__ __forceinline__ void team_sync()
@@ -210,9 +233,9 @@ __device__ __forceinline__ void team_sync()
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
-// Sums of a and b over both CTAs in a fixed order: per warp by shuffles, a CTA's warps in
-// order by its thread 0, then CTA 0's partial plus CTA 1's (read from each CTA's shared
-// memory), so every thread of both CTAs returns the same values (deterministic).
+// Sums of a and b over the two summing CTAs in a fixed order: per warp by shuffles, a CTA's
+// warps in order by its thread 0, then CTA 0's partial plus CTA 1's (read from each CTA's shared
+// memory), so every thread of the cluster returns the same values (deterministic).
 __device__ double2 team_sum2(double a, double b, double *s_red)
 {
     const int t = threadIdx.x;
@@ -258,14 +281,14 @@ __device__ void eval_f(const Team &tm, const TrajDev &td, const double *z, doubl
 
 // The merit F(z) = t_F + 1/2 |r(z)|^2 (T6): the AL terms of the defects and end states, the
 // effort and tracking sums over k = 1..N, and the bound penalty; f must be current for z.
-__device__ double merit(const Team &tm, const TrajDev &td, const double *z, const double *lam, const double *q_star,
+__device__ double merit(const Team &tm, const TrajDev &td, const double *z, const double *lam_rho, const double *q_star,
                         const double *f, const double *x_S, const double *x_T, double *s_red)
 {
     const int N = td.N;
     const double h = z[0] / N;
     double acc = 0.0;
     // defects and end states: rho/2 (c + lam/rho)^2
-    for (int e = tm.tid(); e < NX * (N + 2); e += tm.nthreads()) {
+    for (int e = tm.sum_first(NX * (N + 2)); e < NX * (N + 2); e += tm.sum_stride()) {
         const int k = e / NX, i = e - k * NX;
         double c;
         if (k < N) {
@@ -276,11 +299,11 @@ __device__ double merit(const Team &tm, const TrajDev &td, const double *z, cons
         } else {
             c = z[1 + (size_t)N * NW + i] - x_T[i];
         }
-        const double t = c + lam[e] / td.rho;
+        const double t = c + lam_rho[e];
         acc += 0.5 * td.rho * t * t;
     }
     // effort, tracking and bounds per grid point
-    for (int e = tm.tid(); e < (N + 1) * NW; e += tm.nthreads()) {
+    for (int e = tm.sum_first((N + 1) * NW); e < (N + 1) * NW; e += tm.sum_stride()) {
         const int k = e / NW, i = e - k * NW;
         const double v = z[1 + e];
         if (i < NX) {
@@ -298,54 +321,65 @@ __device__ double merit(const Team &tm, const TrajDev &td, const double *z, cons
     return z[0] + team_sum(acc, s_red);
 }
 
-// Cholesky factor of a 16 x 16 SPD block on one warp (all 32 lanes call; lanes 0-15 hold a
-// row each in registers): the lower triangle of A in, F = the factor's strict lower triangle
-// with 1 / L_pp on its diagonal out (shared memory of the warp). Each pivot's reciprocal square
-// root comes from rsqrt_pivot; the column is scaled by it and the trailing rows updated from
-// shuffled entries, so a pivot costs one short chain of dependent FP64 operations.
-__device__ __noinline__ void warp_factor16(const double *A, double *F, int lane)
+// Elimination of one 16 x 16 SPD block A = L L^T on one warp, with its right-hand sides riding
+// along: P = L^-1 Tl, Q = L^-1 Tr and y = L^-1 f for the two vectors. A row of a right-hand
+// side's transpose takes the same operations as a row of A below the pivot, so the lanes hold
+//   lanes 0-15   row i of A, and column i of Tr;
+//   lanes 16-31  column c of Tl, and (lanes 16, 17) the two vectors,
+// one row in each of two register sets: per pivot one reciprocal square root (rsqrt_pivot), one
+// scaling and one FMA per later column and set, with the pivot's column from shuffles. That is
+// about 400 FP64 warp instructions and one chain of 16 pivots where the factor followed by three
+// column solves took 710 and three more chains. Tl is the transpose of Tl_rows (row-major
+// 16 x 16); Q overwrites Tr, the vectors are solved in place, and A's block receives the strict
+// lower triangle of L with 1 / L_pp on the diagonal. P, Tl_rows or Tr may be null.
+__device__ __noinline__ void warp_eliminate16(double *A, const double *Tl_rows, double *P, double *Tr, double *f_y,
+                                              double *f_v, int lane)
 {
     const unsigned full = 0xffffffffu;
     const int i = lane & (NW - 1);
-    double a[NW], rin[NW];
+    const bool low = lane < NW;
+    double *f = lane == NW ? f_y : f_v;
+    double a[NW], b[NW], diag = 0.0;
 #pragma unroll
-    for (int j = 0; j < NW; ++j) a[j] = j <= i ? A[i * NW + j] : 0.0;
+    for (int j = 0; j < NW; ++j) {
+        a[j] = low ? (j <= i ? A[i * NW + j] : 0.0) : (Tl_rows != nullptr ? Tl_rows[i * NW + j] : 0.0);
+        b[j] = low ? (Tr != nullptr ? Tr[j * NW + i] : 0.0) : (i < 2 ? f[j] : 0.0);
+    }
 #pragma unroll
     for (int p = 0; p < NW; ++p) {
         const double d = __shfl_sync(full, a[p], p);   // the pivot, from lane p
         const double r = rsqrt_pivot(d);
-        rin[p] = r;
-        const double l = i > p ? a[p] * r : (i == p ? d * r : 0.0);   // L[i][p]
+        double l = a[p] * r;                            // L[i][p], or P[p][i]
+        if (low && i <= p) l = i == p ? d * r : 0.0;
+        if (lane == p) diag = r;
         a[p] = l;
+        const double l2 = b[p] * r;
+        b[p] = l2;
 #pragma unroll
         for (int j = p + 1; j < NW; ++j) {
-            const double lj = __shfl_sync(full, l, j);                // L[j][p]
-            if (j <= i) a[j] = fma(-l, lj, a[j]);
+            const double lj = __shfl_sync(full, l, j);  // L[j][p]
+            a[j] = fma(-l, lj, a[j]);
+            b[j] = fma(-l2, lj, b[j]);
         }
     }
-    if (lane < NW) {
+    __syncwarp();
+    if (low) {
 #pragma unroll
-        for (int j = 0; j < NW; ++j) F[i * NW + j] = j < i ? a[j] : (j == i ? rin[i] : 0.0);
+        for (int j = 0; j < NW; ++j) A[i * NW + j] = j < i ? a[j] : (j == i ? diag : 0.0);
+    } else if (P != nullptr) {
+#pragma unroll
+        for (int j = 0; j < NW; ++j) P[j * NW + i] = a[j];
+    }
+    if (low) {
+        if (Tr != nullptr) {
+#pragma unroll
+            for (int j = 0; j < NW; ++j) Tr[j * NW + i] = b[j];
+        }
+    } else if (i < 2) {
+#pragma unroll
+        for (int j = 0; j < NW; ++j) f[j] = b[j];
     }
     __syncwarp();
-}
-
-// dst <- L^-1 src for one right-hand side of this lane (entry rr at src[rr * ss], written to
-// dst[rr * ds]), L in the form of warp_factor16: column by column, a chain of two dependent
-// operations per column.
-__device__ __noinline__ void column_solve16(const double *F, const double *src, int ss, double *dst, int ds)
-{
-    double x[NW];
-#pragma unroll
-    for (int rr = 0; rr < NW; ++rr) x[rr] = src[rr * ss];
-#pragma unroll
-    for (int q = 0; q < NW; ++q) {
-        x[q] *= F[q * NW + q];
-#pragma unroll
-        for (int r = q + 1; r < NW; ++r) x[r] = fma(-F[r * NW + q], x[q], x[r]);
-    }
-#pragma unroll
-    for (int rr = 0; rr < NW; ++rr) dst[rr * ds] = x[rr];
 }
 
 // x_k = L_k^-T (w_k - P_k x_l - Q_k x_r) for both vectors (lanes 0-15 y, 16-31 v, one row
@@ -393,7 +427,7 @@ __device__ __noinline__ void warp_back16(const double *Lk, const double *P, cons
 // The damped Gauss-Newton step dz at z (T6): Jacobian, assembly, block factorisation, solve.
 // dz_local: dz is this CTA's shared-memory copy, which gets every entry; otherwise it is one
 // global vector whose entries the team splits.
-__device__ void lm_step(const Team &tm, const TrajDev &td, const double *z, const double *lam, const double *q_star,
+__device__ void lm_step(const Team &tm, const TrajDev &td, const double *z, const double *q_star,
                         const double *x_S, const double *x_T, double mu, const TrajWs &ws, double *dz, bool dz_local,
                         double *s_red, double *s_blk)
 {
@@ -409,24 +443,20 @@ __device__ void lm_step(const Team &tm, const TrajDev &td, const double *z, cons
         for (int i = 0; i < NX; ++i) x[i] = {w[i], i == j ? 1.0 : 0.0};
         for (int i = 0; i < NU; ++i) u[i] = {w[NX + i], NX + i == j ? 1.0 : 0.0};
         traj_f<Dual>(td, x, u, out, ws.trig + (size_t)k * 10);
-        for (int i = 0; i < NX; ++i) ws.Fj[((size_t)k * NX + i) * NW + j] = out[i].d;
+        for (int i = 0; i < NF; ++i) ws.Fj[((size_t)k * NF + i) * NW + j] = out[NX - NF + i].d;
+    }
+    // defect k: e_k = dd_k/dt_F = -(f_k + f_{k+1}) / (2N) and d_k + lam_k / rho
+    for (int e = t; e < N * NX; e += nt) {
+        const int k = e / NX, r = e - k * NX;
+        const double *w0 = z + 1 + (size_t)k * NW;
+        const double fs = ws.f[e] + ws.f[e + NX];
+        ws.er[e] = -fs / (2.0 * N);
+        ws.dr[e] = w0[NW + r] - w0[r] - 0.5 * h * fs + ws.lr[e];
     }
     team_sync();
     // 2. assembly. Defect k: d_k = x_{k+1} - x_k - h/2 (f_k + f_{k+1}), rows scaled by sqrt(rho):
     //    A_k = dd_k/dw_k = -[I 0] - h/2 Fj_k, B_k = dd_k/dw_{k+1} = [I 0] - h/2 Fj_{k+1},
     //    e_k = dd_k/dt_F = -(f_k + f_{k+1}) / (2N); residual sqrt(rho) (d_k + lam_k / rho).
-    auto Aent = [&](int k, int r, int i) -> double {   // A_k[r][i]
-        return (i == r ? -1.0 : 0.0) - 0.5 * h * ws.Fj[((size_t)k * NX + r) * NW + i];
-    };
-    auto Bent = [&](int k, int r, int i) -> double {   // B_k[r][i] (defect k, w_{k+1})
-        return (i == r ? 1.0 : 0.0) - 0.5 * h * ws.Fj[((size_t)(k + 1) * NX + r) * NW + i];
-    };
-    auto dres = [&](int k, int r) -> double {          // d_k[r] + lam_k[r] / rho
-        const double *w0 = z + 1 + (size_t)k * NW;
-        return w0[NW + r] - w0[r] - 0.5 * h * (ws.f[(size_t)k * NX + r] + ws.f[(size_t)(k + 1) * NX + r]) +
-               lam[(size_t)k * NX + r] / rho;
-    };
-    auto eres = [&](int k, int r) -> double { return -(ws.f[(size_t)k * NX + r] + ws.f[(size_t)(k + 1) * NX + r]) / (2.0 * N); };
     // Diagonal blocks (lower triangles) and off-diagonal blocks from F_k = df/dw at grid
     // point k (c = h/2, I' = [I 0] of 12 x 16): A_k = -(I' + c F_k), B_k = I' - c F_{k+1}, so
     //   A_k^T A_k = I'^T I' + c (I'^T F_k + F_k^T I') + c^2 F_k^T F_k,
@@ -434,27 +464,29 @@ __device__ void lm_step(const Team &tm, const TrajDev &td, const double *z, cons
     // (interior points take both, whose first-order terms cancel) and
     //   A_k^T B_k = -(I'^T I' - c I'^T F_{k+1} + c F_k^T I' - c^2 F_k^T F_{k+1}).
     const double c = 0.5 * h;
-    // one warp per grid point k: F_k and F_{k+1} staged in the warp's shared memory, then the
-    // 136 lower entries of D_k and the 256 of E_k
+    // one warp per grid point k: rows 10 and 11 of F_k and F_{k+1} staged in the warp's shared
+    // memory, then the 136 lower entries of D_k and the 256 of E_k. Row r < 10 of F adds 1 to a
+    // product's entry (r + 6, r + 6) and nothing elsewhere.
     {
         const int warp = tm.warp(), lane = threadIdx.x & 31, n_warps = tm.nwarps();
-        double *sF = s_blk + (size_t)(threadIdx.x >> 5) * kWarpScratch;   // [2][NX][NW]: F_k, F_{k+1}
-        const double *F0 = sF, *F1 = sF + NX * NW;
+        double *sF = s_blk + (size_t)(threadIdx.x >> 5) * kWarpScratch;   // [2][NF][NW]: F_k, F_{k+1}
+        const double *F0 = sF, *F1 = sF + NF * NW;
+        auto Fent = [&](const double *F, int r, int i) -> double {
+            return r < NX - NF ? (i == r + 6 ? 1.0 : 0.0) : F[(r - (NX - NF)) * NW + i];
+        };
         for (int k = warp; k <= N; k += n_warps) {
             __syncwarp();
-            for (int q = lane; q < 2 * NX * NW; q += 32)
-                sF[q] = (q < NX * NW || k < N) ? ws.Fj[(size_t)k * NX * NW + q] : 0.0;
+            for (int q = lane; q < 2 * NF * NW; q += 32)
+                sF[q] = (q < NF * NW || k < N) ? ws.Fj[(size_t)k * NF * NW + q] : 0.0;
             __syncwarp();
             for (int e = lane; e < NW * (NW + 1) / 2; e += 32) {
                 int i, j;
                 tri_index(e, i, j);
-                double f0 = 0.0, f1 = 0.0;
-                for (int r = 0; r < NX; r += 2) {
-                    f0 = fma(F0[r * NW + i], F0[r * NW + j], f0);
-                    f1 = fma(F0[(r + 1) * NW + i], F0[(r + 1) * NW + j], f1);
-                }
+                const bool one = i == j && i >= 6;
+                const double f0 = fma(F0[i], F0[j], one && (i & 1) == 0 ? 1.0 : 0.0);        // even rows
+                const double f1 = fma(F0[NW + i], F0[NW + j], one && (i & 1) != 0 ? 1.0 : 0.0);   // odd rows
                 const double ff = f0 + f1;
-                const double cross = (i < NX ? F0[i * NW + j] : 0.0) + (j < NX ? F0[j * NW + i] : 0.0);
+                const double cross = (i < NX ? Fent(F0, i, j) : 0.0) + (j < NX ? Fent(F0, j, i) : 0.0);
                 const double id = (i == j && i < NX) ? 1.0 : 0.0;
                 double v;
                 if (k == 0) v = id + c * cross + c * c * ff;
@@ -477,40 +509,46 @@ __device__ void lm_step(const Team &tm, const TrajDev &td, const double *z, cons
             if (k < N)
                 for (int e = lane; e < NW * NW; e += 32) {
                     const int i = e >> 4, j = e & (NW - 1);
-                    double p0 = 0.0, p1 = 0.0;
-                    for (int r = 0; r < NX; r += 2) {
-                        p0 = fma(F0[r * NW + i], F1[r * NW + j], p0);
-                        p1 = fma(F0[(r + 1) * NW + i], F1[(r + 1) * NW + j], p1);
-                    }
+                    const bool one = i == j && i >= 6;
+                    const double p0 = fma(F0[i], F1[j], one && (i & 1) == 0 ? 1.0 : 0.0);
+                    const double p1 = fma(F0[NW + i], F1[NW + j], one && (i & 1) != 0 ? 1.0 : 0.0);
                     const double id = (i == j && i < NX) ? 1.0 : 0.0;
-                    const double v = id - c * (i < NX ? F1[i * NW + j] : 0.0) + c * (j < NX ? F0[j * NW + i] : 0.0) -
+                    const double v = id - c * (i < NX ? Fent(F1, i, j) : 0.0) + c * (j < NX ? Fent(F0, j, i) : 0.0) -
                                      c * c * (p0 + p1);
                     ws.E[(size_t)k * NW * NW + e] = -rho * v;
                 }
         }
     }
-    // border column, gradient (stored negated: the solves below take -g)
+    // border column, gradient (stored negated: the solves below take -g): column i of A_k^T and
+    // B_{k-1}^T has entries in rows i - 6 (the constant rows of F), i and the two dense rows
     for (int e = t; e < (N + 1) * NW; e += nt) {
         const int k = e / NW, i = e - k * NW;
         double bv = 0.0, gv = 0.0;
-        if (k < N)
-            for (int r = 0; r < NX; ++r) {
-                const double a = Aent(k, r, i);
-                bv += a * eres(k, r);
-                gv += a * dres(k, r);
-            }
-        if (k > 0)
-            for (int r = 0; r < NX; ++r) {
-                const double bb = Bent(k - 1, r, i);
-                bv += bb * eres(k - 1, r);
-                gv += bb * dres(k - 1, r);
-            }
+        auto add = [&](double a, size_t at) {
+            bv = fma(a, ws.er[at], bv);
+            gv = fma(a, ws.dr[at], gv);
+        };
+        const double *Fk = ws.Fj + (size_t)k * NF * NW;
+        if (k < N) {   // A_k = -[I 0] - h/2 F_k
+            const size_t at = (size_t)k * NX;
+            if (i >= 6) add(-0.5 * h, at + i - 6);
+            if (i < NX - NF) add(-1.0, at + i);
+            add((i == NX - 2 ? -1.0 : 0.0) - 0.5 * h * Fk[i], at + NX - 2);
+            add((i == NX - 1 ? -1.0 : 0.0) - 0.5 * h * Fk[NW + i], at + NX - 1);
+        }
+        if (k > 0) {   // B_{k-1} = [I 0] - h/2 F_k
+            const size_t at = (size_t)(k - 1) * NX;
+            if (i >= 6) add(-0.5 * h, at + i - 6);
+            if (i < NX - NF) add(1.0, at + i);
+            add((i == NX - 2 ? 1.0 : 0.0) - 0.5 * h * Fk[i], at + NX - 2);
+            add((i == NX - 1 ? 1.0 : 0.0) - 0.5 * h * Fk[NW + i], at + NX - 1);
+        }
         bv *= rho;
         gv *= rho;
         const double x = z[1 + e];
         if (i < NX) {
-            if (k == 0) gv += rho * (x - x_S[i] + lam[(size_t)N * NX + i] / rho);
-            if (k == N) gv += rho * (x - x_T[i] + lam[(size_t)(N + 1) * NX + i] / rho);
+            if (k == 0) gv += rho * (x - x_S[i] + ws.lr[(size_t)N * NX + i]);
+            if (k == N) gv += rho * (x - x_T[i] + ws.lr[(size_t)(N + 1) * NX + i]);
             const double viol = x > td.x_max[i] ? x - td.x_max[i] : (x < td.x_min[i] ? x - td.x_min[i] : 0.0);
             gv += td.rho_b * viol;
             if (i < 4 && k >= 1) gv += 2.0 * td.omega_t * (x - q_star[(size_t)k * 4 + i]);
@@ -518,15 +556,15 @@ __device__ void lm_step(const Team &tm, const TrajDev &td, const double *z, cons
             gv += 2.0 * td.omega_s * td.R[i - NX] * x;
         }
         ws.bb[e] = bv;
+        ws.b0[e] = bv;
         ws.g[e] = -gv;
     }
     // the t_F corner and gradient
     double cc = 0.0, gt = 0.0;
-    for (int e = t; e < N * NX; e += nt) {
-        const int k = e / NX, r = e - k * NX;
-        const double ev = eres(k, r);
+    for (int e = tm.sum_first(N * NX); e < N * NX; e += tm.sum_stride()) {
+        const double ev = ws.er[e];
         cc += ev * ev;
-        gt += ev * dres(k, r);
+        gt += ev * ws.dr[e];
     }
     {
         const double2 sums = team_sum2(cc, gt, s_red);   // also orders D, E, bb, g before the solve
@@ -556,36 +594,43 @@ __device__ void lm_step(const Team &tm, const TrajDev &td, const double *z, cons
         for (int m = warp; m < n_odd; m += n_warps) {   // phase A
             const int k = (2 * m + 1) * s, l = k - s, r = k + s;
             const bool has_r = r <= N;
-            warp_factor16(ws.D + (size_t)k * NW * NW, Fw, lane);
-            const int c = lane & (NW - 1);
-            const bool do_p = lane < NW, do_q = lane >= NW && has_r;
-            if (do_p)   // column c of T[k][l] = row c of the coupling E_l
-                column_solve16(Fw, ws.E + (size_t)l * NW * NW + c * NW, 1, ws.P + (size_t)k * NW * NW + c, NW);
-            if (do_q)   // column c of T[k][r] = E_k, solved in place
-                column_solve16(Fw, ws.E + (size_t)k * NW * NW + c, NW, ws.E + (size_t)k * NW * NW + c, NW);
-            if (lane < 2) {
-                double *f = (lane ? ws.g : ws.bb) + (size_t)k * NW;
-                column_solve16(Fw, f, 1, f, 1);
-            }
-            for (int ij = lane; ij < NW * NW; ij += 32) ws.D[(size_t)k * NW * NW + ij] = Fw[ij];
-            __syncwarp();
+            // T[k][l] is the transpose of the coupling E_l; T[k][r] = E_k becomes Q in place
+            warp_eliminate16(ws.D + (size_t)k * NW * NW, ws.E + (size_t)l * NW * NW, ws.P + (size_t)k * NW * NW,
+                             has_r ? ws.E + (size_t)k * NW * NW : nullptr, ws.bb + (size_t)k * NW,
+                             ws.g + (size_t)k * NW, lane);
         }
         team_sync();
         const int n_even = N / (2 * s) + 1;
         for (int m = warp; m < n_even; m += n_warps) {   // phase B
             const int j = 2 * m * s, iL = j - s, iR = j + s;
             const bool hasL = m > 0, hasR = iR <= N;
-            const double *QL = ws.E + (size_t)(hasL ? iL : 0) * NW * NW;
-            const double *PR = ws.P + (size_t)(hasR ? iR : 0) * NW * NW;
-            for (int e = lane; e < NW * NW; e += 32) {
-                const int a = e >> 4, b = e & (NW - 1);
-                if (b > a) continue;
-                double v0 = ws.D[(size_t)j * NW * NW + e], v1 = 0.0;
+            const bool hasE = hasR && iR + s <= N;
+            // Q_(j-s), P_(j+s) and Q_(j+s) staged in the warp's shared memory (coalesced loads,
+            // all in flight together), the 136 lower entries packed over the lanes
+            double *QL = Fw, *PR = Fw + NW * NW, *QR = Fw + 2 * NW * NW;
+            const double2 *gQL = reinterpret_cast<const double2 *>(ws.E + (size_t)(hasL ? iL : 0) * NW * NW);
+            const double2 *gPR = reinterpret_cast<const double2 *>(ws.P + (size_t)(hasR ? iR : 0) * NW * NW);
+            const double2 *gQR = reinterpret_cast<const double2 *>(ws.E + (size_t)(hasE ? iR : 0) * NW * NW);
+#pragma unroll
+            for (int q = 0; q < NW * NW / 64; ++q) {
+                const int at = q * 32 + lane;
+                if (hasL) reinterpret_cast<double2 *>(QL)[at] = gQL[at];
+                if (hasR) reinterpret_cast<double2 *>(PR)[at] = gPR[at];
+                if (hasE) reinterpret_cast<double2 *>(QR)[at] = gQR[at];
+            }
+            __syncwarp();
+            for (int e = lane; e < NW * (NW + 1) / 2; e += 32) {
+                int a, b;
+                tri_index(e, a, b);
+                double *d = ws.D + (size_t)j * NW * NW + a * NW + b;
+                double v0 = *d, v1 = 0.0;
                 if (hasL)
+#pragma unroll
                     for (int q = 0; q < NW; ++q) v0 = fma(-QL[q * NW + a], QL[q * NW + b], v0);
                 if (hasR)
+#pragma unroll
                     for (int q = 0; q < NW; ++q) v1 = fma(-PR[q * NW + a], PR[q * NW + b], v1);
-                ws.D[(size_t)j * NW * NW + e] = v0 + v1;
+                *d = v0 + v1;
             }
             {
                 const int a = lane & (NW - 1), which = lane >> 4;
@@ -593,19 +638,21 @@ __device__ void lm_step(const Team &tm, const TrajDev &td, const double *z, cons
                 double v = f[(size_t)j * NW + a];
                 if (hasL) {
                     const double *w = f + (size_t)iL * NW;
+#pragma unroll
                     for (int q = 0; q < NW; ++q) v = fma(-QL[q * NW + a], w[q], v);
                 }
                 if (hasR) {
                     const double *w = f + (size_t)iR * NW;
+#pragma unroll
                     for (int q = 0; q < NW; ++q) v = fma(-PR[q * NW + a], w[q], v);
                 }
                 f[(size_t)j * NW + a] = v;
             }
-            if (hasR && iR + s <= N) {
-                const double *QR = ws.E + (size_t)iR * NW * NW;
+            if (hasE) {
                 for (int e = lane; e < NW * NW; e += 32) {
                     const int a = e >> 4, b = e & (NW - 1);
                     double v = 0.0;
+#pragma unroll
                     for (int q = 0; q < NW; ++q) v = fma(PR[q * NW + a], QR[q * NW + b], v);
                     ws.E[(size_t)j * NW * NW + e] = -v;
                 }
@@ -616,13 +663,8 @@ __device__ void lm_step(const Team &tm, const TrajDev &td, const double *z, cons
     }
     // block 0: D_0 x_0 = f_0
     if (warp == 0) {
-        warp_factor16(ws.D, Fw, lane);
-        if (lane < 2) {
-            double *f = lane ? ws.g : ws.bb;
-            column_solve16(Fw, f, 1, f, 1);
-        }
-        __syncwarp();
-        warp_back16(Fw, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, ws.bb, ws.g, lane);
+        warp_eliminate16(ws.D, nullptr, nullptr, nullptr, ws.bb, ws.g, lane);
+        warp_back16(ws.D, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, ws.bb, ws.g, lane);
     }
     team_sync();
     // the eliminated blocks, from the last level to the first
@@ -639,19 +681,10 @@ __device__ void lm_step(const Team &tm, const TrajDev &td, const double *z, cons
         team_sync();
     }
     // 4. the border: dt = (-g_t - b^T v) / (c - b^T y), dw = v - y dt, with y = T^-1 b and
-    //    v = T^-1 (-g_w) (b the original border column, kept in the factor-free terms above:
-    //    b^T y and b^T v are recomputed from y and v through T y = b, i.e. b^T y = y^T T y).
-    //    T y = b and T v = -g hold, so b^T y = sum_k b_k . y_k needs the original b: it is
-    //    re-derived here from its definition.
+    //    v = T^-1 (-g_w), b the border column as assembled.
     double by = 0.0, bv = 0.0;
-    for (int e = t; e < (N + 1) * NW; e += nt) {
-        const int k = e / NW, i = e - k * NW;
-        double b = 0.0;
-        if (k < N)
-            for (int r = 0; r < NX; ++r) b += Aent(k, r, i) * eres(k, r);
-        if (k > 0)
-            for (int r = 0; r < NX; ++r) b += Bent(k - 1, r, i) * eres(k - 1, r);
-        b *= rho;
+    for (int e = tm.sum_first((N + 1) * NW); e < (N + 1) * NW; e += tm.sum_stride()) {
+        const double b = ws.b0[e];
         by += b * ws.bb[e];
         bv += b * ws.g[e];
     }
@@ -666,14 +699,15 @@ __device__ void lm_step(const Team &tm, const TrajDev &td, const double *z, cons
 }
 
 // One LM step for each trajectory (a test of the step): dz at (z, lam, mu). Cluster p of
-// kTrajCtas CTAs serves trajectory p.
-__global__ void __cluster_dims__(kTrajCtas, 1, 1) __launch_bounds__(kTrajThreads)
+// CTAS CTAs serves trajectory p.
+template <int CTAS>
+__global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(kTrajThreads)
 k_traj_step(const TrajDev td, const double *q_star, const double *z, const double *lam, double mu, double *ws_base,
             size_t ws_stride, double *dz)
 {
     extern __shared__ double s_mem[];
     const int N = td.N, n_var = 1 + NW * (N + 1), n_eq = NX * (N + 2);
-    const int p = (int)(blockIdx.x / kTrajCtas);
+    const int p = (int)(blockIdx.x / CTAS);
     const Team tm = team_of_block();
     double *s_red = s_mem;                                      // kRedDoubles
     double *s_blk = s_red + kRedDoubles;                        // per warp kWarpScratch
@@ -683,23 +717,24 @@ k_traj_step(const TrajDev td, const double *q_star, const double *z, const doubl
         x_S[i] = i < 4 ? qs[i] : 0.0;
         x_T[i] = i < 4 ? qs[(size_t)N * 4 + i] : 0.0;
     }
-    __syncthreads();
     const TrajWs ws = ws_of(ws_base + (size_t)p * ws_stride, N);
-    lm_step(tm, td, z + (size_t)p * n_var, lam + (size_t)p * n_eq, qs, x_S, x_T, mu, ws, dz + (size_t)p * n_var, false,
-            s_red, s_blk);
+    for (int i = tm.tid(); i < n_eq; i += tm.nthreads()) ws.lr[i] = lam[(size_t)p * n_eq + i] / td.rho;
+    team_sync();
+    lm_step(tm, td, z + (size_t)p * n_var, qs, x_S, x_T, mu, ws, dz + (size_t)p * n_var, false, s_red, s_blk);
 }
 
 // The whole solve (T6) for each trajectory: z in place; stats {t_F, F, max |c|, max bound
-// violation}. Cluster p of kTrajCtas CTAs serves trajectory p; each CTA keeps z, the trial
+// violation}. Cluster p of CTAS CTAs serves trajectory p; each CTA keeps z, the trial
 // point and the step in its shared memory and updates all of them itself (the same values in
-// both), the multipliers and the workspace are global and split.
-__global__ void __cluster_dims__(kTrajCtas, 1, 1) __launch_bounds__(kTrajThreads)
+// all), the multipliers and the workspace are global and split.
+template <int CTAS>
+__global__ void __cluster_dims__(CTAS, 1, 1) __launch_bounds__(kTrajThreads)
 k_traj_solve(const TrajDev td, const double *q_star, double *z_io, double *ws_base, size_t ws_stride, double *lam_ws,
              double *stats)
 {
     extern __shared__ double s_mem[];
     const int N = td.N, n_var = 1 + NW * (N + 1), n_eq = NX * (N + 2);
-    const int p = (int)(blockIdx.x / kTrajCtas), t = threadIdx.x;
+    const int p = (int)(blockIdx.x / CTAS), t = threadIdx.x;
     const Team tm = team_of_block();
     double *s_red = s_mem;
     double *s_blk = s_red + kRedDoubles;
@@ -714,21 +749,24 @@ k_traj_solve(const TrajDev td, const double *q_star, double *z_io, double *ws_ba
         x_T[i] = i < 4 ? qs[(size_t)N * 4 + i] : 0.0;
     }
     for (int i = t; i < n_var; i += blockDim.x) z[i] = z_io[(size_t)p * n_var + i];
-    for (int i = tm.tid(); i < n_eq; i += tm.nthreads()) lam[i] = 0.0;
-    team_sync();
     const TrajWs ws = ws_of(ws_base + (size_t)p * ws_stride, N);
+    for (int i = tm.tid(); i < n_eq; i += tm.nthreads()) {
+        lam[i] = 0.0;
+        ws.lr[i] = 0.0;
+    }
+    team_sync();
     double mu = td.mu0;
     for (int o = 0; o < td.outer; ++o) {
         eval_f(tm, td, z, ws.f);
         team_sync();
-        double F = merit(tm, td, z, lam, qs, ws.f, x_S, x_T, s_red);
+        double F = merit(tm, td, z, ws.lr, qs, ws.f, x_S, x_T, s_red);
         for (int it = 0; it < td.inner; ++it) {
-            lm_step(tm, td, z, lam, qs, x_S, x_T, mu, ws, dz, true, s_red, s_blk);
+            lm_step(tm, td, z, qs, x_S, x_T, mu, ws, dz, true, s_red, s_blk);
             for (int i = t; i < n_var; i += blockDim.x) zn[i] = z[i] + dz[i];
             __syncthreads();
             eval_f(tm, td, zn, ws.f);
             team_sync();
-            const double Fn = merit(tm, td, zn, lam, qs, ws.f, x_S, x_T, s_red);
+            const double Fn = merit(tm, td, zn, ws.lr, qs, ws.f, x_S, x_T, s_red);
             if (Fn < F) {
                 for (int i = t; i < n_var; i += blockDim.x) z[i] = zn[i];
                 F = Fn;
@@ -749,7 +787,9 @@ k_traj_solve(const TrajDev td, const double *q_star, double *z_io, double *ws_ba
                            0.5 * h * (ws.f[(size_t)k * NX + i] + ws.f[(size_t)(k + 1) * NX + i]);
             else if (k == N) c = z[1 + i] - x_S[i];
             else c = z[1 + (size_t)N * NW + i] - x_T[i];
-            lam[e] += td.rho * c;
+            const double l = lam[e] + td.rho * c;
+            lam[e] = l;
+            ws.lr[e] = l / td.rho;
         }
         team_sync();
     }
@@ -796,7 +836,7 @@ k_traj_solve(const TrajDev td, const double *q_star, double *z_io, double *ws_ba
         stats[(size_t)p * 4 + 3] = fmax(v, 0.0);
     }
     __syncthreads();
-    const double Fend = merit(tm, td, z, lam, qs, ws.f, x_S, x_T, s_red);
+    const double Fend = merit(tm, td, z, ws.lr, qs, ws.f, x_S, x_T, s_red);
     if (t == 0 && tm.rank == 0) {
         stats[(size_t)p * 4 + 0] = z[0];
         stats[(size_t)p * 4 + 1] = Fend;
@@ -867,6 +907,7 @@ struct cp_traj {
     TrajDev td{};
     int max_paths = 0;
     size_t ws_stride = 0;   // doubles per trajectory
+    int fit4 = 0, fit8 = 0; // clusters of 4 and of 8 CTAs the device holds at a time
     double *ws = nullptr, *lam = nullptr, *dq_max = nullptr;
 };
 
@@ -874,7 +915,27 @@ namespace {
 
 size_t traj_ws_doubles(int N)
 {
-    return (size_t)(N + 1) * (NX + NX * NW + 2 * NW * NW + 2 * NW + 10) + (size_t)N * NW * NW;
+    return (size_t)(N + 1) * (NX + NF * NW + 2 * NW * NW + 3 * NW + 10) + (size_t)N * (NW * NW + 2 * NX) +
+           (size_t)NX * (N + 2);
+}
+
+size_t traj_smem(int N, bool solve);
+
+// Clusters of `ctas` CTAs of the solver that the device holds at a time.
+template <int CTAS>
+cudaError_t resident_clusters(int N, int *count)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = CTAS;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(CTAS);
+    cfg.blockDim = dim3(kTrajThreads);
+    cfg.dynamicSmemBytes = traj_smem(N, true);
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaOccupancyMaxActiveClusters(count, k_traj_solve<CTAS>, &cfg);
 }
 
 size_t traj_smem(int N, bool solve)
@@ -942,10 +1003,14 @@ int cp_traj_init(const cp_model *model, const cp_traj_params *tp, int32_t max_pa
     t->lam = t->ws + t->ws_stride * max_paths;
     t->dq_max = t->lam + n_eq * max_paths;
     e = cudaMemcpyAsync(t->dq_max, tp->dq_max, sizeof(double) * 4, cudaMemcpyHostToDevice, t->st);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_traj_solve, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)traj_smem(tp->N, true));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_traj_step, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)traj_smem(tp->N, false));
+    // the limit of the largest N: solvers of several sizes share the kernels
+    const int smem = (int)traj_smem(255, true);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_traj_solve<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_traj_solve<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_traj_solve<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_traj_step<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = resident_clusters<4>(tp->N, &t->fit4);
+    if (e == cudaSuccess) e = resident_clusters<8>(tp->N, &t->fit8);
     if (e == cudaSuccess) e = cudaStreamSynchronize(t->st);
     if (e != cudaSuccess) {
         cudaFree(t->ws);
@@ -996,7 +1061,7 @@ int cp_traj_step(cp_traj *t, const double *d_q_star, int32_t n, const double *d_
     if (n > 0 && (!d_q_star || !d_z || !d_lam || !d_dz)) return set_error("NULL argument"), CP_ERR_ARG;
     if (!(mu >= 0.0)) return set_error("mu must be >= 0"), CP_ERR_ARG;
     if (n == 0) return CP_OK;
-    k_traj_step<<<n * kTrajCtas, kTrajThreads, traj_smem(t->td.N, false), t->st>>>(t->td, d_q_star, d_z, d_lam, mu,
+    k_traj_step<2><<<n * 2, kTrajThreads, traj_smem(t->td.N, false), t->st>>>(t->td, d_q_star, d_z, d_lam, mu,
                                                                                  t->ws, t->ws_stride, d_dz);
     CP_LAUNCHED("k_traj_step");
     return CP_OK;
@@ -1009,8 +1074,12 @@ int cp_traj_solve(cp_traj *t, const double *d_q_star, int32_t n, double *d_z, do
     if (n < 0 || n > t->max_paths) return set_error("n = %d outside 0..%d", n, t->max_paths), CP_ERR_ARG;
     if (n > 0 && (!d_q_star || !d_z || !d_stats)) return set_error("NULL argument"), CP_ERR_ARG;
     if (n == 0) return CP_OK;
-    k_traj_solve<<<n * kTrajCtas, kTrajThreads, traj_smem(t->td.N, true), t->st>>>(t->td, d_q_star, d_z, t->ws,
-                                                                                  t->ws_stride, t->lam, d_stats);
+    // CTAs per trajectory: the most of 8, 4 or 2 with which every cluster is resident at once (a
+    // second wave would cost more than the split gives). The results do not depend on it.
+    const int ctas = n <= t->fit8 ? 8 : (n <= t->fit4 ? 4 : 2);
+    auto kern = ctas == 8 ? k_traj_solve<8> : (ctas == 4 ? k_traj_solve<4> : k_traj_solve<2>);
+    kern<<<n * ctas, kTrajThreads, traj_smem(t->td.N, true), t->st>>>(t->td, d_q_star, d_z, t->ws, t->ws_stride,
+                                                                     t->lam, d_stats);
     CP_LAUNCHED("k_traj_solve");
     return CP_OK;
 }
