@@ -324,24 +324,36 @@ k_smooth(const ModelDev m, const SceneDev sc, const SmoothArgs a)
     }
 }
 
-// Sums the groups' partials of each candidate in group order (one warp per candidate).
-__global__ void k_smooth_reduce(int n, int groups, int K, const double *part_J, const float *part_g,
-                                const double *gJ, double *J, float *dxi)
+// Sums the groups' partials of each candidate in group order: one thread per gradient entry
+// (and one more per candidate for J), eight groups' loads in flight before the dependent
+// additions. With a warp per candidate that loaded one group at a time the kernel was bound by
+// the latency of some 4 x 76 loads in a row (64 candidates, K = 32).
+__global__ void __launch_bounds__(128)
+k_smooth_reduce(int n, int groups, int K, const double *__restrict__ part_J, const float *__restrict__ part_g,
+                const double *__restrict__ gJ, double *J, float *dxi)
 {
-    const int cand = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    if (cand >= n) return;
-    if (lane == 0 && J != nullptr) {
-        double acc = 0.0;
-        for (int g = 0; g < groups; ++g) acc += part_J[(size_t)cand * groups + g];
-        J[cand] = acc;
-    }
-    if (dxi == nullptr) return;
-    const float gj = gJ != nullptr ? (float)gJ[cand] : 1.f;
-    for (int t = lane; t < 4 * K; t += 32) {
-        float acc = 0.f;
-        for (int g = 0; g < groups; ++g) acc += part_g[((size_t)cand * groups + g) * 4 * K + t];
-        dxi[(size_t)cand * 4 * K + t] = gj * acc;
+    constexpr int kAhead = 8;
+    const int cand = blockIdx.x, D = 4 * K;
+    for (int t = threadIdx.x; t <= D; t += blockDim.x) {
+        if (t == D) {
+            if (J == nullptr) continue;
+            double acc = 0.0;
+            for (int g = 0; g < groups; ++g) acc += part_J[(size_t)cand * groups + g];
+            J[cand] = acc;
+        } else if (dxi != nullptr) {
+            const float *col = part_g + (size_t)cand * groups * D + t;
+            float acc = 0.f;
+            for (int g0 = 0; g0 < groups; g0 += kAhead) {
+                float v[kAhead];
+#pragma unroll
+                for (int q = 0; q < kAhead; ++q) v[q] = g0 + q < groups ? col[(size_t)(g0 + q) * D] : 0.f;
+#pragma unroll
+                for (int q = 0; q < kAhead; ++q)
+                    if (g0 + q < groups) acc += v[q];
+            }
+            const float gj = gJ != nullptr ? (float)gJ[cand] : 1.f;
+            dxi[(size_t)cand * D + t] = gj * acc;
+        }
     }
 }
 
@@ -384,8 +396,7 @@ int launch_smooth_t(const ModelDev &m, const SceneDev &sc, const SmoothArgs &a, 
     kern<<<grid, threads, smem, st>>>(m, sc, a);
     CP_LAUNCHED("k_smooth");
     if (a.groups > 1) {
-        k_smooth_reduce<<<(a.n * 32 + 255) / 256, 256, 0, st>>>(a.n, a.groups, a.K, a.part_J, a.part_g,
-                                                                a.gJ, a.J, a.dxi);
+        k_smooth_reduce<<<a.n, 128, 0, st>>>(a.n, a.groups, a.K, a.part_J, a.part_g, a.gJ, a.J, a.dxi);
         CP_LAUNCHED("k_smooth_reduce");
     }
     return CP_OK;
