@@ -8,6 +8,8 @@
 
 namespace cp {
 
+struct BatchQueryDev;
+
 // ------------------------------------------------------------------ error plumbing
 
 void set_error(const char *fmt, ...);
@@ -262,6 +264,8 @@ int launch_philox(const uint32_t *ctr, uint32_t k0, uint32_t k1, int64_t n, uint
 int launch_factor(const double *C, double sigma2, const double *sigma_dev, int D, double *L,
                   float *Lt_f, uint32_t *status, cudaStream_t st);
 int factor_configure();
+int batch_factor_clusters(int max_D, int *count);   // clusters resident at a time
+int launch_batch_factor_cluster(const BatchQueryDev *qd, int nq, int max_D, cudaStream_t st);
 int launch_sample(const double *mu, const float *Lt_f, int N, int K, uint64_t seed,
                   uint32_t iter, uint32_t query, float *xi, cudaStream_t st);
 int sample_configure();

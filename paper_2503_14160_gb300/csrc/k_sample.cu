@@ -1,9 +1,11 @@
 // Algorithm 1 step (1): xi_i ~ N(mu, sigma^2 C) (arXiv 2503.14160, Sec. 4.1).
-//   k_factor  L L^T = sigma^2 C, FP64 right-looking Cholesky (L D L^T form) in one CTA, D <= 128
+//   k_batch_factor  L L^T = sigma^2 C of many queries, FP64 right-looking Cholesky (L D L^T form),
+//             one CTA per query, D <= 128 (one query or few: a cluster each, k_factor.cu)
 //   k_sample  z_i from Philox4x32-10 (Salmon et al., SC'11) + Box-Muller, xi_i = mu + L z_i
 // The counter of candidate i, block j, iteration t, query q is (j, i, t, q); the key is
 // the 64-bit seed split into two words. Block j gives the normals z[4j..4j+3].
 #include "cp_internal.cuh"
+#include "fp64_chain.cuh"
 #include "philox.cuh"
 
 namespace cp {
@@ -18,31 +20,6 @@ __global__ void k_philox(const uint4 *__restrict__ ctr, uint32_t k0, uint32_t k1
 
 constexpr int kFactorThreads = 1024;
 constexpr int kFactorMaxD = 4 * CP_MAX_WAYPOINTS;
-
-// 1/a and 1/sqrt(a) for a > 0: a float seed refined by two Newton-Raphson steps in FP64
-// (quadratic convergence: 23 -> 46 -> 92 bits). On a part with a narrow FP64 pipe these
-// short chains are much faster than a library division or square root. Arguments whose
-// float conversion is not a normal number take the IEEE operations instead.
-__device__ __forceinline__ double recip_newton(double a)
-{
-    const float af = (float)a;
-    if (!(af > 1e-30f && af < 1e30f)) return 1.0 / a;
-    double y = (double)__frcp_rn(af);
-    y = fma(y, fma(-a, y, 1.0), y);
-    y = fma(y, fma(-a, y, 1.0), y);
-    return y;
-}
-
-__device__ __forceinline__ double rsqrt_newton(double a)
-{
-    const float af = (float)a;
-    if (!(af > 1e-30f && af < 1e30f)) return 1.0 / sqrt(a);
-    double y = (double)rsqrtf(af);
-    const double h = 0.5 * a;
-    y = y * fma(-h * y, y, 1.5);
-    y = y * fma(-h * y, y, 1.5);
-    return y;
-}
 
 // One CTA, right-looking Cholesky of A = sigma^2 C in shared memory (row stride D + 1) in
 // the unscaled (L D L^T) form: step k takes t_i = a_ik / a_kk for the rows below the pivot,
@@ -119,15 +96,6 @@ __device__ __forceinline__ void factor_body(const double *__restrict__ C, double
     }
     __syncthreads();
     if (tid == 0 && bad) atomicOr(status, DEV_ERR_NOT_PD);
-}
-
-__global__ void __launch_bounds__(kFactorThreads)
-k_factor(const double *__restrict__ C, double sigma2, const double *__restrict__ sigma_dev, int D, double *L,
-         float *Lt, uint32_t *status)
-{
-    if (sigma_dev != nullptr) sigma2 = sigma_dev[0] * sigma_dev[0];   // the step size kept on the device
-    extern __shared__ double A[];
-    factor_body(C, sigma2, D, L, Lt, status, A);
 }
 
 // The factors of every query of a batch, one CTA per query.
@@ -253,23 +221,6 @@ int launch_philox(const uint32_t *ctr, uint32_t k0, uint32_t k1, int64_t n, uint
     return CP_OK;
 }
 
-int factor_configure()
-{
-    const int Dm = 4 * CP_MAX_WAYPOINTS;
-    const int max_smem = (int)(sizeof(double) * Dm * (Dm + 1));
-    CP_CUDA(cudaFuncSetAttribute(k_factor, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
-    return CP_OK;
-}
-
-int launch_factor(const double *C, double sigma2, const double *sigma_dev, int D, double *L,
-                  float *Lt_f, uint32_t *status, cudaStream_t st)
-{
-    const size_t smem = sizeof(double) * (size_t)D * (D + 1);
-    k_factor<<<1, kFactorThreads, smem, st>>>(C, sigma2, sigma_dev, D, L, Lt_f, status);
-    CP_LAUNCHED("k_factor");
-    return CP_OK;
-}
-
 int sample_configure()
 {
     CP_CUDA(cudaFuncSetAttribute(k_sample, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -282,8 +233,17 @@ int sample_configure()
     return CP_OK;
 }
 
+// One cluster per query while they fill the device at most kClusterWaves times, else one CTA per
+// query: at D = 128 a cluster takes about 80 us and holds eight SMs, a CTA 198 us and one SM
+// (the same bits), so two waves of clusters are still the faster form and three are not.
+constexpr int kClusterWaves = 2;
+
 int launch_batch_factor(const BatchQueryDev *qd, int nq, int max_D, cudaStream_t st)
 {
+    int fit = 0;
+    const int rc = batch_factor_clusters(max_D, &fit);
+    if (rc != CP_OK) return rc;
+    if (nq <= kClusterWaves * fit) return launch_batch_factor_cluster(qd, nq, max_D, st);
     const size_t smem = sizeof(double) * (size_t)max_D * (max_D + 1);
     k_batch_factor<<<nq, kFactorThreads, smem, st>>>(qd);
     CP_LAUNCHED("k_batch_factor");

@@ -34,6 +34,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "cp_internal.cuh"
+#include "fp64_chain.cuh"
 
 // An NVTX range over a scope (no-op without a profiling tool).
 struct NvtxScope {
@@ -98,21 +99,6 @@ __device__ __forceinline__ void trig_of(Dual a, const double *cache, double *cw,
     (void)cw;
     c = {cv, -sv * a.d};
     s = {sv, cv * a.d};
-}
-
-// 1 / sqrt(a) in FP64 for the pivots of the block factorisation: an FP32 seed and two
-// Newton steps (quadratic convergence: about 22 -> 44 -> 88 bits), a short dependent chain
-// where FP64 operations wait tens of cycles each. Arguments outside FP32's normal range take
-// the IEEE operations (a non-positive pivot gives NaN, as sqrt would).
-__device__ __forceinline__ double rsqrt_pivot(double a)
-{
-    const float af = (float)a;
-    if (!(af > 1e-30f && af < 1e30f)) return 1.0 / sqrt(a);
-    double y = (double)rsqrtf(af);
-    const double hh = 0.5 * a;
-    y = y * fma(-hh * y, y, 1.5);
-    y = y * fma(-hh * y, y, 1.5);
-    return y;
 }
 
 struct TrajDev {
@@ -326,7 +312,7 @@ __device__ double merit(const Team &tm, const TrajDev &td, const double *z, cons
 // side's transpose takes the same operations as a row of A below the pivot, so the lanes hold
 //   lanes 0-15   row i of A, and column i of Tr;
 //   lanes 16-31  column c of Tl, and (lanes 16, 17) the two vectors,
-// one row in each of two register sets: per pivot one reciprocal square root (rsqrt_pivot), one
+// one row in each of two register sets: per pivot one reciprocal square root (rsqrt_newton), one
 // scaling and one FMA per later column and set, with the pivot's column from shuffles. That is
 // about 400 FP64 warp instructions and one chain of 16 pivots where the factor followed by three
 // column solves took 710 and three more chains. Tl is the transpose of Tl_rows (row-major
@@ -348,7 +334,7 @@ __device__ __noinline__ void warp_eliminate16(double *A, const double *Tl_rows, 
 #pragma unroll
     for (int p = 0; p < NW; ++p) {
         const double d = __shfl_sync(full, a[p], p);   // the pivot, from lane p
-        const double r = rsqrt_pivot(d);
+        const double r = rsqrt_newton(d);
         double l = a[p] * r;                            // L[i][p], or P[p][i]
         if (low && i <= p) l = i == p ? d * r : 0.0;
         if (lane == p) diag = r;

@@ -79,3 +79,33 @@ def test_trajectories_do_not_depend_on_the_cluster_size(lib, crane, N):
         assert np.isfinite(z).all()
     finally:
         lib.cp_traj_destroy(h)
+
+
+@pytest.mark.parametrize("K", [1, 2, 4, 5, 8, 9, 16, 21, 31, 32])
+def test_factor_against_fp64(lib, crane, K):
+    """The cluster factor at every edge of its 16-row blocks: backward error of a few D units of
+    rounding per entry, relative to the geometric mean of the two variances."""
+    import torch
+    from paper_2503_14160_gb300 import workloads
+    D = 4 * K
+    g = np.random.default_rng(K)
+    A = g.normal(size=(D, D + 3)) * np.exp(g.normal(size=(D, 1)))
+    C = A @ A.T
+    sigma = 0.7
+    with lib.Planner(crane, workloads.empty_scene(), lib.make_params(64, K, 2, sigma=sigma)) as pl:
+        lib.cp_set_endpoints(pl.handle, *ENDS[0])
+        mu = torch.zeros(D, dtype=torch.float64, device="cuda")
+        lib.cp_set_distribution(pl.handle, mu, torch.from_numpy(C).cuda(), 1)
+        L = torch.empty(D, D, dtype=torch.float64, device="cuda")
+        lib.cp_get_factor(pl.handle, L)
+        lib.cp_synchronize(pl.handle)
+        L = L.cpu().numpy()
+        assert np.all(np.triu(L, 1) == 0.0)
+        scale = sigma ** 2 * np.sqrt(np.outer(np.diag(C), np.diag(C)))
+        assert np.max(np.abs(L @ L.T - sigma ** 2 * C) / scale) < 4 * (D + 4) * 2.0 ** -53
+        # a lost pivot in the last block is reported
+        C[D - 1, D - 1] = -1.0
+        lib.cp_set_distribution(pl.handle, mu, torch.from_numpy(C).cuda(), 1)
+        with pytest.raises(lib.CranePlanError) as e:
+            lib.cp_synchronize(pl.handle)
+        assert e.value.status == -6
