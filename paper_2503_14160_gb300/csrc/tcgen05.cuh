@@ -1,10 +1,11 @@
 // Thin inline-PTX wrappers for the fifth-generation tensor cores of sm_100-family parts
 // (tcgen05: accumulators in tensor memory, operands described by shared-memory matrix
 // descriptors), mbarriers and bulk copies. Only what the kernels of this library use:
-// kind::tf32 MMAs with M = 128 on one CTA, K-major operands without swizzling.
+// kind::tf32 and kind::f16 (BF16) MMAs with M = 128 on one CTA, K-major operands without
+// swizzling.
 //
-// Operand layout (K-major, no swizzle). A tile of R rows (M or N) by C elements of K, with
-// 4-byte elements, is stored as "core matrices" of 8 rows x 16 bytes (4 elements of K),
+// Operand layout (K-major, no swizzle; BF16 the same with 8 elements of K per core matrix). A
+// tile of R rows (M or N) by C elements of K, with 4-byte elements, is stored as "core matrices" of 8 rows x 16 bytes (4 elements of K),
 // each core matrix 128 contiguous bytes (row r of the core at byte 16 r). Core (g, kc),
 // g = row / 8 and kc = k / 4, starts at byte (g * (C / 4) + kc) * 128, so cores adjacent
 // along K are 128 bytes apart (the descriptor's leading-dimension offset) and cores
@@ -141,6 +142,24 @@ static __device__ __forceinline__ uint64_t desc_kmajor(uint32_t saddr, uint32_t 
 static __host__ __device__ constexpr uint32_t idesc_tf32(int M, int N)
 {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+// Instruction descriptor of kind::f16 with BF16 operands (bits 7-9 and 10-12 = 1), otherwise as
+// above.
+static __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N)
+{
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
+// D[tmem] (+)= A B^T for one K step of 16 BF16 elements; issued by one thread.
+static __device__ __forceinline__ void mma_f16kind(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                                   bool accumulate)
+{
+    asm volatile("{\n\t.reg .pred p;\n\t"
+                 "setp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                 :: "r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate)
+                 : "memory");
 }
 
 // D[tmem] (+)= A B^T for one K step of 8 TF32 elements; issued by one thread.

@@ -109,3 +109,102 @@ def test_factor_against_fp64(lib, crane, K):
         with pytest.raises(lib.CranePlanError) as e:
             lib.cp_synchronize(pl.handle)
         assert e.value.status == -6
+
+
+def _moments_reference(x, w):
+    """mu, C (without eps) and the second moments about x_1, in long double."""
+    x, w = x.astype(np.longdouble), w.astype(np.longdouble)
+    y = x - x[0]
+    s1 = (w[:, None] * y).sum(0)
+    s2 = (w[:, None] * y).T @ y
+    return x[0] + s1, s2 - np.outer(s1, s1), s2, s1
+
+
+@pytest.mark.parametrize("N,K,shape", [(16384, 8, "plain"), (16442, 8, "plain"), (1024, 32, "plain"),
+                                       (2050, 23, "offset"), (4099, 17, "outlier"), (9001, 16, "plain"),
+                                       (3001, 32, "still"), (65536, 32, "plain")])
+def test_integer_moments(lib, crane, N, K, shape):
+    """The tensor-core moments (nu D^2 >= 2^23) against long double. Bound per entry: the two
+    factors' rounding to 2^-55 of the column's bound (at most 4 times the largest deviation times
+    the largest root weight), by Cauchy-Schwarz over the elites, and 16 units of FP64 rounding of
+    the two terms of C."""
+    import torch
+    from paper_2503_14160_gb300 import workloads
+    g = np.random.default_rng(N + K)
+    D, nu = 4 * K, N // 2
+    assert nu * D * D >= 2 ** 23
+    xi = (g.normal(size=(N, D)) * np.exp(g.normal(size=D) * 2)).astype(np.float32)
+    if shape == "offset":
+        xi += np.float32(1000.0)
+    if shape == "outlier":
+        xi[g.integers(0, N, 3)] *= np.float32(2e4)
+    if shape == "still":
+        xi[:, 5] = np.float32(0.3)
+    J = workloads.random_costs(N, seed=N)
+    order = np.argsort(J, kind="stable")[:nu]
+    w = np.log(nu + 0.5) - np.log(np.arange(1, nu + 1))
+    w = w / w.sum()
+    x = xi[order].astype(np.float64)
+    mu_ref, C_ref, s2, s1 = _moments_reference(x, w)
+    with lib.Planner(crane, workloads.empty_scene(), lib.make_params(N, K, 2, eps=0.0)) as pl:
+        lib.cp_set_endpoints(pl.handle, *ENDS[0])
+        lib.cp_update(pl.handle, torch.from_numpy(J).cuda(), torch.from_numpy(xi).cuda())
+        mu = torch.empty(D, dtype=torch.float64, device="cuda")
+        C = torch.empty(D, D, dtype=torch.float64, device="cuda")
+        lib.cp_get_distribution(pl.handle, mu, C)
+        torch.cuda.synchronize()
+    mu, C = mu.cpu().numpy(), C.cpu().numpy()
+    y = np.abs(x - x[0]).max(0)
+    z = 4.0 * y * np.sqrt(w[0]) * 2.0 ** -55            # rounding of one factor
+    root = np.sqrt(nu * np.diag(s2).astype(np.float64))  # sum_j |z_j| at most
+    u = 2.0 ** -53
+    bound = np.outer(z, root) + np.outer(root, z) + 16 * u * (np.abs(s2) + np.abs(np.outer(s1, s1))
+                                                               + np.sqrt(np.outer(np.diag(s2), np.diag(s2))))
+    assert np.all(np.abs(C - C_ref) <= bound.astype(np.float64) + 1e-300)
+    assert np.all(np.abs(mu - mu_ref) <= 4 * y * w[0] * nu * 2.0 ** -55 + 16 * u * (np.abs(mu_ref) + np.abs(s1)) + 1e-300)
+    # no less exact than a plain FP64 sum, over all entries
+    scale = np.sqrt(np.outer(np.diag(s2), np.diag(s2))).astype(np.float64) + 1e-300
+    y64 = x - x[0]
+    plain = (w[:, None] * y64).T @ y64 - np.outer(w @ y64, w @ y64)
+    err = np.linalg.norm(((C - C_ref) / scale).astype(np.float64))
+    assert err <= 1.5 * np.linalg.norm(((plain - C_ref) / scale).astype(np.float64)) + D * u
+
+
+@pytest.mark.parametrize("bad", [np.inf, np.nan, 3e38])
+def test_integer_moments_carry_non_finite_elites(lib, crane, bad):
+    """An elite outside the fixed-point range: its column as FP64 arithmetic gives it, the other
+    columns as without it."""
+    import torch
+    from paper_2503_14160_gb300 import workloads
+    N, K = 4096, 16
+    D, nu = 4 * K, N // 2
+    g = np.random.default_rng(3)
+    xi = g.normal(size=(N, D)).astype(np.float32)
+    J = np.arange(N, dtype=np.float64)
+    out = []
+    for value in (np.float32(bad), xi[7, 9]):
+        x = xi.copy()
+        x[7, 9] = value
+        if bad == 3e38:
+            x[0, 9] = -value
+        with lib.Planner(crane, workloads.empty_scene(), lib.make_params(N, K, 2)) as pl:
+            lib.cp_set_endpoints(pl.handle, *ENDS[0])
+            lib.cp_update(pl.handle, torch.from_numpy(J).cuda(), torch.from_numpy(x).cuda())
+            mu = torch.empty(D, dtype=torch.float64, device="cuda")
+            C = torch.empty(D, D, dtype=torch.float64, device="cuda")
+            lib.cp_get_distribution(pl.handle, mu, C)
+            torch.cuda.synchronize()
+        out.append((mu.cpu().numpy(), C.cpu().numpy()))
+    others = np.arange(D) != 9
+    assert np.array_equal(out[0][0][others], out[1][0][others])
+    assert np.array_equal(out[0][1][np.ix_(others, others)], out[1][1][np.ix_(others, others)])
+    if bad == 3e38:
+        w = np.log(nu + 0.5) - np.log(np.arange(1, nu + 1))
+        w = w / w.sum()
+        x = xi[:nu].astype(np.float64)
+        x[7, 9], x[0, 9] = np.float32(bad), -np.float32(bad)
+        want = (w[:, None] * x).sum(0)[9]
+        assert abs(out[0][0][9] - want) <= 1e-10 * 3e38
+        assert np.isfinite(out[0][1][:, 9]).all()
+    else:
+        assert not np.isfinite(out[0][0][9]) and not np.isfinite(out[0][1][9, 9])
