@@ -21,8 +21,8 @@
 //   column's largest deviation times the largest weight's root) and of the final FP64 value.
 // S1 = sum_j w_j y_j takes the same integers Y times a 63-bit w_j.
 //
-// A CTA takes 64 columns of S2 (all 128 rows) over a range of elites, 32 at a time: 512 threads
-// turn one column of eight elites each into digits in shared memory (K-major core matrices) while
+// A CTA takes 64 columns of S2 (all 128 rows) over a range of elites, 32 at a time: 1024 threads
+// turn one column of four elites each into digits in shared memory (K-major core matrices) while
 // the tensor cores work on the stage before, one thread issues the 68 MMAs of 128 x 64 x 16, and
 // the eight levels fill the 512 columns of tensor memory. Measured TC_MEASURED.
 #include "cp_internal.cuh"
@@ -31,10 +31,12 @@
 namespace cp {
 namespace {
 
-constexpr int kTcThreads = 512;
+constexpr int kTcThreads = 1024;
 constexpr int kTcRows = 128;            // rows of S2 (D <= 128), the MMA's M
 constexpr int kTcCols = 64;             // columns of S2 per CTA, the MMA's N
 constexpr int kStage = 32;              // elites per stage (two K steps of 16)
+constexpr int kPer = kStage * kTcRows / kTcThreads;                // elites of a thread per stage: 4
+constexpr int kAcc = kTcRows * kTcCols / kTcThreads;               // entries of a thread: 8
 constexpr int kEpoch = 4;               // stages per accumulation: 128 elites
 constexpr int kDigits = 7, kLevels = 8;
 constexpr uint32_t kLbo = 128, kSbo = kStage / 8 * 128;            // core-matrix offsets, bytes
@@ -116,29 +118,32 @@ __device__ __forceinline__ void moments_tc_body(const MomentsTc &a, int tile, in
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = s_tmem;
-    // this thread's column and its eight elites of every stage
+    // this thread's column and its four elites of every stage
     const int c = tid & (kTcRows - 1), g = tid / kTcRows;
     const bool on = c < a.D, own = on && c / kTcCols == tile;
     const int ey = on ? bound_exponent(a.colmax[c]) : 0;
     const int drop = mean_drop(a.scale[1]);
     const long long X1 = on ? fixed_of(a.elites[c], ey) : 0;
     long long s1 = 0;
-    long long hi[16], lo[16];
+    long long hi[kAcc], lo[kAcc];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) hi[i] = lo[i] = 0;
+    for (int i = 0; i < kAcc; ++i) hi[i] = lo[i] = 0;
     bool late = false;
     // the stage's accumulators as integers: weights 2^24, 2^16, 2^8, 1 into hi (levels 0-3) and
-    // lo (levels 4-7); warp w holds rows 32 (w mod 4) .. and columns 16 (w / 4) ..
+    // lo (levels 4-7); warp w holds rows 32 (w mod 4) .. and columns 8 (w / 4) ..
     auto drain = [&]() {
         __syncwarp();
-        const uint32_t at = tmem + ((uint32_t)(warp & 3) << 21) + 16u * (uint32_t)(warp >> 2);
+        const uint32_t at = tmem + ((uint32_t)(warp & 3) << 21) + (uint32_t)(kAcc * (warp >> 2));
 #pragma unroll
-        for (int l = 0; l < kLevels; ++l) {
-            float v[16];
-            tc::tmem_ld16(at + (uint32_t)(l * kTcCols), v);
+        for (int l = 0; l < kLevels; l += 2) {
+            uint32_t v[2 * kAcc];
+            tc::tmem_ld8_async(at + (uint32_t)(l * kTcCols), v);
+            tc::tmem_ld8_async(at + (uint32_t)((l + 1) * kTcCols), v + kAcc);
+            tc::tmem_ld_wait<2 * kAcc>(v);
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const long long p = (long long)__float2int_rn(v[i]) * (1 << 8 * (3 - (l & 3)));
+            for (int i = 0; i < kAcc; ++i) {
+                const long long p = (long long)__float2int_rn(__uint_as_float(v[i])) * (1 << 8 * (3 - (l & 3))) +
+                                    (long long)__float2int_rn(__uint_as_float(v[kAcc + i])) * (1 << 8 * (2 - (l & 3)));
                 if (l < 4) hi[i] += p;
                 else lo[i] += p;
             }
@@ -150,18 +155,22 @@ __device__ __forceinline__ void moments_tc_body(const MomentsTc &a, int tile, in
             if (a.status != nullptr) atomicOr(a.status, DEV_ERR_TIMEOUT);
         }
     };
+    float x[kPer];   // this thread's elites of the next stage, loaded a stage ahead
+    auto load = [&](int i) {
+        const int j0 = (first + i) * kStage + kPer * g;
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) x[q] = on && i < n && j0 + q < a.nu ? a.elites[(size_t)(j0 + q) * a.D + c] : 0.f;
+    };
+    load(0);
     for (int i = 0; i < n; ++i) {
         if (i >= 2) wait(i - 2);
         if (on) {
-            unsigned char *dst = buf + (size_t)(i & 1) * kStageBytes + (uint32_t)(c >> 3) * kSbo + (uint32_t)g * kLbo +
-                                 (uint32_t)(c & 7) * 16u;
-            const int j0 = (first + i) * kStage + 8 * g;
-            float x[8];
+            unsigned char *dst = buf + (size_t)(i & 1) * kStageBytes + (uint32_t)(c >> 3) * kSbo +
+                                 (uint32_t)(g >> 1) * kLbo + (uint32_t)(c & 7) * 16u + (uint32_t)(g & 1) * 8u;
+            const int j0 = (first + i) * kStage + kPer * g;
+            unsigned long long u[kPer];   // Z with every digit biased by 128
 #pragma unroll
-            for (int q = 0; q < 8; ++q) x[q] = j0 + q < a.nu ? a.elites[(size_t)(j0 + q) * a.D + c] : 0.f;
-            unsigned long long u[8];   // Z with every digit biased by 128
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
+            for (int q = 0; q < kPer; ++q) {
                 const bool in = j0 + q < a.nu;
                 const long long Y = in ? fixed_of(x[q], ey) - X1 : 0;
                 const long long Z = in ? scale63(Y, a.W[j0 + q]) : 0;
@@ -171,9 +180,9 @@ __device__ __forceinline__ void moments_tc_body(const MomentsTc &a, int tile, in
 #pragma unroll
             for (int s = 0; s < kDigits; ++s) {
                 const int byte = kDigits - 1 - s;   // digit s: bits 8 byte .. 8 byte + 7
-                uint32_t w[4];
+                uint32_t w[kPer / 2];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
+                for (int q = 0; q < kPer / 2; ++q) {
                     const uint32_t p = byte < 4 ? (uint32_t)u[2 * q] : (uint32_t)(u[2 * q] >> 32);
                     const uint32_t r = byte < 4 ? (uint32_t)u[2 * q + 1] : (uint32_t)(u[2 * q + 1] >> 32);
                     // two biased digits b = 128 h + m in 16-bit lanes; as BF16 (128 + m) - (256 -
@@ -182,9 +191,10 @@ __device__ __forceinline__ void moments_tc_body(const MomentsTc &a, int tile, in
                     const uint32_t m2 = (x2 & 0x007F007Fu) | 0x43004300u, h2 = (x2 & 0x00800080u) ^ 0x43804380u;
                     asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(w[q]) : "r"(m2), "r"(h2));
                 }
-                *reinterpret_cast<uint4 *>(dst + s * kSliceBytes) = make_uint4(w[0], w[1], w[2], w[3]);
+                *reinterpret_cast<uint2 *>(dst + s * kSliceBytes) = make_uint2(w[0], w[1]);
             }
         }
+        load(i + 1);
         tc::fence_async_smem();
         if (i > 0 && i % kEpoch == 0) {
             wait(i - 1);
@@ -229,8 +239,8 @@ __device__ __forceinline__ void moments_tc_body(const MomentsTc &a, int tile, in
     const int tiles = (a.D + kTcCols - 1) / kTcCols, row = 32 * (warp & 3) + lane;
     const size_t at = ((size_t)part * tiles + tile) * kTcCols;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        const size_t e = (at + 16 * (warp >> 2) + i) * kTcRows + row;
+    for (int i = 0; i < kAcc; ++i) {
+        const size_t e = (at + kAcc * (warp >> 2) + i) * kTcRows + row;
         a.hi[e] = hi[i];
         a.lo[e] = lo[i];
     }
@@ -382,7 +392,7 @@ int launch_moments_tc(const MomentsTc &a, int parts, int num_sms, cudaStream_t s
 {
     CP_CUDA(cudaMemsetAsync(a.colmax, 0, sizeof(uint32_t) * a.D, st));
     const int rows = (a.nu + 15) / 16;
-    k_moments_range<<<rows < num_sms ? rows : num_sms, 256, 0, st>>>(a);
+    k_moments_range<<<rows < 4 * num_sms ? rows : 4 * num_sms, 256, 0, st>>>(a);
     CP_LAUNCHED("k_moments_range");
     k_moments_tc<<<dim3(parts, moments_tc_tiles(a.D)), kTcThreads, kTcSmem, st>>>(a);
     CP_LAUNCHED("k_moments_tc");

@@ -126,6 +126,25 @@ static __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v)
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// 8 consecutive columns of this thread's lane, as tmem_ld16, without the wait: the registers
+// hold the values only after tmem_ld_wait() (several loads can be in flight before it).
+static __device__ __forceinline__ void tmem_ld8_async(uint32_t taddr, uint32_t *r)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+
+// Waits for this thread's tensor-memory loads; passing the registers through keeps their uses
+// behind the wait.
+template <int N>
+static __device__ __forceinline__ void tmem_ld_wait(uint32_t *r)
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < N; ++i) asm volatile("" : "+r"(r[i]));
+}
+
 // ---------------------------------------------------------------- MMA
 
 // Shared-memory matrix descriptor, K-major, no swizzle: start address, leading-dimension
