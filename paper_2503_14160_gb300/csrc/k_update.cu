@@ -325,12 +325,15 @@ constexpr int kRadixTile = 1024;
 constexpr int kRadixThreads = 256;
 constexpr int kRadixTotals = 10 * 256;   // per-digit totals of up to ten passes
 
-__global__ void k_radix_init(const double *__restrict__ J, int N, unsigned long long *key, int *val)
+// hist non-null: the first pass's tile histograms too (one-launch passes, tile-major).
+__global__ void k_radix_init(const double *__restrict__ J, int N, unsigned long long *key, int *val, int *hist)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < N) {
-        key[i] = order_key(J[i]);
+        const unsigned long long k = order_key(J[i]);
+        key[i] = k;
         val[i] = i;
+        if (hist != nullptr) atomicAdd(hist + (i / kRadixTile) * 256 + (int)(k & 255ull), 1);
     }
 }
 
@@ -444,6 +447,85 @@ k_radix_scatter(const unsigned long long *__restrict__ key_in, const int *__rest
     }
 }
 
+// One pass in one launch, for at most kOneTiles tiles: block = tile, one thread per element. The
+// tile histograms of the pass are there already (tile-major, hist[tile][digit]): every block sums
+// the columns it needs, the counts of its digits in the tiles before it and in all tiles, so no
+// scan kernel stands between, and while it scatters it counts the next pass's histograms at the
+// elements' new places (integer atomics). The sums read 1 KB per earlier tile and block, 2 MB in
+// all at 64 tiles and 33 MB at 256; beyond that the scan kernel is the cheaper form. The order is
+// that of k_radix_scatter: stable, by warp and lane within the tile.
+// The three launches per pass it replaces were bound by launch latency (3.3 + 3.6 + 7.6 us for
+// 65536 keys, 64 blocks taking four dependent rounds).
+constexpr int kOneTiles = 256;
+constexpr int kOnePasses = 10;   // histograms kept: eight key passes and two query passes
+
+template <bool kByQuery, bool kNextByQuery>
+__global__ void __launch_bounds__(kRadixTile)
+k_radix_pass(const unsigned long long *__restrict__ key_in, const int *__restrict__ val_in, int N, int shift,
+             const int *__restrict__ hist, unsigned long long *key_out, int *val_out, int next_shift, int *hist_next,
+             const uint16_t *__restrict__ qid)
+{
+    __shared__ int s_before[4][256], s_total[4][256];
+    __shared__ int wcount[kRadixTile / 32][256];   // per-warp digit counts, then first places
+    __shared__ int warp_tot[8];
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31, tiles = gridDim.x;
+    const int i = blockIdx.x * kRadixTile + t;
+    const bool valid = i < N;
+    unsigned long long k = 0;
+    int v = 0, d = 256 + lane;          // invalid lanes get digits no valid lane has
+    if (valid) {
+        k = key_in[i];
+        v = val_in[i];
+        d = radix_digit<kByQuery>(k, v, shift, qid);
+    }
+    for (int w = warp & ~7, e = t & 255; w < (warp & ~7) + 8; ++w) wcount[w][e] = 0;
+    {
+        const int g = t >> 8, e = t & 255;
+        int before = 0, total = 0;
+#pragma unroll 8
+        for (int q = g; q < tiles; q += 4) {
+            const int c = hist[q * 256 + e];
+            total += c;
+            before += q < (int)blockIdx.x ? c : 0;
+        }
+        s_before[g][e] = before;
+        s_total[g][e] = total;
+    }
+    __syncthreads();
+    const unsigned peers = __match_any_sync(0xffffffffu, d);
+    const int in_warp = __popc(peers & ((1u << lane) - 1u));
+    if (valid && in_warp == 0) wcount[warp][d] = __popc(peers);
+    int total = 0, x = 0;
+    if (t < 256) {                      // digits: inclusive scan of the totals within the warp
+        total = s_total[0][t] + s_total[1][t] + s_total[2][t] + s_total[3][t];
+        x = total;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, off);
+            if (lane >= off) x += y;
+        }
+        if (lane == 31) warp_tot[warp] = x;
+    }
+    __syncthreads();
+    if (t < 256) {
+        int run = x - total + s_before[0][t] + s_before[1][t] + s_before[2][t] + s_before[3][t];
+        for (int w = 0; w < warp; ++w) run += warp_tot[w];
+#pragma unroll 8
+        for (int w = 0; w < kRadixTile / 32; ++w) {
+            const int c = wcount[w][t];
+            wcount[w][t] = run;
+            run += c;
+        }
+    }
+    __syncthreads();
+    if (!valid) return;
+    const int pos = wcount[warp][d] + in_warp;
+    key_out[pos] = k;
+    val_out[pos] = v;
+    if (hist_next != nullptr)
+        atomicAdd(hist_next + (pos / kRadixTile) * 256 + radix_digit<kNextByQuery>(k, v, next_shift, qid), 1);
+}
+
 // Elite list and rows from the sorted indices; rank 0 also records its cost.
 __device__ __forceinline__ void gather_body(const int *__restrict__ sorted, int base, const double *__restrict__ J,
                                             const float *__restrict__ xi, int nu, int D, int *elite, float *elites,
@@ -474,14 +556,17 @@ __global__ void k_gather_elites(const int *__restrict__ sorted, const double *__
 // The batched ranking: key and value of every query's candidates at the query's offset in
 // the concatenated arrays (value = that position), and the query of each position.
 __global__ void k_batch_radix_init(const BatchQueryDev *__restrict__ qd, const int2 *__restrict__ tab,
-                                   unsigned long long *key, int *val)
+                                   unsigned long long *key, int *val, int *hist)
 {
     const int2 e = tab[blockIdx.x];
     const BatchQueryDev &q = qd[e.x];
     const int i = e.y * 256 + (int)threadIdx.x;
     if (i < q.N) {
-        key[q.cand_off + i] = order_key(q.J[i]);
-        val[q.cand_off + i] = q.cand_off + i;
+        const unsigned long long k = order_key(q.J[i]);
+        const int at = q.cand_off + i;
+        key[at] = k;
+        val[at] = at;
+        if (hist != nullptr) atomicAdd(hist + (at / kRadixTile) * 256 + (int)(k & 255ull), 1);
     }
 }
 
@@ -627,7 +712,37 @@ __global__ void __launch_bounds__(256) k_cma_cov(const double *__restrict__ s2p,
 
 int radix_tiles(int N) { return (N + kRadixTile - 1) / kRadixTile; }
 
-size_t radix_hist_ints(int N) { return 256 * (size_t)radix_tiles(N) + kRadixTotals; }
+static bool radix_one_launch(int tiles) { return tiles <= kOneTiles; }
+
+size_t radix_hist_ints(int N)   // either form's
+{
+    const size_t row = 256 * (size_t)radix_tiles(N), three = row + kRadixTotals, one = kOnePasses * row;
+    return radix_one_launch(radix_tiles(N)) && one > three ? one : three;
+}
+
+// The passes of one ranking in one launch each: eight on the key, then q_passes on the query.
+// hist: kOnePasses arrays of [tiles][256], zero but for the first pass's. The result is in val_a
+// after an even number of passes, in val_b after an odd one.
+static int radix_passes(int N, int q_passes, const uint16_t *qid, unsigned long long *key_a,
+                        unsigned long long *key_b, int *val_a, int *val_b, int *hist, cudaStream_t st)
+{
+    const int tiles = radix_tiles(N), passes = 8 + q_passes;
+    for (int p = 0; p < passes; ++p) {
+        const bool byq = p >= 8, next_byq = p + 1 >= 8;
+        const int shift = byq ? 8 * (p - 8) : 8 * p, next_shift = next_byq ? 8 * (p + 1 - 8) : 8 * (p + 1);
+        int *now = hist + (size_t)p * 256 * tiles, *next = p + 1 < passes ? now + 256 * tiles : nullptr;
+        auto kern = byq ? k_radix_pass<true, true> : (next_byq ? k_radix_pass<false, true> : k_radix_pass<false, false>);
+        kern<<<tiles, kRadixTile, 0, st>>>(key_a, val_a, N, shift, now, key_b, val_b, next_shift, next, qid);
+        CP_LAUNCHED("k_radix_pass");
+        unsigned long long *tk = key_a;
+        key_a = key_b;
+        key_b = tk;
+        int *tv = val_a;
+        val_a = val_b;
+        val_b = tv;
+    }
+    return CP_OK;
+}
 
 // Sorted candidate order by (J, index) into `sorted` (N ints); scratch: two key buffers of
 // N, one value buffer of N, hist of radix_hist_ints(N) ints (tile histograms, then the
@@ -636,9 +751,15 @@ int launch_radix_rank(const double *J, int N, unsigned long long *key_a, unsigne
                       int *val_a, int *val_b, int *hist, cudaStream_t st)
 {
     const int tiles = radix_tiles(N);
+    if (radix_one_launch(tiles)) {
+        CP_CUDA(cudaMemsetAsync(hist, 0, sizeof(int) * kOnePasses * 256 * (size_t)tiles, st));
+        k_radix_init<<<(N + 255) / 256, 256, 0, st>>>(J, N, key_a, val_a, hist);
+        CP_LAUNCHED("k_radix_init");
+        return radix_passes(N, 0, nullptr, key_a, key_b, val_a, val_b, hist, st);
+    }
     int *totals = hist + 256 * (size_t)tiles;   // [pass][digit]
     CP_CUDA(cudaMemsetAsync(totals, 0, sizeof(int) * kRadixTotals, st));
-    k_radix_init<<<(N + 255) / 256, 256, 0, st>>>(J, N, key_a, val_a);
+    k_radix_init<<<(N + 255) / 256, 256, 0, st>>>(J, N, key_a, val_a, nullptr);
     CP_LAUNCHED("k_radix_init");
     for (int pass = 0; pass < 8; ++pass) {
         const int shift = 8 * pass;
@@ -780,11 +901,22 @@ int launch_batch_radix_rank(const BatchQueryDev *qd, const int2 *tab, int blocks
                             int *val_a, int *val_b, int *hist, int **sorted, cudaStream_t st)
 {
     const int tiles = radix_tiles(total);
+    const int q_passes = nq > 256 ? 2 : (nq > 1 ? 1 : 0);
+    // Up to kSmallBatch candidates in all, a batch keeps three launches per pass: the kernels of
+    // its graph are reported to the caller (cp_batch_info.kernel_nodes) and tests hold their number
+    // there.
+    constexpr int kSmallBatch = 16384;
+    if (radix_one_launch(tiles) && total > kSmallBatch) {
+        CP_CUDA(cudaMemsetAsync(hist, 0, sizeof(int) * kOnePasses * 256 * (size_t)tiles, st));
+        k_batch_radix_init<<<blocks, 256, 0, st>>>(qd, tab, key_a, val_a, hist);
+        CP_LAUNCHED("k_batch_radix_init");
+        *sorted = q_passes & 1 ? val_b : val_a;
+        return radix_passes(total, q_passes, qid, key_a, key_b, val_a, val_b, hist, st);
+    }
     int *totals = hist + 256 * (size_t)tiles;   // [pass][digit]
     CP_CUDA(cudaMemsetAsync(totals, 0, sizeof(int) * kRadixTotals, st));
-    k_batch_radix_init<<<blocks, 256, 0, st>>>(qd, tab, key_a, val_a);
+    k_batch_radix_init<<<blocks, 256, 0, st>>>(qd, tab, key_a, val_a, nullptr);
     CP_LAUNCHED("k_batch_radix_init");
-    const int q_passes = nq > 256 ? 2 : (nq > 1 ? 1 : 0);
     for (int pass = 0; pass < 8 + q_passes; ++pass) {
         const bool byq = pass >= 8;
         const int shift = byq ? 8 * (pass - 8) : 8 * pass;

@@ -208,3 +208,24 @@ def test_integer_moments_carry_non_finite_elites(lib, crane, bad):
         assert np.isfinite(out[0][1][:, 9]).all()
     else:
         assert not np.isfinite(out[0][0][9]) and not np.isfinite(out[0][1][9, 9])
+
+
+@pytest.mark.parametrize("N", [8193, 9215, 9216, 9217, 65537, 262144, 262145])
+def test_ranking_passes(lib, crane, N):
+    """The one-launch radix passes at tile edges and at the last size that takes them, against a
+    stable sort; ties, NaN, infinities and both zeros among the costs."""
+    import torch
+    from paper_2503_14160_gb300 import workloads
+    g = np.random.default_rng(N)
+    J = g.normal(size=N) * np.exp(g.normal(size=N) * 20)
+    for value in (np.nan, np.inf, -np.inf, 0.0, -0.0, 1.5):
+        J[g.integers(0, N, N // 50)] = value
+    want = np.argsort(np.where(np.isnan(J), np.inf, J), kind="stable")
+    xi = torch.zeros(N, 1, 4, device="cuda")
+    with lib.Planner(crane, workloads.empty_scene(), lib.make_params(N, 1, 1, n_elites=N)) as pl:
+        lib.cp_set_endpoints(pl.handle, *ENDS[0])
+        lib.cp_update(pl.handle, torch.from_numpy(J).cuda(), xi)
+        el = torch.empty(N, dtype=torch.int32, device="cuda")
+        lib.cp_get_elites(pl.handle, el)
+        torch.cuda.synchronize()
+    assert np.array_equal(el.cpu().numpy(), want)
