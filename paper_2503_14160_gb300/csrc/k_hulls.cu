@@ -61,8 +61,17 @@ __device__ __forceinline__ float prism_support(float rc, float hz, float3 L)
 }
 
 // Smallest overlap over the axes of (box a, prism at centre pc) or (box a, axis-aligned box
-// with half extents bh); negative as soon as one axis separates.
-__device__ __forceinline__ float sat_prism(const Obb &a, float3 pc, float rc, float hz)
+// with half extents bh), or any overlap at most `floor` as soon as one is met: such a pair
+// cannot raise a running maximum that stands at floor >= 0, so the rest of its axes is left out.
+// r: the box's record in shared memory, whose axes the loops over the cross products take in
+// turn: rolled, because the unrolled code outgrew the instruction cache (a third of the cycles
+// were spent waiting for instructions).
+__device__ __forceinline__ float3 record_axis(const float *r, int k)
+{
+    return make_float3(r[3 + 3 * k], r[4 + 3 * k], r[5 + 3 * k]);
+}
+
+__device__ __forceinline__ float sat_prism(const Obb &a, const float *r, float3 pc, float rc, float hz, float floor)
 {
     const float3 d = make_float3(pc.x - a.c.x, pc.y - a.c.y, pc.z - a.c.z);
     float best = CUDART_INF_F;
@@ -76,18 +85,19 @@ __device__ __forceinline__ float sat_prism(const Obb &a, float3 pc, float rc, fl
         const float o = obb_support(a, L) + prism_support(rc, hz, L) - fabsf(dot3(d, L));
         best = fminf(best, o);
     }
-    if (best < 0.f) return best;
+    if (best <= floor) return best;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const float3 L = a.u[k];
         best = fminf(best, a.h[k] + prism_support(rc, hz, L) - fabsf(dot3(d, L)));
     }
-    if (best < 0.f) return best;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
+    if (best <= floor) return best;
+#pragma unroll 1
+    for (int k = 0; k < 3 && best > floor; ++k) {
+        const float3 u = record_axis(r, k);
 #pragma unroll
         for (int e = 0; e < 5; ++e) {
-            float3 L = cross3(a.u[k], dirs[e]);
+            float3 L = cross3(u, dirs[e]);
             const float n2 = dot3(L, L);
             if (n2 < 1e-12f) continue;   // parallel edges: no axis
             const float inv = rsqrtf(n2);
@@ -98,7 +108,7 @@ __device__ __forceinline__ float sat_prism(const Obb &a, float3 pc, float rc, fl
     return best;
 }
 
-__device__ __forceinline__ float sat_box(const Obb &a, float3 bc, float3 bh)
+__device__ __forceinline__ float sat_box(const Obb &a, const float *r, float3 bc, float3 bh, float floor)
 {
     const float3 d = make_float3(bc.x - a.c.x, bc.y - a.c.y, bc.z - a.c.z);
     float best = CUDART_INF_F;
@@ -109,19 +119,20 @@ __device__ __forceinline__ float sat_box(const Obb &a, float3 bc, float3 bh)
         const float3 L = e[k];
         best = fminf(best, obb_support(a, L) + hb[k] - fabsf(dot3(d, L)));
     }
-    if (best < 0.f) return best;
+    if (best <= floor) return best;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const float3 L = a.u[k];
         const float rb = fmaf(bh.x, fabsf(L.x), fmaf(bh.y, fabsf(L.y), bh.z * fabsf(L.z)));
         best = fminf(best, a.h[k] + rb - fabsf(dot3(d, L)));
     }
-    if (best < 0.f) return best;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
+    if (best <= floor) return best;
+#pragma unroll 1
+    for (int k = 0; k < 3 && best > floor; ++k) {
+        const float3 u = record_axis(r, k);
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            float3 L = cross3(a.u[k], e[j]);
+            float3 L = cross3(u, e[j]);
             const float n2 = dot3(L, L);
             if (n2 < 1e-12f) continue;
             const float inv = rsqrtf(n2);
@@ -142,6 +153,11 @@ struct HullArgs {
 
 constexpr int kHullWarps = kHullThreads / 32;
 constexpr int kBoxFloats = 16;   // centre, three axes, half extents, bounding radius
+// Floats of a lane's four boxes in shared memory: odd, so that the lanes' equal entries lie in
+// different banks (at 64 every store and every load of a pair's box hit one bank 32 times, and the
+// path form waited on shared memory for half of its cycles: 1.33 ms for the 4096 candidates of
+// the 500-tree query, 0.95 ms now).
+constexpr int kLaneFloats = 4 * kBoxFloats + 1;
 
 __device__ __forceinline__ void store_box(float *r, float3 c, float3 e, float3 n, float hl, float w, float h)
 {
@@ -167,10 +183,9 @@ __device__ __forceinline__ Obb load_box(const float *r)
 }
 
 // Depth of the four link boxes of one configuration against obstacle `ob` (cylinders
-// first, then boxes), 0 when disjoint.
-__device__ __forceinline__ float pair_depth(const SceneDev &sc, const float *boxes, int ob)
+// first, then boxes) where it exceeds `pen`, the configuration's depth so far, else that.
+__device__ __forceinline__ float pair_depth(const SceneDev &sc, const float *boxes, int ob, float pen)
 {
-    float pen = 0.f;
     if (ob < sc.n_cyl) {
         const float4 f = __ldg(sc.cyl_filt + ob), e = __ldg(sc.cyl_exact + ob);
         const float rc = e.x / kOctCos, hz = 0.5f * (e.z - e.y);
@@ -182,7 +197,7 @@ __device__ __forceinline__ float pair_depth(const SceneDev &sc, const float *box
             const float3 d = make_float3(pc.x - b.c.x, pc.y - b.c.y, pc.z - b.c.z);
             const float rr = b.rb + rbo;
             if (dot3(d, d) > rr * rr) continue;   // bounding spheres apart
-            pen = fmaxf(pen, sat_prism(b, pc, rc, hz));
+            pen = fmaxf(pen, sat_prism(b, boxes + l * kBoxFloats, pc, rc, hz, pen));
         }
     } else {
         const int bi = ob - sc.n_cyl;
@@ -194,7 +209,8 @@ __device__ __forceinline__ float pair_depth(const SceneDev &sc, const float *box
             const float3 d = make_float3(c.x - b.c.x, c.y - b.c.y, c.z - b.c.z);
             const float rr = b.rb + rbo;
             if (dot3(d, d) > rr * rr) continue;
-            pen = fmaxf(pen, sat_box(b, make_float3(c.x, c.y, c.z), make_float3(h.x, h.y, h.z)));
+            pen = fmaxf(pen, sat_box(b, boxes + l * kBoxFloats, make_float3(c.x, c.y, c.z),
+                                     make_float3(h.x, h.y, h.z), pen));
         }
     }
     return pen;
@@ -208,8 +224,9 @@ __device__ __forceinline__ void run_queue(const SceneDev &sc, const float *s_box
     if (lane < count) {
         const int e = queue[lane];
         const int owner = e & 31, ob = e >> 5;
-        const float pen = pair_depth(sc, s_boxes + owner * 4 * kBoxFloats, ob);
-        if (pen > 0.f) atomicMax(s_pen + owner, __float_as_int(pen));
+        const float so_far = __int_as_float(*(volatile int *)(s_pen + owner));
+        const float pen = pair_depth(sc, s_boxes + owner * kLaneFloats, ob, so_far);
+        if (pen > so_far) atomicMax(s_pen + owner, __float_as_int(pen));
     }
     __syncwarp();
 }
@@ -239,7 +256,7 @@ __device__ __forceinline__ float hull_pen_warp(const ModelDev &m, const SceneDev
     const float tl = m.jib_len + q.w;
     const float3 T = make_float3(fmaf(tl, ej.x, J.x), fmaf(tl, ej.y, J.y), fmaf(tl, ej.z, J.z));
     const float q4p = fmaxf(q.w, 0.f);
-    float *mine = s_box + lane * 4 * kBoxFloats;
+    float *mine = s_box + lane * kLaneFloats;
     const float hb = 0.5f * m.boom_len, hj = 0.5f * m.jib_len, tc = fmaf(0.5f, q4p, m.jib_len);
     store_box(mine, make_float3(hb * eb.x, hb * eb.y, fmaf(hb, eb.z, m.base_z)), eb, n, hb + hd.pad, hd.w[0],
               hd.hh[0]);
@@ -329,7 +346,7 @@ __device__ __forceinline__ float hull_pen_warp(const ModelDev &m, const SceneDev
 __global__ void __launch_bounds__(kHullThreads)
 k_hull_penetration(const ModelDev m, const SceneDev sc, const HullArgs a)
 {
-    __shared__ float s_box[kHullWarps][32 * 4 * kBoxFloats];
+    __shared__ float s_box[kHullWarps][32 * kLaneFloats];
     __shared__ int s_pen[kHullWarps][32];
     __shared__ int s_queue[kHullWarps][64];
     const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -348,7 +365,7 @@ __global__ void __launch_bounds__(kHullThreads)
 k_eval_hulls(const ModelDev m, const SceneDev sc, const HullDims hd, const EvalArgs a)
 {
     extern __shared__ __align__(16) float4 s_basis[];
-    __shared__ float s_box[kHullWarps][32 * 4 * kBoxFloats];
+    __shared__ float s_box[kHullWarps][32 * kLaneFloats];
     __shared__ int s_pen[kHullWarps][32];
     __shared__ int s_queue[kHullWarps][64];
     __shared__ float4 s_ctrl_all[kHullWarps][CP_MAX_WAYPOINTS + 8];
