@@ -43,21 +43,78 @@ __device__ __forceinline__ float3 cross3(float3 a, float3 b)
     return make_float3(fmaf(a.y, b.z, -a.z * b.y), fmaf(a.z, b.x, -a.x * b.z), fmaf(a.x, b.y, -a.y * b.x));
 }
 
+// Axes with components that are zero by construction (Z: a bit per component, x lowest). The
+// compiler keeps a product by a zero it knows, since 0 times infinity is not 0; the forms below
+// leave it out: fma(a, 0, b) is b and fma(a, b, 0) is the rounded a b, so the values are the same
+// (rounded products as such: the compiler may not join them with a later sum).
+constexpr int kZx = 1, kZy = 2, kZz = 4;
+
+template <int Z>
+__device__ __forceinline__ float dot_axis(float3 u, float3 L)
+{
+    if (Z == 0) return dot3(u, L);
+    if (Z == kZx) return fmaf(u.y, L.y, u.z * L.z);
+    if (Z == kZy) return fmaf(u.x, L.x, u.z * L.z);
+    if (Z == kZz) return fmaf(u.x, L.x, u.y * L.y);
+    if (Z == (kZy | kZz)) return __fmul_rn(u.x, L.x);
+    if (Z == (kZx | kZz)) return __fmul_rn(u.y, L.y);
+    return __fmul_rn(u.z, L.z);
+}
+
+template <int Z>
 __device__ __forceinline__ float obb_support(const Obb &a, float3 L)
 {
-    return fmaf(a.h[0], fabsf(dot3(a.u[0], L)), fmaf(a.h[1], fabsf(dot3(a.u[1], L)), a.h[2] * fabsf(dot3(a.u[2], L))));
+    return fmaf(a.h[0], fabsf(dot_axis<Z>(a.u[0], L)),
+                fmaf(a.h[1], fabsf(dot_axis<Z>(a.u[1], L)), a.h[2] * fabsf(dot_axis<Z>(a.u[2], L))));
 }
 
 // Support of the octagonal prism (circumradius rc, half height hz) along a unit axis: the
 // largest |v . L| over the four vertex directions at (k + 1/2) 45 degrees, times rc, plus
 // hz |L_z|.
+template <int Z>
 __device__ __forceinline__ float prism_support(float rc, float hz, float3 L)
 {
     // vertex directions (cos, sin) of 22.5 and 67.5 degrees; the other two are their mirrors
     const float a = 0.92387953251128674f, b = 0.38268343236508977f;
-    const float v0 = fabsf(fmaf(a, L.x, b * L.y)), v1 = fabsf(fmaf(b, L.x, a * L.y));
-    const float v2 = fabsf(fmaf(-b, L.x, a * L.y)), v3 = fabsf(fmaf(-a, L.x, b * L.y));
-    return fmaf(rc, fmaxf(fmaxf(v0, v1), fmaxf(v2, v3)), hz * fabsf(L.z));
+    float v;
+    if ((Z & (kZx | kZy)) == (kZx | kZy)) return __fmul_rn(hz, fabsf(L.z));
+    if (Z & kZx) {
+        v = fabsf(__fmul_rn(a, L.y));                       // the larger factor of the two
+    } else if (Z & kZy) {
+        v = fabsf(__fmul_rn(a, L.x));
+    } else {
+        const float v0 = fabsf(fmaf(a, L.x, b * L.y)), v1 = fabsf(fmaf(b, L.x, a * L.y));
+        const float v2 = fabsf(fmaf(-b, L.x, a * L.y)), v3 = fabsf(fmaf(-a, L.x, b * L.y));
+        v = fmaxf(fmaxf(v0, v1), fmaxf(v2, v3));
+    }
+    return Z & kZz ? __fmul_rn(rc, v) : fmaf(rc, v, hz * fabsf(L.z));
+}
+
+template <int Z>
+__device__ __forceinline__ float prism_overlap(const Obb &a, float rc, float hz, float3 d, float3 L)
+{
+    return obb_support<Z>(a, L) + prism_support<Z>(rc, hz, L) - fabsf(dot_axis<Z>(d, L));
+}
+
+template <int Z>
+__device__ __forceinline__ float box_overlap(const Obb &a, float3 bh, float3 d, float3 L)
+{
+    float rb;
+    if (Z == kZx) rb = fmaf(bh.y, fabsf(L.y), bh.z * fabsf(L.z));
+    else if (Z == kZy) rb = fmaf(bh.x, fabsf(L.x), bh.z * fabsf(L.z));
+    else rb = fmaf(bh.x, fabsf(L.x), bh.y * fabsf(L.y));   // kZz
+    return obb_support<Z>(a, L) + rb - fabsf(dot_axis<Z>(d, L));
+}
+
+// L / |L| for a cross product of two edges; false when they are parallel (no axis).
+template <int Z>
+__device__ __forceinline__ bool unit_axis(float3 &L)
+{
+    const float n2 = dot_axis<Z>(L, L);
+    if (n2 < 1e-12f) return false;
+    const float inv = rsqrtf(n2);
+    L = make_float3(L.x * inv, L.y * inv, L.z * inv);
+    return true;
 }
 
 // Smallest overlap over the axes of (box a, prism at centre pc) or (box a, axis-aligned box
@@ -74,36 +131,33 @@ __device__ __forceinline__ float3 record_axis(const float *r, int k)
 __device__ __forceinline__ float sat_prism(const Obb &a, const float *r, float3 pc, float rc, float hz, float floor)
 {
     const float3 d = make_float3(pc.x - a.c.x, pc.y - a.c.y, pc.z - a.c.z);
-    float best = CUDART_INF_F;
+    const float h = kSqrtHalf;
     // prism faces: z, then the four side normals at multiples of 45 degrees
-    const float3 dirs[5] = {make_float3(0.f, 0.f, 1.f), make_float3(1.f, 0.f, 0.f),
-                            make_float3(kSqrtHalf, kSqrtHalf, 0.f), make_float3(0.f, 1.f, 0.f),
-                            make_float3(-kSqrtHalf, kSqrtHalf, 0.f)};
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        const float3 L = dirs[k];
-        const float o = obb_support(a, L) + prism_support(rc, hz, L) - fabsf(dot3(d, L));
-        best = fminf(best, o);
-    }
+    float best = prism_overlap<kZx | kZy>(a, rc, hz, d, make_float3(0.f, 0.f, 1.f));
+    best = fminf(best, prism_overlap<kZy | kZz>(a, rc, hz, d, make_float3(1.f, 0.f, 0.f)));
+    best = fminf(best, prism_overlap<kZz>(a, rc, hz, d, make_float3(h, h, 0.f)));
+    best = fminf(best, prism_overlap<kZx | kZz>(a, rc, hz, d, make_float3(0.f, 1.f, 0.f)));
+    best = fminf(best, prism_overlap<kZz>(a, rc, hz, d, make_float3(-h, h, 0.f)));
     if (best <= floor) return best;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const float3 L = a.u[k];
-        best = fminf(best, a.h[k] + prism_support(rc, hz, L) - fabsf(dot3(d, L)));
+        best = fminf(best, a.h[k] + prism_support<0>(rc, hz, L) - fabsf(dot3(d, L)));
     }
     if (best <= floor) return best;
 #pragma unroll 1
     for (int k = 0; k < 3 && best > floor; ++k) {
         const float3 u = record_axis(r, k);
-#pragma unroll
-        for (int e = 0; e < 5; ++e) {
-            float3 L = cross3(u, dirs[e]);
-            const float n2 = dot3(L, L);
-            if (n2 < 1e-12f) continue;   // parallel edges: no axis
-            const float inv = rsqrtf(n2);
-            L = make_float3(L.x * inv, L.y * inv, L.z * inv);
-            best = fminf(best, obb_support(a, L) + prism_support(rc, hz, L) - fabsf(dot3(d, L)));
-        }
+        float3 L = make_float3(u.y, -u.x, 0.f);                       // u x z
+        if (unit_axis<kZz>(L)) best = fminf(best, prism_overlap<kZz>(a, rc, hz, d, L));
+        L = make_float3(0.f, u.z, -u.y);                              // u x (1, 0, 0)
+        if (unit_axis<kZx>(L)) best = fminf(best, prism_overlap<kZx>(a, rc, hz, d, L));
+        L = make_float3(-(u.z * h), u.z * h, fmaf(u.x, h, -(u.y * h)));   // u x (h, h, 0)
+        if (unit_axis<0>(L)) best = fminf(best, prism_overlap<0>(a, rc, hz, d, L));
+        L = make_float3(-u.z, 0.f, u.x);                              // u x (0, 1, 0)
+        if (unit_axis<kZy>(L)) best = fminf(best, prism_overlap<kZy>(a, rc, hz, d, L));
+        L = make_float3(-(u.z * h), -(u.z * h), fmaf(u.x, h, u.y * h));   // u x (-h, h, 0)
+        if (unit_axis<0>(L)) best = fminf(best, prism_overlap<0>(a, rc, hz, d, L));
     }
     return best;
 }
@@ -111,14 +165,9 @@ __device__ __forceinline__ float sat_prism(const Obb &a, const float *r, float3 
 __device__ __forceinline__ float sat_box(const Obb &a, const float *r, float3 bc, float3 bh, float floor)
 {
     const float3 d = make_float3(bc.x - a.c.x, bc.y - a.c.y, bc.z - a.c.z);
-    float best = CUDART_INF_F;
-    const float3 e[3] = {make_float3(1.f, 0.f, 0.f), make_float3(0.f, 1.f, 0.f), make_float3(0.f, 0.f, 1.f)};
-    const float hb[3] = {bh.x, bh.y, bh.z};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const float3 L = e[k];
-        best = fminf(best, obb_support(a, L) + hb[k] - fabsf(dot3(d, L)));
-    }
+    float best = obb_support<kZy | kZz>(a, make_float3(1.f, 0.f, 0.f)) + bh.x - fabsf(d.x);
+    best = fminf(best, obb_support<kZx | kZz>(a, make_float3(0.f, 1.f, 0.f)) + bh.y - fabsf(d.y));
+    best = fminf(best, obb_support<kZx | kZy>(a, make_float3(0.f, 0.f, 1.f)) + bh.z - fabsf(d.z));
     if (best <= floor) return best;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -130,16 +179,12 @@ __device__ __forceinline__ float sat_box(const Obb &a, const float *r, float3 bc
 #pragma unroll 1
     for (int k = 0; k < 3 && best > floor; ++k) {
         const float3 u = record_axis(r, k);
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            float3 L = cross3(u, e[j]);
-            const float n2 = dot3(L, L);
-            if (n2 < 1e-12f) continue;
-            const float inv = rsqrtf(n2);
-            L = make_float3(L.x * inv, L.y * inv, L.z * inv);
-            const float rb = fmaf(bh.x, fabsf(L.x), fmaf(bh.y, fabsf(L.y), bh.z * fabsf(L.z)));
-            best = fminf(best, obb_support(a, L) + rb - fabsf(dot3(d, L)));
-        }
+        float3 L = make_float3(0.f, u.z, -u.y);                       // u x (1, 0, 0)
+        if (unit_axis<kZx>(L)) best = fminf(best, box_overlap<kZx>(a, bh, d, L));
+        L = make_float3(-u.z, 0.f, u.x);                              // u x (0, 1, 0)
+        if (unit_axis<kZy>(L)) best = fminf(best, box_overlap<kZy>(a, bh, d, L));
+        L = make_float3(u.y, -u.x, 0.f);                              // u x (0, 0, 1)
+        if (unit_axis<kZz>(L)) best = fminf(best, box_overlap<kZz>(a, bh, d, L));
     }
     return best;
 }
