@@ -171,7 +171,7 @@ struct cp_planner {
     float *grad = nullptr;      // [N][D] gradient buffer for polish
     float4 *ends_f = nullptr;   // [2] {q0, qd} in float, written with the end points
     unsigned long long *work = nullptr;   // [2] broad-phase survivors and box tests while timing
-    int *eval_queue = nullptr;            // the polar evaluation's item counter
+    int *eval_queue = nullptr;            // [2] item counters of the evaluation and of the smooth cost
     size_t item_cap = 0;                  // work items the item_sum / item_count buffers hold
     unsigned long long *rkey_a = nullptr, *rkey_b = nullptr;   // radix sort scratch
     int *rval_a = nullptr, *rval_b = nullptr, *rhist = nullptr;
@@ -507,7 +507,7 @@ int run_eval(cp_planner *p, const float *d_xi, int n, double *d_J, uint8_t *d_fl
     rc = p->timer.end(ST_EVAL, p->st);
     if (rc != CP_OK) return rc;
     return launch_eval_finalize(p->item_sum, p->item_count, n, a.P, p->prm.w_c, p->prm.w_l, p->prm.lambda_c,
-                                d_J, d_flag, d_terms, p->st);
+                                d_J, d_flag, d_terms, p->st, nullptr, p->eval_queue);
 }
 
 int run_factor(cp_planner *p)
@@ -558,7 +558,6 @@ int run_update(cp_planner *p, const double *d_J, const float *d_xi)
             return rc;
     }
     if (p->prm.update_rule == CP_UPDATE_CMAES) {
-        CP_CUDA(cudaMemcpyAsync(p->mu_prev, p->mu, sizeof(double) * p->D, cudaMemcpyDeviceToDevice, p->st));
         if ((rc = launch_cma_update(p->elites, p->w, p->nu, p->D, p->mu_prev, p->L, p->cmak, p->iteration,
                                     p->mom_y, p->cov_part, p->mean_part, p->mu, p->C, p->p_sigma, p->p_c, p->cma,
                                     p->st)) != CP_OK)
@@ -798,7 +797,7 @@ int cp_plan_init(const cp_model *model, const cp_scene *scene, const cp_params *
     const size_t o_sp_g = L.take<float>(units_max * D);
     const size_t o_sp_J = L.take<double>(units_max);
     const size_t o_work = L.take<unsigned long long>(2);
-    const size_t o_eval_queue = L.take<int>(1);
+    const size_t o_eval_queue = L.take<int>(2);
     const size_t o_metrics = L.take<double>((size_t)kMetricsRing * kMetricsCols);
     const size_t o_metrics_part = L.take<double>(3 * (size_t)kMetricsBlocks);
     const size_t o_cma = L.take<double>(4);
@@ -969,6 +968,7 @@ int cp_set_endpoints(cp_planner *p, const double h_q0[4], const double h_qd[4])
     CP_CUDA(cudaMemcpyAsync(p->consts, ends, sizeof ends, cudaMemcpyHostToDevice, p->st));
     // the rank counters are zero between updates; a reset restores that after any failure
     CP_CUDA(cudaMemsetAsync(p->rank, 0, sizeof(int) * p->N, p->st));
+    CP_CUDA(cudaMemsetAsync(p->eval_queue, 0, sizeof(int), p->st));   // and so is the evaluation's item counter
     p->q0f = make_float4((float)h_q0[0], (float)h_q0[1], (float)h_q0[2], (float)h_q0[3]);
     p->qdf = make_float4((float)h_qd[0], (float)h_qd[1], (float)h_qd[2], (float)h_qd[3]);
     int rc = launch_init_distribution(p->consts, p->consts + 4, p->consts + 8, p->consts + 12, p->K,
@@ -1147,7 +1147,7 @@ static int run_smooth(cp_planner *p, const float *xi, int n, const double *gJ, d
 {
     return launch_smooth(p->mdev, p->sdev, xi, n, p->K, p->S, p->q0f, p->qdf, p->basis,
                          p->prm.smooth_margin, p->prm.smooth_beta, p->prm.w_c * p->prm.lambda_c,
-                         p->prm.w_l, gJ, J, dxi, p->smooth_part_g, p->smooth_part_J, p->eval_queue,
+                         p->prm.w_l, gJ, J, dxi, p->smooth_part_g, p->smooth_part_J, p->eval_queue + 1,
                          p->num_sms, p->st);
 }
 

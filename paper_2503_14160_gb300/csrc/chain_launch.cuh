@@ -1,0 +1,43 @@
+// Launches of a chain of dependent kernels (programmatic dependent launch). A plan's iteration is
+// some ten short kernels, each needing all of the one before, so the gap between them counts: with
+// the attribute below a kernel's blocks may be placed while the kernel before still runs, and
+// after_previous(), the first statement of every such kernel, waits until that one has completed
+// and its writes are visible. Every kernel of a chain waits, so completion is transitive: whatever
+// follows a kernel on the stream sees everything before it. The wait has no limit of its own: it
+// ends when the kernel before ends, as an ordinary launch would begin.
+// Measured with the node that cleared the evaluation's counter gone too: an iteration of the 20-tree
+// query 59 -> 48.5 us, update and sample of 65536 candidates 382 -> 356 us.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace cp {
+
+#ifdef __CUDACC__
+// Waits for the kernel before, then lets the next one's blocks be placed.
+static __device__ __forceinline__ void after_previous()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// kern<<<grid, block, smem, st>>>(args...) with the attribute. The kernel's first statement is
+// after_previous().
+template <typename... P, typename... A>
+inline void launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);   // an error is the last error, as of <<<>>>
+}
+#endif
+
+}  // namespace cp

@@ -173,8 +173,9 @@ struct EvalArgs {
     unsigned long long *work;   // optional [2]: += obstacles that passed the unit box test,
                                 // += (unit, obstacle) box tests run (polar index form)
     uint32_t *status;           // device status word (DEV_ERR_*) or null
-    int *queue;                 // polar form: the next work item to take (zeroed before each
-                                // launch); null: items in a fixed stride over the warps
+    int *queue;                 // the next work item to take (zero before the launch; the
+                                // finalize that follows sets it back); null: items in a fixed
+                                // stride over the warps
     const float4 *basis;        // [S][2]: {b0..b3}(u_m), {b0..b3}(u_m) - {b0..b3}(u_{m-1})
     double *item_sum;           // [n][P][4] {J_p, sum pen, J_l, length}
     uint32_t *item_count;       // [n][P] checkpoints in collision
@@ -209,7 +210,8 @@ int launch_eval(const ModelDev &m, const SceneDev &sc, const EvalArgs &a, int nu
 int launch_eval_finalize(const double *item_sum, const uint32_t *item_count, int n, int P,
                          double w_c, double w_l, double lambda_c, double *J, uint8_t *flag,
                          double *terms, cudaStream_t st,
-                         const uint32_t *status = nullptr);   // nonzero *status: NaN J, flagged
+                         const uint32_t *status = nullptr,    // nonzero *status: NaN J, flagged
+                         int *queue = nullptr);               // the evaluation's item counter: back to zero
 int launch_signed_distance(const ModelDev &m, const SceneDev &sc, const float *q, int n,
                            float *d, cudaStream_t st);
 int launch_ik(const ModelDev &m, const SceneDev &sc, const float *targets, const float *q_init, int n,
@@ -285,7 +287,7 @@ struct CmaConsts {
 };
 CmaConsts cma_consts(int D, int nu);
 int launch_cma_reset(double sigma0, int D, double *cma, double *p_sigma, double *p_c, cudaStream_t st);
-int launch_cma_update(const float *elites, const double *w, int nu, int D, const double *mu_prev,
+int launch_cma_update(const float *elites, const double *w, int nu, int D, double *mu_prev,
                       const double *L, const CmaConsts &k, int t, double *yw, double *s2p, double *s1p, double *mu,
                       double *C, double *p_sigma, double *p_c, double *cma, cudaStream_t st);
 int elite_slices(int N, int D, int nu, int num_sms);

@@ -1,5 +1,5 @@
 // How the warps of an evaluation launch take its work items. With a counter
-// (EvalArgs::queue, zeroed before the launch) lane 0 takes the next item and the warp shares
+// (EvalArgs::queue, zero before the launch) lane 0 takes the next item and the warp shares
 // it, so candidates of uneven cost (those in contact take the exact distances) even out over
 // the warps; without one the items go round the warps in a fixed stride. The counter only
 // grows, so every warp leaves once the items are handed out. Called by whole warps.

@@ -11,6 +11,7 @@
 // against every cylinder; only pairs that pass it (sphere within reach of the cylinder) take
 // the exact capped-cylinder distance. A second kernel adds each candidate's item sums in a
 // fixed order in FP64.
+#include "chain_launch.cuh"
 #include "eval_common.cuh"
 #include "item_queue.cuh"
 
@@ -183,6 +184,7 @@ template <int NSPH>
 __global__ void __launch_bounds__(kEvalThreads, kEvalBroadMinBlocks)
 k_eval_broad(const ModelDev m, const SceneDev sc, const EvalArgs a)
 {
+    after_previous();
     extern __shared__ __align__(16) float4 smem[];
     float4 *s_filt = smem;
     float4 *s_exact = s_filt + sc.n_cyl;
@@ -267,6 +269,7 @@ template <int NSPH>
 __global__ void __launch_bounds__(kEvalThreads, kEvalMinBlocks)
 k_eval(const ModelDev m, const SceneDev sc, const EvalArgs a)
 {
+    after_previous();
     // Shared memory: per cylinder the filter record {cx, cy, W, reach} and the exact record
     // {R, z_lo, z_hi, bound}; per box its centre and half extent; the spline basis table.
     extern __shared__ __align__(16) float4 smem[];
@@ -438,17 +441,16 @@ int launch_eval(const ModelDev &m, const SceneDev &sc, const EvalArgs &a, int nu
     if (units == 0) return CP_OK;
     const size_t smem = eval_smem_bytes(sc.n_cyl, sc.n_box, a.S);
     const int cpsm = a.ctas_per_sm;
-    if (a.queue != nullptr) CP_CUDA(cudaMemsetAsync(a.queue, 0, sizeof(int), st));
     if (m.n_spheres == 12) {
         if (a.broadphase)
-            k_eval_broad<12><<<eval_grid(k_eval_broad<12>, smem, num_sms, units, cpsm), kEvalThreads, smem, st>>>(m, sc, a);
+            launch_chained(k_eval_broad<12>, eval_grid(k_eval_broad<12>, smem, num_sms, units, cpsm), kEvalThreads, smem, st, m, sc, a);
         else
-            k_eval<12><<<eval_grid(k_eval<12>, smem, num_sms, units, cpsm), kEvalThreads, smem, st>>>(m, sc, a);
+            launch_chained(k_eval<12>, eval_grid(k_eval<12>, smem, num_sms, units, cpsm), kEvalThreads, smem, st, m, sc, a);
     } else {
         if (a.broadphase)
-            k_eval_broad<16><<<eval_grid(k_eval_broad<16>, smem, num_sms, units, cpsm), kEvalThreads, smem, st>>>(m, sc, a);
+            launch_chained(k_eval_broad<16>, eval_grid(k_eval_broad<16>, smem, num_sms, units, cpsm), kEvalThreads, smem, st, m, sc, a);
         else
-            k_eval<16><<<eval_grid(k_eval<16>, smem, num_sms, units, cpsm), kEvalThreads, smem, st>>>(m, sc, a);
+            launch_chained(k_eval<16>, eval_grid(k_eval<16>, smem, num_sms, units, cpsm), kEvalThreads, smem, st, m, sc, a);
     }
     CP_LAUNCHED("k_eval");
     return CP_OK;

@@ -25,6 +25,7 @@
 // (the pivot's chain); the last CTA's early columns, with up to 64 pairs, 1300 on average.
 #include <cooperative_groups.h>
 
+#include "chain_launch.cuh"
 #include "cp_internal.cuh"
 #include "fp64_chain.cuh"
 #include "tcgen05.cuh"
@@ -207,6 +208,7 @@ __global__ void __launch_bounds__(kFactorThreads)
 k_factor(const double *__restrict__ C, double sigma2, const double *__restrict__ sigma_dev, int D, double *L,
          float *Lt, uint32_t *status)
 {
+    after_previous();
     extern __shared__ __align__(16) double sm[];
     if (sigma_dev != nullptr) sigma2 = sigma_dev[0] * sigma_dev[0];   // the step size kept on the device
     factor_cluster(C, sigma2, D, (int)gridDim.x, L, Lt, status, sm);
@@ -222,19 +224,21 @@ k_batch_factor_cluster(const BatchQueryDev *__restrict__ qd, int n_ctas)
 }
 
 struct ClusterLaunch {
-    cudaLaunchAttribute attr{};
+    cudaLaunchAttribute attr[2] = {};
     cudaLaunchConfig_t cfg{};
-    ClusterLaunch(int blocks, int n_ctas, cudaStream_t st)
+    ClusterLaunch(int blocks, int n_ctas, cudaStream_t st, bool chained)
     {
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = n_ctas;
-        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = n_ctas;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // k_factor: chain_launch.cuh
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.gridDim = dim3(blocks);
         cfg.blockDim = dim3(kFactorThreads);
         cfg.dynamicSmemBytes = factor_smem(n_ctas);
         cfg.stream = st;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = chained ? 2 : 1;
     }
 };
 
@@ -252,7 +256,7 @@ int launch_factor(const double *C, double sigma2, const double *sigma_dev, int D
                   float *Lt_f, uint32_t *status, cudaStream_t st)
 {
     const int n_ctas = (D + kRows - 1) / kRows;
-    const ClusterLaunch l(n_ctas, n_ctas, st);
+    const ClusterLaunch l(n_ctas, n_ctas, st, true);
     CP_CUDA(cudaLaunchKernelEx(&l.cfg, k_factor, C, sigma2, sigma_dev, D, L, Lt_f, status));
     CP_LAUNCHED("k_factor");
     return CP_OK;
@@ -260,7 +264,7 @@ int launch_factor(const double *C, double sigma2, const double *sigma_dev, int D
 
 int batch_factor_clusters(int max_D, int *count)
 {
-    const ClusterLaunch l(kMaxCtas, (max_D + kRows - 1) / kRows, nullptr);
+    const ClusterLaunch l(kMaxCtas, (max_D + kRows - 1) / kRows, nullptr, false);
     CP_CUDA(cudaOccupancyMaxActiveClusters(count, k_batch_factor_cluster, &l.cfg));
     return CP_OK;
 }
@@ -268,7 +272,7 @@ int batch_factor_clusters(int max_D, int *count)
 int launch_batch_factor_cluster(const BatchQueryDev *qd, int nq, int max_D, cudaStream_t st)
 {
     const int n_ctas = (max_D + kRows - 1) / kRows;
-    const ClusterLaunch l(nq * n_ctas, n_ctas, st);
+    const ClusterLaunch l(nq * n_ctas, n_ctas, st, false);
     CP_CUDA(cudaLaunchKernelEx(&l.cfg, k_batch_factor_cluster, qd, n_ctas));
     CP_LAUNCHED("k_batch_factor_cluster");
     return CP_OK;

@@ -8,6 +8,7 @@
 // and eight items' loads are in flight before the dependent FP64 additions (each holds a
 // scheduler's FP64 unit for some 70 cycles whatever its lanes do) take them in item order. The
 // kernel is bound by the latency of one such chain.
+#include "chain_launch.cuh"
 #include "cp_internal.cuh"
 
 namespace cp {
@@ -72,8 +73,10 @@ __device__ __forceinline__ void finalize_body(const double *__restrict__ item_su
 __global__ void __launch_bounds__(256)
 k_eval_finalize(const double *__restrict__ item_sum, const uint32_t *__restrict__ item_count, int n, int P,
                 double w_c, double w_l, double lambda_c, double *J, uint8_t *flag, double *terms,
-                const uint32_t *status)
+                const uint32_t *status, int *queue)
 {
+    after_previous();
+    if (queue != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *queue = 0;
     const int t = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     finalize_body(item_sum, item_count, n, P, w_c, w_l, lambda_c, J, flag, terms, status, t / kFinalLanes,
                   t % kFinalLanes);
@@ -102,12 +105,11 @@ k_batch_finalize(const BatchQueryDev *__restrict__ qd, const int2 *__restrict__ 
 
 int launch_eval_finalize(const double *item_sum, const uint32_t *item_count, int n, int P,
                          double w_c, double w_l, double lambda_c, double *J, uint8_t *flag,
-                         double *terms, cudaStream_t st, const uint32_t *status)
+                         double *terms, cudaStream_t st, const uint32_t *status, int *queue)
 {
     if (n == 0) return CP_OK;
     const int threads = 256, per = threads / kFinalLanes;
-    k_eval_finalize<<<(unsigned)((n + per - 1) / per), threads, 0, st>>>(
-        item_sum, item_count, n, P, w_c, w_l, lambda_c, J, flag, terms, status);
+    launch_chained(k_eval_finalize, (unsigned)((n + per - 1) / per), threads, 0, st,  item_sum, item_count, n, P, w_c, w_l, lambda_c, J, flag, terms, status, queue);
     CP_LAUNCHED("k_eval_finalize");
     return CP_OK;
 }

@@ -19,6 +19,7 @@
 // not matter because the kernel takes a minimum of exactly computed distances.
 #include <cmath>
 
+#include "chain_launch.cuh"
 #include "eval_common.cuh"
 
 namespace cp {
@@ -244,6 +245,7 @@ template <int NSPH, bool kExtras>
 __global__ void __launch_bounds__(kPolarThreads, CP_POLAR_MIN_BLOCKS)
 k_eval_polar(const ModelDev m, const SceneDev sc, const PolarDev g, const EvalArgs a)
 {
+    after_previous();
     // Shared memory: the spline table, then per warp the control points of its candidate.
     extern __shared__ __align__(16) float4 s_basis[];
     float4 *s_ctrl = s_basis + 2 * a.S + (threadIdx.x >> 5) * kCtrlSlots;
@@ -414,8 +416,7 @@ int launch_eval_polar(const ModelDev &m, const SceneDev &sc, const PolarDev &g, 
     const int needed = (items + kPolarThreads / 32 - 1) / (kPolarThreads / 32);
     int grid = num_sms * per_sm;
     if (grid > needed) grid = needed;
-    if (a.queue != nullptr) CP_CUDA(cudaMemsetAsync(a.queue, 0, sizeof(int), st));
-    kern<<<grid, kPolarThreads, smem, st>>>(m, sc, g, a);
+    launch_chained(kern, grid, kPolarThreads, smem, st, m, sc, g, a);
     CP_LAUNCHED("k_eval_polar");
     return CP_OK;
 }

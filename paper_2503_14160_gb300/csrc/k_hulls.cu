@@ -19,6 +19,7 @@
 // lane; a pair whose bounding spheres (the link box's and the obstacle's) do not meet is
 // skipped, and a pair's axes are tried with the cheap obstacle axes first and stop at the
 // first separating one.
+#include "chain_launch.cuh"
 #include "eval_common.cuh"
 #include "item_queue.cuh"
 
@@ -409,6 +410,7 @@ k_hull_penetration(const ModelDev m, const SceneDev sc, const HullArgs a)
 __global__ void __launch_bounds__(kHullThreads)
 k_eval_hulls(const ModelDev m, const SceneDev sc, const HullDims hd, const EvalArgs a)
 {
+    after_previous();
     extern __shared__ __align__(16) float4 s_basis[];
     __shared__ float s_box[kHullWarps][32 * kLaneFloats];
     __shared__ int s_pen[kHullWarps][32];
@@ -462,8 +464,7 @@ int launch_eval_hulls(const ModelDev &m, const SceneDev &sc, const HullDims &d, 
     const long long items = (long long)a.n * a.P;
     long long blocks = (items + kHullWarps - 1) / kHullWarps;
     if (blocks > (long long)num_sms * per_sm) blocks = (long long)num_sms * per_sm;
-    if (a.queue != nullptr) CP_CUDA(cudaMemsetAsync(a.queue, 0, sizeof(int), st));
-    k_eval_hulls<<<(unsigned)blocks, kHullThreads, smem, st>>>(m, sc, d, a);
+    launch_chained(k_eval_hulls, (unsigned)blocks, kHullThreads, smem, st, m, sc, d, a);
     CP_LAUNCHED("k_eval_hulls");
     return CP_OK;
 }

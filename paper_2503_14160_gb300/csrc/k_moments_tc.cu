@@ -25,6 +25,7 @@
 // turn one column of four elites each into digits in shared memory (K-major core matrices) while
 // the tensor cores work on the stage before, one thread issues the 68 MMAs of 128 x 64 x 16, and
 // the eight levels fill the 512 columns of tensor memory. Measured TC_MEASURED.
+#include "chain_launch.cuh"
 #include "cp_internal.cuh"
 #include "tcgen05.cuh"
 
@@ -311,11 +312,13 @@ __global__ void __launch_bounds__(256) k_moments_range(const MomentsTc a) { rang
 
 __global__ void __launch_bounds__(kTcThreads, 1) k_moments_tc(const MomentsTc a)
 {
+    after_previous();
     moments_tc_body(a, blockIdx.y, blockIdx.x, gridDim.x);
 }
 
 __global__ void __launch_bounds__(kCombGroups *kTcRows) k_moments_tc_combine(const MomentsTc a, int parts)
 {
+    after_previous();
     combine_tc_body(a, blockIdx.x, parts);
 }
 
@@ -394,9 +397,9 @@ int launch_moments_tc(const MomentsTc &a, int parts, int num_sms, cudaStream_t s
     const int rows = (a.nu + 15) / 16;
     k_moments_range<<<rows < 4 * num_sms ? rows : 4 * num_sms, 256, 0, st>>>(a);
     CP_LAUNCHED("k_moments_range");
-    k_moments_tc<<<dim3(parts, moments_tc_tiles(a.D)), kTcThreads, kTcSmem, st>>>(a);
+    launch_chained(k_moments_tc, dim3(parts, moments_tc_tiles(a.D)), kTcThreads, kTcSmem, st, a);
     CP_LAUNCHED("k_moments_tc");
-    k_moments_tc_combine<<<a.D, kCombGroups * kTcRows, 0, st>>>(a, parts);
+    launch_chained(k_moments_tc_combine, a.D, kCombGroups * kTcRows, 0, st, a, parts);
     CP_LAUNCHED("k_moments_tc_combine");
     return CP_OK;
 }

@@ -4,6 +4,7 @@
 //   k_sample  z_i from Philox4x32-10 (Salmon et al., SC'11) + Box-Muller, xi_i = mu + L z_i
 // The counter of candidate i, block j, iteration t, query q is (j, i, t, q); the key is
 // the 64-bit seed split into two words. Block j gives the normals z[4j..4j+3].
+#include "chain_launch.cuh"
 #include "cp_internal.cuh"
 #include "fp64_chain.cuh"
 #include "philox.cuh"
@@ -187,6 +188,7 @@ __global__ void __launch_bounds__(kSampleThreads)
 k_sample(const double *__restrict__ mu, const float *__restrict__ Lt, int N, int K,
          uint32_t k0, uint32_t k1, uint32_t iter, uint32_t query, float *xi)
 {
+    after_previous();
     extern __shared__ __align__(16) float sm[];
     const int per_block = kSampleWarps * kSampleCands;
     sample_body(mu, Lt, K, k0, k1, iter, query, xi, blockIdx.x * per_block, gridDim.x * per_block, N, sm);
@@ -270,8 +272,7 @@ int launch_sample(const double *mu, const float *Lt_f, int N, int K, uint64_t se
     if (per_sm < 1) per_sm = 1;
     int blocks = (N + kSampleWarps * kSampleCands - 1) / (kSampleWarps * kSampleCands);
     if (blocks > sms * per_sm) blocks = sms * per_sm;
-    k_sample<<<blocks, kSampleThreads, smem, st>>>(mu, Lt_f, N, K, (uint32_t)seed,
-                                                   (uint32_t)(seed >> 32), iter, query, xi);
+    launch_chained(k_sample, blocks, kSampleThreads, smem, st, mu, Lt_f, N, K, (uint32_t)seed, (uint32_t)(seed >> 32), iter, query, xi);
     CP_LAUNCHED("k_sample");
     return CP_OK;
 }

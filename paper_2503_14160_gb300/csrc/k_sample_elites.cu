@@ -26,6 +26,7 @@
 // normal nu + d.
 #include <algorithm>
 
+#include "chain_launch.cuh"
 #include "cp_internal.cuh"
 #include "philox.cuh"
 #include "tcgen05.cuh"
@@ -226,6 +227,7 @@ __global__ void __launch_bounds__(kTcThreads + 32)
 k_sample_elites(const float *__restrict__ Yp, int N, int D, int n_chunks, int slices, uint32_t tmem_cols,
                 const PhiloxKeys key, uint32_t iter, uint32_t query, float *P, uint32_t *status, int withhold)
 {
+    after_previous();
     extern __shared__ __align__(128) float smem[];
     __shared__ __align__(8) uint64_t a_full[kStages], b_full[kStages], done[kStages];
     __shared__ uint32_t s_tmem;
@@ -380,6 +382,7 @@ __global__ void k_sample_reduce(const float *__restrict__ P, int slices, const f
                                 int D, int nu, float eps_scale, const PhiloxKeys key, uint32_t iter,
                                 uint32_t query, float *xi)
 {
+    after_previous();
     const int D4 = D >> 2;
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (int64_t)N * D4) return;
@@ -503,13 +506,10 @@ int launch_sample_elites(const float *Yp, const float *mu_f, int N, int K, int n
     if (slices > chunks) slices = chunks;
     const PhiloxKeys key = philox_keys((uint32_t)seed, (uint32_t)(seed >> 32));
     dim3 grid((N + kTcM - 1) / kTcM, slices);
-    k_sample_elites<<<grid, kTcThreads + 32, tc_smem_bytes(Dp), st>>>(Yp, N, D, chunks, slices, tmem_columns(Dp), key,
-                                                                  iter, query, P, status, withhold ? 1 : 0);
+    launch_chained(k_sample_elites, grid, kTcThreads + 32, tc_smem_bytes(Dp), st, Yp, N, D, chunks, slices, tmem_columns(Dp), key, iter, query, P, status, withhold ? 1 : 0);
     CP_LAUNCHED("k_sample_elites");
     const int64_t total = (int64_t)N * (D / 4);
-    k_sample_reduce<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(P, slices, mu_f, N, D, nu,
-                                                                     (float)(sigma * sqrt(eps)), key, iter,
-                                                                     query, xi);
+    launch_chained(k_sample_reduce, (unsigned)((total + 255) / 256), 256, 0, st, P, slices, mu_f, N, D, nu, (float)(sigma * sqrt(eps)), key, iter, query, xi);
     CP_LAUNCHED("k_sample_reduce");
     return CP_OK;
 }

@@ -10,6 +10,9 @@
 //                    C = sum_j w_j (xi_(j) - mu)(xi_(j) - mu)^T + eps I (about the new
 //                    mean) in one FP64 pass about the best elite, 16x16 output tiles x
 //                    chunks of elites, chunk partials summed in a fixed order (deterministic)
+#include <cmath>
+
+#include "chain_launch.cuh"
 #include "cp_internal.cuh"
 
 namespace cp {
@@ -52,6 +55,7 @@ __global__ void k_weights(int nu, double *w)
 __global__ void __launch_bounds__(kRankThreads)
 k_rank_count(const double *__restrict__ J, int N, int *rank)
 {
+    after_previous();
     __shared__ unsigned long long s_key[kRankPer];
     const int i = blockIdx.x * kRankThreads + threadIdx.x;
     const unsigned long long ki = i < N ? order_key(J[i]) : 0ull;
@@ -75,6 +79,7 @@ __global__ void k_scatter(int *__restrict__ rank, const double *__restrict__ J,
                           const float *__restrict__ xi, int N, int nu, int D, int *elite,
                           float *elites, double *best_J)
 {
+    after_previous();
     const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (warp >= N) return;
@@ -167,6 +172,7 @@ __device__ __forceinline__ void moments_prep_body(const float *__restrict__ elit
 __global__ void k_moments_prep(const float *__restrict__ elites, const double *__restrict__ w, int nu, int D,
                                double *Y, double *WY)
 {
+    after_previous();
     moments_prep_body(elites, w, nu, D, Y, WY, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
@@ -174,6 +180,7 @@ __global__ void __launch_bounds__(256)
 k_moments_partial(const double *__restrict__ Y, const double *__restrict__ WY, int nu, int D,
                   int per, int n_chunks, double *s2p, double *s1p)
 {
+    after_previous();
     moments_partial_body(Y, WY, nu, D, per, n_chunks, s2p, s1p, blockIdx.x, blockIdx.y);
 }
 
@@ -206,26 +213,34 @@ k_batch_moments_partial(const BatchQueryDev *__restrict__ qd, const int2 *__rest
 // (P = 32 / G), the pairings across lanes go through xor shuffles within the group and the
 // rest inside the lane, so the additions are the same and so are the bits. Every lane of the
 // warp calls it (full-warp shuffles); the total is returned on every lane of the group.
+// An FP64 addition holds its unit for some 70 cycles, so those of a zero that no term has reached
+// are left out: the first term is taken as it is, and a level that pairs sums l < n with sums
+// l + off >= n does nothing (few chunks: the smallest query has four, and three additions).
 template <int G>
 __device__ __forceinline__ double tree_sum(const double *__restrict__ v, int n, size_t stride, int sub)
 {
     constexpr int P = 32 / G;
     double s[P];
-#pragma unroll
-    for (int i = 0; i < P; ++i) s[i] = 0.0;
     const int l0 = sub * P;
-    for (int q0 = 0; q0 < n; q0 += 32) {
+#pragma unroll
+    for (int i = 0; i < P; ++i) s[i] = l0 + i < n ? v[(size_t)(l0 + i) * stride] : 0.0;
+    for (int q0 = 32; q0 < n; q0 += 32) {
+        double t[P];
+#pragma unroll
+        for (int i = 0; i < P; ++i) t[i] = q0 + l0 + i < n ? v[(size_t)(q0 + l0 + i) * stride] : 0.0;
 #pragma unroll
         for (int i = 0; i < P; ++i)
-            if (q0 + l0 + i < n) s[i] += v[(size_t)(q0 + l0 + i) * stride];
+            if (q0 + l0 + i < n) s[i] += t[i];
     }
 #pragma unroll
     for (int off = 16; off >= P; off >>= 1) {   // partner lane sub + off / P holds sums l + off
+        if (n <= off) continue;
 #pragma unroll
         for (int i = 0; i < P; ++i) s[i] += __shfl_xor_sync(0xffffffffu, s[i], off / P);
     }
 #pragma unroll
     for (int off = P / 2; off > 0; off >>= 1) {
+        if (n <= off) continue;
 #pragma unroll
         for (int i = 0; i < off; ++i) s[i] += s[i + off];
     }
@@ -235,20 +250,18 @@ __device__ __forceinline__ double tree_sum(const double *__restrict__ v, int n, 
 // Lanes per sum of the moment combine: four lanes, eight running sums each.
 constexpr int kSumLanes = 4;
 
-// S1 of rows 0 .. r_last into shared memory (one thread per row), for the entries of a block.
+// S1 of rows 0 .. r_last into shared memory (kSumLanes lanes per row), for the entries of a block
+// of whole warps.
 __device__ __forceinline__ void stage_s1(const double *__restrict__ s1p, int n_chunks, int D, int r_last,
                                          double *s_s1)
 {
-    for (int r = threadIdx.x; r <= r_last && r < D; r += blockDim.x) s_s1[r] = tree_sum<1>(s1p + r, n_chunks, D, 0);
+    const int per = (int)blockDim.x / kSumLanes, sub = (int)threadIdx.x % kSumLanes;
+    for (int r0 = 0; r0 <= r_last; r0 += per) {
+        const int r = r0 + (int)threadIdx.x / kSumLanes;
+        const double s = tree_sum<kSumLanes>(s1p + min(r, D - 1), n_chunks, D, sub);
+        if (r < D && sub == 0) s_s1[r] = s;
+    }
     __syncthreads();
-}
-
-// Row of the last lower-triangle entry a block of blockDim.x threads starting at entry e0 holds.
-__device__ __forceinline__ int last_row(int e0, int D)
-{
-    int r, c;
-    tri_index(min(e0 + (int)blockDim.x, D * (D + 1) / 2) - 1, r, c);
-    return r;
 }
 
 // S1 of row r (its chunk partials summed in the fixed order above, kSumLanes lanes per row),
@@ -284,6 +297,7 @@ __device__ __forceinline__ void moments_combine_body(const double *__restrict__ 
 __global__ void __launch_bounds__(128)
 k_moments_s1(double *s1p, int n_chunks, int D, const float *__restrict__ elites, double *mu)
 {
+    after_previous();
     const int g = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     moments_s1_body(s1p, n_chunks, D, elites, mu, g / kSumLanes, g % kSumLanes);
 }
@@ -292,6 +306,7 @@ __global__ void __launch_bounds__(128)
 k_moments_combine(const double *__restrict__ s2p, const double *__restrict__ s1, int n_chunks, int D, double eps,
                   double *C)
 {
+    after_previous();
     const int g = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     moments_combine_body(s2p, s1, n_chunks, D, eps, C, g / kSumLanes, g % kSumLanes);
 }
@@ -465,6 +480,7 @@ k_radix_pass(const unsigned long long *__restrict__ key_in, const int *__restric
              const int *__restrict__ hist, unsigned long long *key_out, int *val_out, int next_shift, int *hist_next,
              const uint16_t *__restrict__ qid)
 {
+    after_previous();
     __shared__ int s_before[4][256], s_total[4][256];
     __shared__ int wcount[kRadixTile / 32][256];   // per-warp digit counts, then first places
     __shared__ int warp_tot[8];
@@ -550,6 +566,7 @@ __global__ void k_gather_elites(const int *__restrict__ sorted, const double *__
                                 const float *__restrict__ xi, int nu, int D, int *elite,
                                 float *elites, double *best_J)
 {
+    after_previous();
     gather_body(sorted, 0, J, xi, nu, D, elite, elites, best_J, (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5));
 }
 
@@ -604,19 +621,23 @@ __global__ void k_cma_reset(double sigma0, int D, double *cma, double *p_sigma, 
 // One CTA: the new mean m' = x_(1) + S1, the mean shift m' - m, z = L^-1 (m' - m) by forward
 // substitution with the current factor L (L L^T = sigma^2 C, so z = L_C^-1 (m' - m) / sigma
 // with L_C the Cholesky factor of C), the step-size path and its length, h_sigma, the
-// covariance path, and sigma'. L is staged in shared memory (row stride D + 1); warp 0
+// covariance path, and sigma'. path_len and path_max: the two sides' factors of the test
+// |p_sigma| / sqrt(1 - (1 - c_sigma)^(2 (t + 1))) < (1.4 + 2 / (D + 1)) chi_n, functions of the
+// iteration alone. L is staged in shared memory (row stride D + 1); warp 0
 // runs the substitution column by column, lane l holding rows l, l + 32, l + 64, l + 96,
 // each new z_j passed by a shuffle, so the dependent chain has no block barrier.
 __global__ void __launch_bounds__(kCmaThreads)
 k_cma_paths(const double *__restrict__ s1p, int n_chunks, int D, const float *__restrict__ elites,
-            const double *__restrict__ mu_prev, const double *__restrict__ L, CmaConsts k, int t,
+            double *__restrict__ mu_prev, const double *__restrict__ L, CmaConsts k, double path_len, double path_max,
             double *mu, double *p_sigma, double *p_c, double *cma)
 {
+    after_previous();
     extern __shared__ double s_L[];   // [D][D + 1]
-    __shared__ double s_b[kCmaThreads];
+    __shared__ double s_b[kCmaThreads], s_rinv[kCmaThreads];
     __shared__ double s_red[kCmaThreads / 32];
     const int r = threadIdx.x, lane = r & 31;
     const int ld = D + 1;
+#pragma unroll 4
     for (int idx = r; idx < D * D; idx += kCmaThreads) {
         const int i = idx / D, j = idx - i * D;
         if (j <= i) s_L[i * ld + j] = L[idx];
@@ -624,12 +645,16 @@ k_cma_paths(const double *__restrict__ s1p, int n_chunks, int D, const float *__
     double shift = 0.0;
     if (r < D) {
         double s1 = 0.0;
+#pragma unroll 8
         for (int c = 0; c < n_chunks; ++c) s1 += s1p[(size_t)c * D + r];
-        const double m_new = (double)elites[r] + s1;
-        shift = m_new - mu_prev[r];
+        const double m_new = (double)elites[r] + s1, m_old = mu[r];
+        shift = m_new - m_old;
+        mu_prev[r] = m_old;
         mu[r] = m_new;
         s_b[r] = shift;
     }
+    __syncthreads();
+    if (r < D) s_rinv[r] = 1.0 / s_L[r * ld + r];   // one division per lane, on the warps of all schedulers
     __syncthreads();
     if (r < 32) {
         double b[4], rinv[4];
@@ -637,7 +662,7 @@ k_cma_paths(const double *__restrict__ s1p, int n_chunks, int D, const float *__
         for (int i = 0; i < 4; ++i) {
             const int row = lane + 32 * i;
             b[i] = row < D ? s_b[row] : 0.0;
-            rinv[i] = row < D ? 1.0 / s_L[row * ld + row] : 0.0;
+            rinv[i] = row < D ? s_rinv[row] : 0.0;
         }
 #pragma unroll
         for (int slot = 0; slot < 4; ++slot) {
@@ -670,8 +695,7 @@ k_cma_paths(const double *__restrict__ s1p, int n_chunks, int D, const float *__
     double n2 = 0.0;
     for (int w = 0; w < kCmaThreads / 32; ++w) n2 += s_red[w];
     const double norm = sqrt(n2);
-    const double h = norm / sqrt(1.0 - pow(1.0 - k.c_sigma, 2.0 * (t + 1)))
-                     < (1.4 + 2.0 / (D + 1)) * k.chi_n ? 1.0 : 0.0;
+    const double h = norm / path_len < path_max ? 1.0 : 0.0;
     if (r < D) p_c[r] = fma(1.0 - k.c_c, p_c[r], h * sqrt(k.c_c * (2.0 - k.c_c) * k.mu_eff) * (shift / sigma));
     if (r == 0) {
         cma[1] = sigma;
@@ -681,23 +705,25 @@ k_cma_paths(const double *__restrict__ s1p, int n_chunks, int D, const float *__
     }
 }
 
-// One thread per lower-triangle entry: the elites' weighted scatter about the OLD mean m from
+// kSumLanes lanes per lower-triangle entry: the elites' weighted scatter about the OLD mean m from
 // the moments about x_(1) (with d = x_(1) - m and weights summing to one:
 // S2 + S1 d^T + d S1^T + d d^T), then C' = a C + c_1 p_c p_c^T + c_mu scatter / sigma^2 with
 // a = 1 + c_1 (1 - h_sigma) c_c (2 - c_c) - c_1 - c_mu.
-__global__ void __launch_bounds__(256) k_cma_cov(const double *__restrict__ s2p, const double *__restrict__ s1p, int n_chunks,
+__global__ void __launch_bounds__(128) k_cma_cov(const double *__restrict__ s2p, const double *__restrict__ s1p, int n_chunks,
                           int D, const float *__restrict__ elites, const double *__restrict__ mu_prev,
                           const double *__restrict__ p_c, const double *__restrict__ cma, CmaConsts k,
                           double *C)
 {
+    after_previous();
     __shared__ double s_s1[4 * CP_MAX_WAYPOINTS];
-    const int e0 = (int)(blockIdx.x * blockDim.x);
-    stage_s1(s1p, n_chunks, D, last_row(e0, D), s_s1);
-    const int e = e0 + (int)threadIdx.x;
-    if (e >= D * (D + 1) / 2) return;
+    const int entries = D * (D + 1) / 2, sub = (int)threadIdx.x % kSumLanes;
+    const int e = ((int)(blockIdx.x * blockDim.x) + (int)threadIdx.x) / kSumLanes;
     int r, c;
-    tri_index(e, r, c);
-    const double s2 = tree_sum<1>(s2p + (size_t)r * D + c, n_chunks, (size_t)D * D, 0);
+    tri_index(min((int)((blockIdx.x + 1) * blockDim.x) / kSumLanes, entries) - 1, r, c);
+    stage_s1(s1p, n_chunks, D, r, s_s1);
+    tri_index(min(e, entries - 1), r, c);
+    const double s2 = tree_sum<kSumLanes>(s2p + (size_t)r * D + c, n_chunks, (size_t)D * D, sub);
+    if (e >= entries || sub != 0) return;
     const double sr = s_s1[r], sc = s_s1[c];
     const double dr = (double)elites[r] - mu_prev[r], dc = (double)elites[c] - mu_prev[c];
     const double scatter = fma(dr, dc, fma(dr, sc, fma(sr, dc, s2)));
@@ -732,7 +758,7 @@ static int radix_passes(int N, int q_passes, const uint16_t *qid, unsigned long 
         const int shift = byq ? 8 * (p - 8) : 8 * p, next_shift = next_byq ? 8 * (p + 1 - 8) : 8 * (p + 1);
         int *now = hist + (size_t)p * 256 * tiles, *next = p + 1 < passes ? now + 256 * tiles : nullptr;
         auto kern = byq ? k_radix_pass<true, true> : (next_byq ? k_radix_pass<false, true> : k_radix_pass<false, false>);
-        kern<<<tiles, kRadixTile, 0, st>>>(key_a, val_a, N, shift, now, key_b, val_b, next_shift, next, qid);
+        launch_chained(kern, tiles, kRadixTile, 0, st, key_a, val_a, N, shift, now, key_b, val_b, next_shift, next, qid);
         CP_LAUNCHED("k_radix_pass");
         unsigned long long *tk = key_a;
         key_a = key_b;
@@ -784,8 +810,7 @@ int launch_gather_elites(const int *sorted, const double *J, const float *xi, in
                          int *elite, float *elites, double *best_J, cudaStream_t st)
 {
     const int threads = 256;
-    k_gather_elites<<<(nu * 32 + threads - 1) / threads, threads, 0, st>>>(sorted, J, xi, nu, D, elite,
-                                                                          elites, best_J);
+    launch_chained(k_gather_elites, (nu * 32 + threads - 1) / threads, threads, 0, st, sorted, J, xi, nu, D, elite, elites, best_J);
     CP_LAUNCHED("k_gather_elites");
     return CP_OK;
 }
@@ -829,7 +854,7 @@ int launch_weights(int nu, double *w, cudaStream_t st)
 int launch_rank(const double *J, int N, int nu, int *rank, cudaStream_t st)
 {
     dim3 grid((N + kRankThreads - 1) / kRankThreads, (N + kRankPer - 1) / kRankPer);
-    k_rank_count<<<grid, kRankThreads, 0, st>>>(J, N, rank);
+    launch_chained(k_rank_count, grid, kRankThreads, 0, st, J, N, rank);
     CP_LAUNCHED("k_rank_count");
     (void)nu;
     return CP_OK;
@@ -840,7 +865,7 @@ int launch_scatter(int *rank, const double *J, const float *xi, int N, int nu, i
 {
     const int threads = 256;
     const int blocks = (N * 32 + threads - 1) / threads;
-    k_scatter<<<blocks, threads, 0, st>>>(rank, J, xi, N, nu, D, elite, elites, best_J);
+    launch_chained(k_scatter, blocks, threads, 0, st, rank, J, xi, N, nu, D, elite, elites, best_J);
     CP_LAUNCHED("k_scatter");
     return CP_OK;
 }
@@ -852,7 +877,7 @@ int launch_cma_reset(double sigma0, int D, double *cma, double *p_sigma, double 
     return CP_OK;
 }
 
-// CMA-ES update: mu_prev must hold the mean before the update; mu, C, p_sigma, p_c and cma
+// CMA-ES update: mu_prev receives the mean before the update; mu, C, p_sigma, p_c and cma
 // are updated in place (L is the factor of sigma^2 C before the update).
 static int launch_moments_partial(const float *elites, const double *w, int nu, int D, double *yw, double *s2p,
                                   double *s1p, int *n_chunks_out, cudaStream_t st)
@@ -861,16 +886,16 @@ static int launch_moments_partial(const float *elites, const double *w, int nu, 
     const int n_chunks = (nu + per - 1) / per;
     const int tiles = (D + 15) / 16;
     double *Y = yw, *WY = yw + (size_t)nu * D;
-    k_moments_prep<<<(nu * D + 255) / 256, 256, 0, st>>>(elites, w, nu, D, Y, WY);
+    launch_chained(k_moments_prep, (nu * D + 255) / 256, 256, 0, st, elites, w, nu, D, Y, WY);
     CP_LAUNCHED("k_moments_prep");
     dim3 grid(tiles * (tiles + 1) / 2, n_chunks);
-    k_moments_partial<<<grid, 256, 0, st>>>(Y, WY, nu, D, per, n_chunks, s2p, s1p);
+    launch_chained(k_moments_partial, grid, 256, 0, st, Y, WY, nu, D, per, n_chunks, s2p, s1p);
     CP_LAUNCHED("k_moments_partial");
     *n_chunks_out = n_chunks;
     return CP_OK;
 }
 
-int launch_cma_update(const float *elites, const double *w, int nu, int D, const double *mu_prev,
+int launch_cma_update(const float *elites, const double *w, int nu, int D, double *mu_prev,
                       const double *L, const CmaConsts &k, int t, double *yw, double *s2p, double *s1p, double *mu,
                       double *C, double *p_sigma, double *p_c, double *cma, cudaStream_t st)
 {
@@ -878,10 +903,11 @@ int launch_cma_update(const float *elites, const double *w, int nu, int D, const
     int rc = launch_moments_partial(elites, w, nu, D, yw, s2p, s1p, &n_chunks, st);
     if (rc != CP_OK) return rc;
     const size_t smem = sizeof(double) * (size_t)D * (D + 1);
-    k_cma_paths<<<1, kCmaThreads, smem, st>>>(s1p, n_chunks, D, elites, mu_prev, L, k, t, mu, p_sigma, p_c, cma);
+    launch_chained(k_cma_paths, 1, kCmaThreads, smem, st, s1p, n_chunks, D, elites, mu_prev, L, k, std::sqrt(1.0 - std::pow(1.0 - k.c_sigma, 2.0 * (t + 1))),
+                   (1.4 + 2.0 / (D + 1)) * k.chi_n, mu, p_sigma, p_c, cma);
     CP_LAUNCHED("k_cma_paths");
     const int entries = D * (D + 1) / 2;
-    k_cma_cov<<<(entries + 255) / 256, 256, 0, st>>>(s2p, s1p, n_chunks, D, elites, mu_prev, p_c, cma, k, C);
+    launch_chained(k_cma_cov, (entries * kSumLanes + 127) / 128, 128, 0, st, s2p, s1p, n_chunks, D, elites, mu_prev, p_c, cma, k, C);
     CP_LAUNCHED("k_cma_cov");
     return CP_OK;
 }
@@ -977,9 +1003,9 @@ int launch_moments(const float *elites, const double *w, int nu, int D, double e
     int rc = launch_moments_partial(elites, w, nu, D, yw, s2p, s1p, &n_chunks, st);
     if (rc != CP_OK) return rc;
     const int entries = D * (D + 1) / 2;
-    k_moments_s1<<<(D + 31) / 32, 128, 0, st>>>(s1p, n_chunks, D, elites, mu);
+    launch_chained(k_moments_s1, (D + 31) / 32, 128, 0, st, s1p, n_chunks, D, elites, mu);
     CP_LAUNCHED("k_moments_s1");
-    k_moments_combine<<<(entries + 31) / 32, 128, 0, st>>>(s2p, s1p + (size_t)n_chunks * D, n_chunks, D, eps, C);
+    launch_chained(k_moments_combine, (entries + 31) / 32, 128, 0, st, s2p, s1p + (size_t)n_chunks * D, n_chunks, D, eps, C);
     CP_LAUNCHED("k_moments_combine");
     return CP_OK;
 }
