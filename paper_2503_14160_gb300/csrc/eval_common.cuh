@@ -114,27 +114,122 @@ static __device__ __forceinline__ void crane_place(const ModelDev &m, float q4s,
     }
 }
 
-// Sphere centres at configuration q (chain of Sec. 2 in the linear placement form), in
-// polar form: every centre is (c1 h, s1 h, z) with (c1, s1) the cosine and sine of the slew
-// angle and h the signed horizontal distance from the slew axis.
+// Sines and cosines of the chain: slew, boom elevation, jib elevation (q2 + q3).
 // kFastTrig: the reduced hardware sine and cosine above (the evaluation forms, which must all
 // agree bit for bit); otherwise the accurate library sincosf (the forward-kinematics entry
 // point and the smooth cost, whose softplus penalty is checked to 1e-4 relative).
+struct ChainTrig {
+    float s1, c1, s2, c2, s23, c23;
+};
+
+template <bool kFastTrig = true>
+static __device__ __forceinline__ ChainTrig chain_trig(float4 q)
+{
+    ChainTrig t;
+    if (kFastTrig) {
+        sincos_reduced(q.x, &t.s1, &t.c1);
+        sincos_reduced(q.y, &t.s2, &t.c2);
+        sincos_reduced(q.y + q.z, &t.s23, &t.c23);
+    } else {
+        sincosf(q.x, &t.s1, &t.c1);
+        sincosf(q.y, &t.s2, &t.c2);
+        sincosf(q.y + q.z, &t.s23, &t.c23);
+    }
+    return t;
+}
+
+// Sphere centres at configuration q (chain of Sec. 2 in the linear placement form), in
+// polar form: every centre is (c1 h, s1 h, z) with (c1, s1) the cosine and sine of the slew
+// angle and h the signed horizontal distance from the slew axis.
 template <int NSPH, bool kFastTrig = true>
 static __device__ __forceinline__ void crane_fk_polar(const ModelDev &m, float4 q, float *h, float *z,
                                                float &s1, float &c1)
 {
-    float s2, c2, s23, c23;
-    if (kFastTrig) {
-        sincos_reduced(q.x, &s1, &c1);
-        sincos_reduced(q.y, &s2, &c2);
-        sincos_reduced(q.y + q.z, &s23, &c23);
-    } else {
-        sincosf(q.x, &s1, &c1);
-        sincosf(q.y, &s2, &c2);
-        sincosf(q.y + q.z, &s23, &c23);
+    const ChainTrig t = chain_trig<kFastTrig>(q);
+    s1 = t.s1;
+    c1 = t.c1;
+    crane_place<NSPH>(m, q.w, t.s2, t.c2, t.s23, t.c23, h, z);
+}
+
+// The placement of each sphere in shared memory, {alpha, beta, gamma, -delta} and its radius, for
+// code that takes the spheres a lane needs one by one: the lanes of a warp then read different
+// entries, where arrays in registers would have every lane go through all of them.
+template <int NSPH>
+struct SphereTable {
+    float4 place[NSPH];
+    float radius[NSPH];
+
+    __device__ __forceinline__ void fill(const ModelDev &m)   // the block syncs afterwards
+    {
+        if (threadIdx.x < NSPH) {
+            const SphereLin t = m.sph[threadIdx.x];
+            place[threadIdx.x] = make_float4(t.alpha, t.beta, t.gamma, -t.delta);
+            radius[threadIdx.x] = t.radius;
+        }
     }
-    crane_place<NSPH>(m, q.w, s2, c2, s23, c23, h, z);
+};
+
+// L = gamma q4 + beta, h and z of the sphere placed by t, by the operations of crane_place (the
+// same bits).
+static __device__ __forceinline__ void place_sphere(const ChainTrig &g, float base_z, float q4, float4 t, float &L,
+                                                    float &h, float &z)
+{
+    L = fmaf(t.z, q4, t.y);
+    h = fmaf(t.x, g.c2, __fmul_rn(L, g.c23));
+    z = base_z + fmaf(t.x, g.s2, fmaf(L, g.s23, t.w));
+}
+
+// The spheres whose packed filter value is below zero (its sign bit is set), sphere s in bit s.
+template <int NSPH>
+static __device__ __forceinline__ uint32_t sign_mask(const float2 *t)
+{
+    uint32_t in = 0u;
+#pragma unroll
+    for (int p = NSPH / 2 - 1; p >= 0; --p) {
+        in = __funnelshift_l(__float_as_uint(t[p].y), in, 1);
+        in = __funnelshift_l(__float_as_uint(t[p].x), in, 1);
+    }
+    return in;
+}
+
+// The smallest exact distance of the spheres in `in` to the cylinder at (cx, cy) with record e
+// (only those within its height range widened by r_max and the gate), or to a box; +inf when there
+// is none. A lane has one or two spheres in reach of an obstacle, and not the ones its neighbours
+// have: walking its own takes as many steps as the lane with the most, where the unrolled form
+// went through all twelve (one distance each as soon as any lane needs it). The centre is taken
+// from rounded products, as every form takes it. Measured on plans and batches from the initial
+// distribution, where contacts are frequent: dense forest 95.1 -> 87.1 ms per 20 iterations, 16
+// batched queries 96.1 -> 80.0 ms, 3001 candidates among 300 trees and 10 boxes 100 -> 80 us.
+template <int NSPH>
+static __device__ __forceinline__ float walk_cylinder(const SphereTable<NSPH> &tab, const ChainTrig &g, float base_z,
+                                                      float q4, float r_max, uint32_t in, float cx, float cy, float4 e)
+{
+    float d = CUDART_INF_F;
+    const float zlo = e.y - r_max - kZGate, zhi = e.z + r_max + kZGate;
+    while (in != 0u) {
+        const int s = __ffs(in) - 1;
+        in &= in - 1;
+        float L, h, z;
+        place_sphere(g, base_z, q4, tab.place[s], L, h, z);
+        if (z > zlo && z < zhi)
+            d = fminf(d, sdf_cylinder(__fmul_rn(g.c1, h), __fmul_rn(g.s1, h), z, cx, cy, e) - tab.radius[s]);
+    }
+    return d;
+}
+
+template <int NSPH>
+static __device__ __forceinline__ float walk_box(const SphereTable<NSPH> &tab, const ChainTrig &g, float base_z,
+                                                 float q4, uint32_t in, float4 bc, float4 bh)
+{
+    float d = CUDART_INF_F;
+    while (in != 0u) {
+        const int s = __ffs(in) - 1;
+        in &= in - 1;
+        float L, h, z;
+        place_sphere(g, base_z, q4, tab.place[s], L, h, z);
+        d = fminf(d, sdf_box(__fmul_rn(g.c1, h), __fmul_rn(g.s1, h), z, bc, bh) - tab.radius[s]);
+    }
+    return d;
 }
 
 // The same centres in Cartesian form, x = c1 h and y = s1 h.

@@ -115,42 +115,18 @@ __device__ __forceinline__ float exact_cylinders(const ModelDev &m, const float 
     return d;
 }
 
-// Exact distance of every sphere whose polar filter passes against one cylinder: with the
-// obstacle centre at p along the lane's plane and q across it, sphere s passes when
-// (h_s - p)^2 < (R + r_max)^2 + margin - q^2 = rhs and its centre is within the cylinder's
-// height range widened by r_max and the gate. The distance itself is taken from the
-// Cartesian centre (c1 h, s1 h, z), rounded products (no contraction into the distance's
-// differences), the same values the exhaustive form uses.
+// The spheres of one lane in reach of a surviving obstacle whose centre is (cx, cy): with the
+// centre at p along the lane's plane and q across it, sphere s passes when (h_s - p)^2 < bound -
+// q^2 (two packed FP32x2 operations per sphere pair, H2 holding the in-band h and 1e30 for the
+// others). bound: (R + r_max)^2 + margin of a cylinder, the square of a box's reach (its half
+// diagonal, r_max and 1 cm).
 template <int NSPH>
-__device__ __forceinline__ float exact_polar(const ModelDev &m, const float *H, const float *Z,
-                                             float c1, float s1, float p, float rhs, float4 f,
-                                             float4 e)
+__device__ __forceinline__ uint32_t spheres_in_reach(const float2 *H2, float c1, float s1, float cx, float cy,
+                                                     float bound)
 {
-    float d = CUDART_INF_F;
-    const float zlo = e.y - m.r_max - kZGate, zhi = e.z + m.r_max + kZGate;
-#pragma unroll
-    for (int s = 0; s < NSPH; ++s) {
-        const float dh = H[s] - p;
-        if (fmaf(dh, dh, -rhs) < 0.f && Z[s] > zlo && Z[s] < zhi)
-            d = fminf(d, sdf_cylinder(__fmul_rn(c1, H[s]), __fmul_rn(s1, H[s]), Z[s], f.x, f.y, e) -
-                             m.sph[s].radius);
-    }
-    return d;
-}
-
-// A surviving cylinder (filter record f = {cx, cy, W, reach}, exact record e = {R, z_lo,
-// z_hi, (R + r_max)^2 + margin}) against the unit's spheres at one lane: its centre at p
-// along the lane's plane and q across it; sphere s passes the polar filter when
-// (h_s - p)^2 < e.w - q^2 (two packed FP32x2 operations per sphere pair, H2 holding the
-// in-band h and 1e30 for the others), and the passing spheres take the exact distance.
-template <int NSPH>
-__device__ __forceinline__ float survivor_cylinder(const ModelDev &m, const float *H, const float *Z,
-                                                   const float2 *H2, float c1, float s1, float4 f, float4 e,
-                                                   const float *zero)
-{
-    const float p = fmaf(c1, f.x, s1 * f.y);
-    const float q = fmaf(c1, f.y, -(s1 * f.x));
-    const float rhs = fmaf(-q, q, e.w);
+    const float p = fmaf(c1, cx, s1 * cy);
+    const float q = fmaf(c1, cy, -(s1 * cx));
+    const float rhs = fmaf(-q, q, bound);
     const float2 mp2 = make_float2(-p, -p), mr2 = make_float2(-rhs, -rhs);
     float2 t[NSPH / 2];
 #pragma unroll
@@ -158,27 +134,14 @@ __device__ __forceinline__ float survivor_cylinder(const ModelDev &m, const floa
         const float2 dh = __fadd2_rn(H2[k], mp2);
         t[k] = __ffma2_rn(dh, dh, mr2);
     }
-    return any_negative<NSPH>(t) ? exact_polar<NSPH>(m, H, Z, c1, s1, p, rhs, f, e) : CUDART_INF_F;
-}
-
-// A surviving box (centre c, half extent hb) against every sphere of the lane.
-template <int NSPH>
-__device__ __forceinline__ float survivor_box(const ModelDev &m, const float *H, const float *Z, float c1,
-                                              float s1, float4 c, float4 hb)
-{
-    float d = CUDART_INF_F;
-#pragma unroll
-    for (int s = 0; s < NSPH; ++s)
-        d = fminf(d, sdf_box(__fmul_rn(c1, H[s]), __fmul_rn(s1, H[s]), Z[s], c, hb) - m.sph[s].radius);
-    return d;
+    return any_negative<NSPH>(t) ? sign_mask<NSPH>(t) : 0u;
 }
 
 // The evaluation with the broad phase (the default form). Per unit: the checkpoints and
 // the kinematics in polar form, the unit box, then rounds of 32 obstacles: each lane tests
 // one obstacle against the box, and the warp takes the survivors one by one (a uniform
 // loop) through the per-sphere polar filter, two packed FP32x2 operations per sphere pair,
-// and the exact distance where it passes. Boxes take the same broad phase and then the
-// exact distance for every sphere. Its distances are those of the exhaustive form for
+// and the exact distance of the spheres that pass (walk_cylinder, walk_box). Its distances are those of the exhaustive form for
 // every pair that can be in contact, so both forms give the same results bit for bit.
 template <int NSPH>
 __global__ void __launch_bounds__(kEvalThreads, kEvalBroadMinBlocks)
@@ -194,14 +157,15 @@ k_eval_broad(const ModelDev m, const SceneDev sc, const EvalArgs a)
     float4 *s_group = s_basis + 2 * a.S;
     float4 *s_ctrl = s_group + n_groups(sc.n_cyl) + (threadIdx.x >> 5) * kCtrlSlots;
     __shared__ __align__(8) uint64_t staging_bar;
-    if (!stage_bulk(&staging_bar, s_filt, s_exact, s_bc, s_bh, s_basis, s_group, sc, a)) return;
+    __shared__ SphereTable<NSPH> s_tab;
+    s_tab.fill(m);
+    if (!stage_bulk(&staging_bar, s_filt, s_exact, s_bc, s_bh, s_basis, s_group, sc, a)) return;   // syncs
 
     const int lane = threadIdx.x & 31;
     const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int n_warps = (int)((gridDim.x * blockDim.x) >> 5);
     const int items = a.n * a.P;
     uint32_t tested = 0;   // broad-phase survivors of this warp's units
-    const float zero[NSPH] = {};
     const float zlo = sc.z_lo_all - m.r_max - kZGate, zhi = sc.z_hi_all + m.r_max + kZGate;
 
     for (int it = queue_first(a, warp, lane); it < items; it = queue_next(a, it, n_warps, lane)) {
@@ -211,17 +175,22 @@ k_eval_broad(const ModelDev m, const SceneDev sc, const EvalArgs a)
         uint32_t count = 0;
         for (int chunk = ir.c0; chunk < ir.c1; ++chunk) {
             const Checkpoint c = checkpoint_at(m, a, s_basis, s_ctrl, chunk, lane);
-            float H[NSPH], Z[NSPH], s1, c1;
-            crane_fk_polar<NSPH>(m, c.q, H, Z, s1, c1);
+            const ChainTrig tr = chain_trig(c.q);
+            const float s1 = tr.s1, c1 = tr.c1;
             // Spheres above or below every obstacle by more than r_max (the vertical gate over
             // the whole scene) can penetrate nothing: they leave the unit box, and their packed
             // h is pushed far away so that no polar filter passes them.
-            const UnitFrame fr = unit_frame_band<NSPH>(s1, c1, H, Z, zlo, zhi);
+            UnitFrame fr;
             float2 H2[NSPH / 2];
+            {
+                float H[NSPH], Z[NSPH];
+                crane_place<NSPH>(m, c.q.w, tr.s2, tr.c2, tr.s23, tr.c23, H, Z);
+                fr = unit_frame_band<NSPH>(s1, c1, H, Z, zlo, zhi);
 #pragma unroll
-            for (int q = 0; q < NSPH / 2; ++q)
-                H2[q] = make_float2(Z[2 * q] > zlo && Z[2 * q] < zhi ? H[2 * q] : 1e30f,
-                                    Z[2 * q + 1] > zlo && Z[2 * q + 1] < zhi ? H[2 * q + 1] : 1e30f);
+                for (int q = 0; q < NSPH / 2; ++q)
+                    H2[q] = make_float2(Z[2 * q] > zlo && Z[2 * q] < zhi ? H[2 * q] : 1e30f,
+                                        Z[2 * q + 1] > zlo && Z[2 * q + 1] < zhi ? H[2 * q + 1] : 1e30f);
+            }
 
             float dmin = CUDART_INF_F;
             const int n_grp = n_groups(sc.n_cyl);
@@ -243,7 +212,9 @@ k_eval_broad(const ModelDev m, const SceneDev sc, const EvalArgs a)
                     while (mask) {
                         const int ob = __shfl_sync(0xffffffffu, o, __ffs(mask) - 1);
                         mask &= mask - 1;
-                        dmin = fminf(dmin, survivor_cylinder<NSPH>(m, H, Z, H2, c1, s1, s_filt[ob], s_exact[ob], zero));
+                        const float4 f = s_filt[ob], e = s_exact[ob];
+                        const uint32_t in = spheres_in_reach<NSPH>(H2, c1, s1, f.x, f.y, e.w);
+                        if (in) dmin = fminf(dmin, walk_cylinder<NSPH>(s_tab, tr, m.base_z, c.q.w, m.r_max, in, f.x, f.y, e));
                     }
                 }
             }
@@ -254,7 +225,9 @@ k_eval_broad(const ModelDev m, const SceneDev sc, const EvalArgs a)
                 while (mask) {
                     const int ob = base + __ffs(mask) - 1;
                     mask &= mask - 1;
-                    dmin = fminf(dmin, survivor_box<NSPH>(m, H, Z, c1, s1, s_bc[ob], s_bh[ob]));
+                    const float4 cb = s_bc[ob];
+                    const uint32_t in = spheres_in_reach<NSPH>(H2, c1, s1, cb.x, cb.y, cb.w * cb.w);
+                    if (in) dmin = fminf(dmin, walk_box<NSPH>(s_tab, tr, m.base_z, c.q.w, in, cb, s_bh[ob]));
                 }
             }
             unit_accumulate(a, c, dmin, ir.cand, chunk, lane, acc, count);
