@@ -479,6 +479,7 @@ int run_eval(cp_planner *p, const float *d_xi, int n, double *d_J, uint8_t *d_fl
     a.ends = p->ends_f;
     a.ctas_per_sm = p->prm.eval_ctas_per_sm;
     a.withhold_staging = p->prm.debug_withhold_staging == 1;
+    a.want_len = d_terms != nullptr;
     a.broadphase = p->prm.eval_exhaustive ? 0 : 1;
     a.work = p->timer.on ? p->work : nullptr;
     if (p->timer.on) {
@@ -1523,7 +1524,7 @@ int record_batch(cp_batch *b)
         if ((rc = launch_batch_sample(b->qdev, b->tab_sample, b->n_sample, b->max_K, (uint32_t)t, b->st)) != CP_OK)
             return rc;
         if ((rc = launch_batch_eval_polar(b->mdev, b->ev_pop, b->tiles_pop, b->n_tiles_pop, b->queue + t, b->max_S,
-                                          b->shape.threads, b->eval_blocks, b->st)) != CP_OK)
+                                          b->shape.threads, b->eval_blocks, false, b->st)) != CP_OK)
             return rc;
         if ((rc = launch_batch_finalize(b->qdev, b->tab_cand, b->n_cand, nullptr, b->st)) != CP_OK) return rc;
         int *sorted = nullptr;
@@ -1542,7 +1543,7 @@ int record_batch(cp_batch *b)
     if ((rc = launch_batch_outputs(b->qdev, b->nq, true, nullptr, 0, b->st)) != CP_OK) return rc;
     const int mean_blocks = std::max(1, std::min(b->eval_blocks, b->n_tiles_mean));
     if ((rc = launch_batch_eval_polar(b->mdev, b->ev_mean, b->tiles_mean, b->n_tiles_mean, b->queue + b->iters,
-                                      b->max_S, b->shape.threads, mean_blocks, b->st)) != CP_OK)
+                                      b->max_S, b->shape.threads, mean_blocks, true, b->st)) != CP_OK)
         return rc;
     if ((rc = launch_batch_finalize(b->qdev, nullptr, b->nq, b->ev_mean, b->st)) != CP_OK) return rc;
     if ((rc = launch_batch_outputs(b->qdev, b->nq, false, b->d_out, kOutStride, b->st)) != CP_OK) return rc;
@@ -1966,7 +1967,7 @@ int cp_batch_evaluate(cp_batch *b, int32_t reps, double *ms)
         CP_CUDA(cudaMemsetAsync(counter, 0, sizeof(int), b->st));
         CP_CUDA(cudaEventRecord(b->ev0, b->st));
         int rc = launch_batch_eval_polar(b->mdev, b->ev_pop, b->tiles_pop, b->n_tiles_pop, counter, b->max_S,
-                                         b->shape.threads, b->eval_blocks, b->st);
+                                         b->shape.threads, b->eval_blocks, false, b->st);
         if (rc != CP_OK) return rc;
         CP_CUDA(cudaEventRecord(b->ev1, b->st));
         CP_CUDA(cudaEventSynchronize(b->ev1));

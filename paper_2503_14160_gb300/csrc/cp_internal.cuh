@@ -169,6 +169,7 @@ struct EvalArgs {
     const float4 *ends;         // optional device copy {q0, qd}, read at run time
     int ctas_per_sm;            // persistent-grid CTAs per SM (0: as many as fit)
     int withhold_staging;       // test hook: issue no staging copy, so its wait runs out
+    int want_len;               // the terms (and with them the path length) are asked for
     int broadphase;             // 1: per-unit broad phase before the per-sphere filter
     unsigned long long *work;   // optional [2]: += obstacles that passed the unit box test,
                                 // += (unit, obstacle) box tests run (polar index form)
@@ -387,7 +388,7 @@ int launch_batch_sample(const BatchQueryDev *qd, const int2 *tab, int blocks, in
 constexpr int kBatchSampleCands = 256;   // candidates per block of the batched sampler
 int batch_eval_configure();
 int launch_batch_eval_polar(const ModelDev &m, const BatchEvalDev *qd, const int4 *tiles, int n_tiles, int *queue,
-                            int max_S, int threads, int blocks, cudaStream_t st);
+                            int max_S, int threads, int blocks, bool want_len, cudaStream_t st);
 int batch_eval_max_blocks(const ModelDev &m, int threads, int max_S, int num_sms);
 // tab non-null: the populations (blocks of 256 candidates); null: the mean candidates of
 // `blocks` queries, whose evaluation is described by mean_ev.

@@ -77,6 +77,25 @@ static __device__ __forceinline__ float3 sdf_box_grad(float x, float y, float z,
     return make_float3(0.f, 0.f, sz);
 }
 
+// Conversions between floats and integers, rounding to an integral float among them, run on the
+// FP64 unit of this part: a warp instruction holds it for 64 cycles, and the seven of a unit had it
+// busy for 75% of the polar evaluation's cycles. Adding 1.5 x 2^23 rounds to an integer (to
+// nearest, ties to even) in the FP32 adder, for |v| < 2^22; further out the result is an integer
+// next to v, which the uses below allow.
+constexpr float kRoundShift = 12582912.f;
+
+static __device__ __forceinline__ float round_even(float v)
+{
+    return __fadd_rn(__fadd_rn(v, kRoundShift), -kRoundShift);
+}
+
+// The integer next to v (ties to even), saturating outwards: monotone in v for every v (the bits of
+// floats of one sign are), far values beyond any index either way.
+static __device__ __forceinline__ int round_index(float v)
+{
+    return __float_as_int(__fadd_rn(v, kRoundShift)) - 0x4B400000;
+}
+
 // Sine and cosine of an angle for the kinematics: the angle reduced to [-pi, pi] by 2 pi in
 // two parts (Cody and Waite's additive reduction; 2 pi = 6.28318548202514648 - 1.7484555e-7,
 // both parts exact in FP32, so the reduced angle is within a few 1e-7 rad of the true one for
@@ -85,11 +104,13 @@ static __device__ __forceinline__ float3 sdf_box_grad(float x, float y, float z,
 // most about 10.5 m) that moves a sphere centre by under 1e-5 m, within the 2e-5 m to which
 // the distances are checked against the FP64 oracle; the accurate library sincosf costs
 // several times the instructions on this hottest path.
-static __device__ __forceinline__ void sincos_reduced(float x, float *s, float *c)
+// Returns the reduced angle.
+static __device__ __forceinline__ float sincos_reduced(float x, float *s, float *c)
 {
-    const float k = rintf(x * 0.159154943091895336f);
+    const float k = round_even(__fmul_rn(x, 0.159154943091895336f));
     const float r = fmaf(k, 1.7484555e-7f, fmaf(-k, 6.28318548202514648f, x));
     __sincosf(r, s, c);
+    return r;
 }
 
 // Heights and signed horizontal distances of the sphere centres from the sines and cosines of the
@@ -120,6 +141,7 @@ static __device__ __forceinline__ void crane_place(const ModelDev &m, float q4s,
 // point and the smooth cost, whose softplus penalty is checked to 1e-4 relative).
 struct ChainTrig {
     float s1, c1, s2, c2, s23, c23;
+    float phi;   // kFastTrig: the slew angle reduced to [-pi, pi] (|q1| < 2^14)
 };
 
 template <bool kFastTrig = true>
@@ -127,10 +149,11 @@ static __device__ __forceinline__ ChainTrig chain_trig(float4 q)
 {
     ChainTrig t;
     if (kFastTrig) {
-        sincos_reduced(q.x, &t.s1, &t.c1);
+        t.phi = sincos_reduced(q.x, &t.s1, &t.c1);
         sincos_reduced(q.y, &t.s2, &t.c2);
         sincos_reduced(q.y + q.z, &t.s23, &t.c23);
     } else {
+        t.phi = q.x;
         sincosf(q.x, &t.s1, &t.c1);
         sincosf(q.y, &t.s2, &t.c2);
         sincosf(q.y + q.z, &t.s23, &t.c23);
@@ -453,7 +476,7 @@ static __device__ __forceinline__ bool unit_near(const UnitFrame &f, float4 r, f
 // Lanes past n_s evaluate the last checkpoint and are marked invalid.
 struct Checkpoint {
     float4 q;
-    float jp, len, jl;
+    float jp, jl;   // the increment's length is sqrt(jp)
     int k;
     bool valid;
 };
@@ -487,7 +510,6 @@ static __device__ __forceinline__ Checkpoint checkpoint_at(const ModelDev &m, co
     c.q = combine4(bw, P0, P1, P2, P3);
     const float4 dq = combine4(dbw, P0, P1, P2, P3);   // q(s_k) - q(s_{k-1})
     c.jp = fmaf(dq.x, dq.x, fmaf(dq.y, dq.y, fmaf(dq.z, dq.z, dq.w * dq.w)));
-    c.len = sqrtf(c.jp);
     // limit excess per joint: only one of v - q_max and q_min - v can be positive (q_min <
     // q_max), so max(0, v - q_max)^2 + max(0, q_min - v)^2 is e^2 with e the larger of the two
     // clamped at 0, the same rounding as the two-term form; the differences and squares packed
@@ -522,8 +544,10 @@ static __device__ __forceinline__ ItemRange item_range(const EvalArgs &a, int it
 // one value, so lane 8 j ends with the sum of value j (6 shuffles instead of 20); lane 8 j
 // keeps the item's FP64 sum of value j. The ballot word of checkpoints in collision and the
 // per-checkpoint penalty are written when asked for; a kernel compiled with kExtras false
-// (launched only when neither is asked for) leaves out their tests.
-template <bool kExtras = true>
+// (launched only when neither is asked for) leaves out their tests, and one with kLen false
+// (launched when the terms are not asked for, as by a plan's iterations) the length's square
+// root: J does not contain it.
+template <bool kExtras = true, bool kLen = true>
 static __device__ __forceinline__ void unit_accumulate(const EvalArgs &a, const Checkpoint &c, float dmin,
                                                        int cand, int chunk, int lane, double &acc,
                                                        uint32_t &count)
@@ -531,7 +555,7 @@ static __device__ __forceinline__ void unit_accumulate(const EvalArgs &a, const 
     const float pen = fmaxf(0.f, -dmin);
     const bool hit = c.valid && (dmin < 0.f);
     const float v0 = c.valid ? c.jp : 0.f, v1 = c.valid ? pen : 0.f;
-    const float v2 = c.valid ? c.jl : 0.f, v3 = c.valid ? c.len : 0.f;
+    const float v2 = c.valid ? c.jl : 0.f, v3 = kLen && c.valid ? sqrtf(c.jp) : 0.f;
     const bool hi16 = (lane & 16) != 0, hi8 = (lane & 8) != 0;
     const float r0 = __shfl_xor_sync(0xffffffffu, hi16 ? v0 : v2, 16);
     const float r1 = __shfl_xor_sync(0xffffffffu, hi16 ? v1 : v3, 16);

@@ -143,7 +143,8 @@ __device__ __forceinline__ uint32_t spheres_in_reach(const float2 *H2, float c1,
 // loop) through the per-sphere polar filter, two packed FP32x2 operations per sphere pair,
 // and the exact distance of the spheres that pass (walk_cylinder, walk_box). Its distances are those of the exhaustive form for
 // every pair that can be in contact, so both forms give the same results bit for bit.
-template <int NSPH>
+// kPlain: neither the per-checkpoint outputs nor the terms are asked for.
+template <int NSPH, bool kPlain>
 __global__ void __launch_bounds__(kEvalThreads, kEvalBroadMinBlocks)
 k_eval_broad(const ModelDev m, const SceneDev sc, const EvalArgs a)
 {
@@ -230,7 +231,7 @@ k_eval_broad(const ModelDev m, const SceneDev sc, const EvalArgs a)
                     if (in) dmin = fminf(dmin, walk_box<NSPH>(s_tab, tr, m.base_z, c.q.w, in, cb, s_bh[ob]));
                 }
             }
-            unit_accumulate(a, c, dmin, ir.cand, chunk, lane, acc, count);
+            unit_accumulate<!kPlain, !kPlain>(a, c, dmin, ir.cand, chunk, lane, acc, count);
         }
         item_flush(a, it, acc, count, lane);
     }
@@ -403,8 +404,10 @@ int eval_ensure_smem(size_t smem_bytes)
     int rc;
     if ((rc = raise_smem(k_eval<12>, smem_bytes)) != CP_OK) return rc;
     if ((rc = raise_smem(k_eval<16>, smem_bytes)) != CP_OK) return rc;
-    if ((rc = raise_smem(k_eval_broad<12>, smem_bytes)) != CP_OK) return rc;
-    return raise_smem(k_eval_broad<16>, smem_bytes);
+    if ((rc = raise_smem(k_eval_broad<12, true>, smem_bytes)) != CP_OK) return rc;
+    if ((rc = raise_smem(k_eval_broad<12, false>, smem_bytes)) != CP_OK) return rc;
+    if ((rc = raise_smem(k_eval_broad<16, true>, smem_bytes)) != CP_OK) return rc;
+    return raise_smem(k_eval_broad<16, false>, smem_bytes);
 }
 
 int launch_eval(const ModelDev &m, const SceneDev &sc, const EvalArgs &a, int num_sms,
@@ -413,18 +416,10 @@ int launch_eval(const ModelDev &m, const SceneDev &sc, const EvalArgs &a, int nu
     const int units = a.n * a.P;   // work items
     if (units == 0) return CP_OK;
     const size_t smem = eval_smem_bytes(sc.n_cyl, sc.n_box, a.S);
-    const int cpsm = a.ctas_per_sm;
-    if (m.n_spheres == 12) {
-        if (a.broadphase)
-            launch_chained(k_eval_broad<12>, eval_grid(k_eval_broad<12>, smem, num_sms, units, cpsm), kEvalThreads, smem, st, m, sc, a);
-        else
-            launch_chained(k_eval<12>, eval_grid(k_eval<12>, smem, num_sms, units, cpsm), kEvalThreads, smem, st, m, sc, a);
-    } else {
-        if (a.broadphase)
-            launch_chained(k_eval_broad<16>, eval_grid(k_eval_broad<16>, smem, num_sms, units, cpsm), kEvalThreads, smem, st, m, sc, a);
-        else
-            launch_chained(k_eval<16>, eval_grid(k_eval<16>, smem, num_sms, units, cpsm), kEvalThreads, smem, st, m, sc, a);
-    }
+    const bool plain = a.words_out == nullptr && a.pen_out == nullptr && !a.want_len;
+    auto kern = m.n_spheres == 12 ? (a.broadphase ? (plain ? k_eval_broad<12, true> : k_eval_broad<12, false>) : k_eval<12>)
+                                  : (a.broadphase ? (plain ? k_eval_broad<16, true> : k_eval_broad<16, false>) : k_eval<16>);
+    launch_chained(kern, eval_grid(kern, smem, num_sms, units, a.ctas_per_sm), kEvalThreads, smem, st, m, sc, a);
     CP_LAUNCHED("k_eval");
     return CP_OK;
 }

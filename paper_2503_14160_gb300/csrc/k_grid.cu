@@ -36,8 +36,6 @@ constexpr int kCtrlSlots = CP_MAX_WAYPOINTS + 8;   // control points per warp, f
 constexpr float kPolarPadR = 1e-3f;                // m: rounding of rho, |h| and the ring index
 constexpr float kPolarPadA = 1e-4f;                // rad: rounding of the angles and bin index
 constexpr float kPi = 3.14159265358979323846f;
-constexpr float kTwoPiHi = 6.28318548202514648f;   // 2 pi = kTwoPiHi + kTwoPiLo (Cody-Waite)
-constexpr float kTwoPiLo = -1.7484555e-7f;
 
 // Bins of an obstacle record r = {cx, cy, ., reach}: a0 .. a0 + na - 1 (mod n_ang), and the
 // ring of its centre. A point within `reach` of the centre has, when rho > reach, an angle
@@ -133,14 +131,11 @@ __global__ void k_polar_fill(const SceneDev sc, const PolarDev g, int *cursor, f
     }
 }
 
-// Slew angle wrapped to [-pi, pi]: Cody-Waite reduction by 2 pi in two parts (accurate to a
-// few 1e-7 rad for |phi| below 2^14 rad), in FP64 beyond.
-__device__ __forceinline__ float wrap_angle(float phi)
+// Slew angles from 2^14 rad on wrapped to [-pi, pi] in FP64 (below that the kinematics' reduced
+// angle is accurate to a few 1e-7 rad). A call of its own: inlined, the compiler predicated its
+// five FP64 instructions instead of branching, and every unit held the FP64 unit for them.
+__device__ __noinline__ float wrap_far(float phi)
 {
-    if (fabsf(phi) < 16384.f) {
-        const float k = rintf(phi * 0.159154943091895336f);
-        return fmaf(-k, kTwoPiLo, fmaf(-k, kTwoPiHi, phi));
-    }
     const double d = (double)phi;
     return (float)(d - 6.283185307179586477 * rint(d * 0.15915494309189533577));
 }
@@ -151,7 +146,7 @@ __device__ __forceinline__ float wrap_angle(float phi)
 // and the exact distance of those that pass. kExtras false leaves out the work counters and
 // the per-checkpoint outputs (the plan's own evaluations ask for neither); the sums are the
 // same.
-template <int NSPH, bool kExtras = true>
+template <int NSPH, bool kExtras, bool kLen>
 static __device__ __forceinline__ void polar_item(const ModelDev &m, const SceneDev &sc, const PolarDev &g,
                                                   const EvalArgs &a, const SphereTable<NSPH> &tab,
                                                   const float4 *s_basis, float4 *s_ctrl, int it, int lane,
@@ -177,7 +172,7 @@ static __device__ __forceinline__ void polar_item(const ModelDev &m, const Scene
         }
         float dmin = CUDART_INF_F;
         if (hmin <= hmax) {
-            const float phi0 = wrap_angle(c.q.x);
+            const float phi0 = fabsf(c.q.x) < 16384.f ? tr.phi : wrap_far(c.q.x);
 #pragma unroll 1
             for (int side = 0; side < 2; ++side) {
                 // spheres with h >= 0 lie on the half-line at the slew angle, those with h < 0
@@ -186,10 +181,13 @@ static __device__ __forceinline__ void polar_item(const ModelDev &m, const Scene
                 const float r_hi = side ? -hmin : hmax;
                 if (!(r_lo <= r_hi)) continue;
                 const float ang = side ? (phi0 >= 0.f ? phi0 - kPi : phi0 + kPi) : phi0;
-                const int bin = min(max((int)floorf((ang + kPi) * g.inv_da), 0), g.n_ang - 1);
+                // v - 1/2 to the nearest integer is the floor of v but on the very boundary between
+                // two cells, where either will do: the index lists every obstacle in each bin
+                // within kPolarPadA of its reach, and `reach` carries kPolarPadR
+                const int bin = min(max(round_index(fmaf(ang + kPi, g.inv_da, -0.5f)), 0), g.n_ang - 1);
                 const float reach = g.w_max + kPolarPadR;
-                const int r0 = min(max((int)floorf((r_lo - reach) * g.inv_dr), 0), g.n_ring - 1);
-                const int r1 = min(max((int)floorf((r_hi + reach) * g.inv_dr), 0), g.n_ring - 1);
+                const int r0 = min(max(round_index(fmaf(r_lo - reach, g.inv_dr, -0.5f)), 0), g.n_ring - 1);
+                const int r1 = min(max(round_index(fmaf(r_hi + reach, g.inv_dr, -0.5f)), 0), g.n_ring - 1);
                 const int cell = bin * g.n_ring;
                 const int beg = __ldg(g.cell_start + cell + r0);
                 const int end = min(__ldg(g.cell_start + cell + r1 + 1), g.capacity);
@@ -221,12 +219,12 @@ static __device__ __forceinline__ void polar_item(const ModelDev &m, const Scene
             }
         }
         __syncwarp();
-        unit_accumulate<kExtras>(a, c, dmin, ir.cand, chunk, lane, acc, count);
+        unit_accumulate<kExtras, kLen>(a, c, dmin, ir.cand, chunk, lane, acc, count);
     }
     item_flush(a, it, acc, count, lane);
 }
 
-template <int NSPH, bool kExtras>
+template <int NSPH, bool kExtras, bool kLen>
 __global__ void __launch_bounds__(kPolarThreads, CP_POLAR_MIN_BLOCKS)
 k_eval_polar(const ModelDev m, const SceneDev sc, const PolarDev g, const EvalArgs a)
 {
@@ -252,11 +250,11 @@ k_eval_polar(const ModelDev m, const SceneDev sc, const PolarDev g, const EvalAr
             if (lane == 0) it = atomicAdd(a.queue, 1);
             it = __shfl_sync(0xffffffffu, it, 0);
             if (it >= items) break;
-            polar_item<NSPH, kExtras>(m, sc, g, a, s_tab, s_basis, s_ctrl, it, lane, survivors, tests);
+            polar_item<NSPH, kExtras, kLen>(m, sc, g, a, s_tab, s_basis, s_ctrl, it, lane, survivors, tests);
         }
     } else {
         for (int it = warp; it < items; it += n_warps)
-            polar_item<NSPH, kExtras>(m, sc, g, a, s_tab, s_basis, s_ctrl, it, lane, survivors, tests);
+            polar_item<NSPH, kExtras, kLen>(m, sc, g, a, s_tab, s_basis, s_ctrl, it, lane, survivors, tests);
     }
     if (kExtras && a.work != nullptr) {
         const uint32_t ws = __reduce_add_sync(0xffffffffu, survivors);
@@ -273,7 +271,7 @@ k_eval_polar(const ModelDev m, const SceneDev sc, const PolarDev g, const EvalAr
 // holds, the CTA restages: it copies the query's view (its evaluation arguments, obstacle
 // records and polar index) and the query's spline table into shared memory. The warps then
 // take the tile's items in turn; an item's arithmetic is that of the single-query launch.
-template <int NSPH, int THREADS, int MINB>
+template <int NSPH, int THREADS, int MINB, bool kLen>
 __global__ void __launch_bounds__(THREADS, MINB)
 k_batch_eval_polar(const ModelDev m, const BatchEvalDev *__restrict__ qd, const int4 *__restrict__ tiles,
                    int n_tiles, int *queue, int max_S)
@@ -305,7 +303,7 @@ k_batch_eval_polar(const ModelDev m, const BatchEvalDev *__restrict__ qd, const 
             __syncthreads();
         }
         for (int it = tile.y + wib; it < tile.z; it += W)   // the batch asks for no counters or outputs
-            polar_item<NSPH, false>(m, s_q.sc, s_q.g, s_q.a, s_tab, s_basis, s_ctrl, it, lane, survivors, tests);
+            polar_item<NSPH, false, kLen>(m, s_q.sc, s_q.g, s_q.a, s_tab, s_basis, s_ctrl, it, lane, survivors, tests);
         __syncthreads();   // the tile's items are done before s_tile and s_q change
     }
 }
@@ -395,8 +393,10 @@ int launch_eval_polar(const ModelDev &m, const SceneDev &sc, const PolarDev &g, 
     const size_t smem = sizeof(float4) * (2 * (size_t)a.S + (size_t)(kPolarThreads / 32) * kCtrlSlots);
     // the plain form (no work counters, no per-checkpoint outputs) drops their bookkeeping
     const bool extras = a.work != nullptr || a.words_out != nullptr || a.pen_out != nullptr;
-    auto kern = m.n_spheres == 12 ? (extras ? k_eval_polar<12, true> : k_eval_polar<12, false>)
-                                  : (extras ? k_eval_polar<16, true> : k_eval_polar<16, false>);
+    auto pick = [&](auto plain, auto terms, auto full) { return extras ? full : (a.want_len ? terms : plain); };
+    auto kern = m.n_spheres == 12
+                    ? pick(k_eval_polar<12, false, false>, k_eval_polar<12, false, true>, k_eval_polar<12, true, true>)
+                    : pick(k_eval_polar<16, false, false>, k_eval_polar<16, false, true>, k_eval_polar<16, true, true>);
     int per_sm = 0;
     CP_CUDA(raise_polar_smem(kern, smem));
     CP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPolarThreads, smem));
@@ -411,20 +411,26 @@ int launch_eval_polar(const ModelDev &m, const SceneDev &sc, const PolarDev &g, 
 }
 
 // Batched form: CTAs of 128, 256 or 512 threads (block shape picked by the autotuner).
-template <int NSPH, int THREADS>
+template <int NSPH, int THREADS, bool kLen>
 static auto batch_eval_kernel()
 {
-    constexpr int MINB = THREADS == 128 ? 2 * CP_POLAR_MIN_BLOCKS : (THREADS == 256 ? CP_POLAR_MIN_BLOCKS : 1);
-    return k_batch_eval_polar<NSPH, THREADS, MINB>;
+    constexpr int MINB = CP_POLAR_MIN_BLOCKS * 256 / THREADS;   // the same warps per SM for every shape
+    return k_batch_eval_polar<NSPH, THREADS, MINB, kLen>;
 }
 
-template <int NSPH>
+template <int NSPH, bool kLen>
 static void *batch_eval_fn(int threads)
 {
-    if (threads == 128) return (void *)batch_eval_kernel<NSPH, 128>();
-    if (threads == 256) return (void *)batch_eval_kernel<NSPH, 256>();
-    if (threads == 512) return (void *)batch_eval_kernel<NSPH, 512>();
+    if (threads == 128) return (void *)batch_eval_kernel<NSPH, 128, kLen>();
+    if (threads == 256) return (void *)batch_eval_kernel<NSPH, 256, kLen>();
+    if (threads == 512) return (void *)batch_eval_kernel<NSPH, 512, kLen>();
     return nullptr;
+}
+
+static void *batch_eval_fn(int n_spheres, int threads, bool want_len)
+{
+    if (n_spheres == 12) return want_len ? batch_eval_fn<12, true>(threads) : batch_eval_fn<12, false>(threads);
+    return want_len ? batch_eval_fn<16, true>(threads) : batch_eval_fn<16, false>(threads);
 }
 
 static size_t batch_eval_smem(int threads, int max_S)
@@ -434,23 +440,26 @@ static size_t batch_eval_smem(int threads, int max_S)
 
 int batch_eval_max_blocks(const ModelDev &m, int threads, int max_S, int num_sms)
 {
-    void *fn = m.n_spheres == 12 ? batch_eval_fn<12>(threads) : batch_eval_fn<16>(threads);
-    if (fn == nullptr) return set_error("batched evaluation: %d threads per CTA is not 128, 256 or 512", threads), -1;
     const size_t smem = batch_eval_smem(threads, max_S);
-    cudaFuncAttributes at{};
-    CP_CUDA(cudaFuncGetAttributes(&at, fn));
-    if ((size_t)at.maxDynamicSharedSizeBytes < smem)
-        CP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    void *fn = nullptr;
+    for (const bool len : {true, false}) {   // the mean paths' form, then the populations'
+        fn = batch_eval_fn(m.n_spheres, threads, len);
+        if (fn == nullptr) return set_error("batched evaluation: %d threads per CTA is not 128, 256 or 512", threads), -1;
+        cudaFuncAttributes at{};
+        CP_CUDA(cudaFuncGetAttributes(&at, fn));
+        if ((size_t)at.maxDynamicSharedSizeBytes < smem)
+            CP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    }
     int per_sm = 0;
     CP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem));
     return (per_sm < 1 ? 1 : per_sm) * num_sms;
 }
 
 int launch_batch_eval_polar(const ModelDev &m, const BatchEvalDev *qd, const int4 *tiles, int n_tiles, int *queue,
-                            int max_S, int threads, int blocks, cudaStream_t st)
+                            int max_S, int threads, int blocks, bool want_len, cudaStream_t st)
 {
     if (n_tiles == 0) return CP_OK;
-    void *fn = m.n_spheres == 12 ? batch_eval_fn<12>(threads) : batch_eval_fn<16>(threads);
+    void *fn = batch_eval_fn(m.n_spheres, threads, want_len);
     if (fn == nullptr) return set_error("batched evaluation: %d threads per CTA is not 128, 256 or 512", threads), CP_ERR_ARG;
     const size_t smem = batch_eval_smem(threads, max_S);
     ModelDev mm = m;
