@@ -264,7 +264,8 @@ int launch_factor(const double *C, double sigma2, const double *sigma_dev, int D
 
 int batch_factor_clusters(int max_D, int *count)
 {
-    const ClusterLaunch l(kMaxCtas, (max_D + kRows - 1) / kRows, nullptr, false);
+    const int n_ctas = (max_D + kRows - 1) / kRows;
+    const ClusterLaunch l(n_ctas, n_ctas, nullptr, false);   // the grid a whole number of clusters
     CP_CUDA(cudaOccupancyMaxActiveClusters(count, k_batch_factor_cluster, &l.cfg));
     return CP_OK;
 }

@@ -229,3 +229,23 @@ def test_ranking_passes(lib, crane, N):
         lib.cp_get_elites(pl.handle, el)
         torch.cuda.synchronize()
     assert np.array_equal(el.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("K", [2, 8, 12, 20, 24, 28, 32])
+def test_batch_factor_cluster_sizes(lib, crane, K):
+    """Every number of 16-row blocks of the largest factor of a batch: the batch can be set up, and
+    its plans are those of its planners alone."""
+    from paper_2503_14160_gb300 import workloads
+    Ks = [K, 3]
+    scenes = [lib.HostScene.from_scene(workloads.empty_scene()) for _ in Ks]
+    params = [lib.make_params(80, k, 4, seed=q, query=q, grid_cell=0.5) for q, k in enumerate(Ks)]
+    b = lib.cp_batch_init(lib.make_model(crane), scenes, params, [e[0] for e in ENDS], [e[1] for e in ENDS], 2)
+    try:
+        res = lib.cp_batch_run(b, len(Ks), K=Ks)
+        for q, k in enumerate(Ks):
+            p = lib.cp_batch_planner(b, q)
+            lib.cp_set_endpoints(p, *ENDS[q])
+            ctrl, _ = lib.cp_plan(p, 2, K=k)
+            assert np.array_equal(res[q][0], ctrl)
+    finally:
+        lib.cp_batch_destroy(b)
