@@ -19,16 +19,23 @@
 // w_k = (x_k, u_k) with a border for t_F (the defects couple neighbours and t_F); it is
 // factored block by block (16 x 16 Cholesky factors L_k, L_k^-1 E_k) and the border is taken
 // through its Schur complement. The dynamics' Jacobian per grid point comes from forward-mode
-// differentiation (value and one derivative per pass, 16 passes). Everything is FP64: a
+// differentiation (one derivative per pass, 16 passes). Everything is FP64: a
 // cluster of two, four or eight CTAs of 512 threads per trajectory.
 //
-// What bounds it: the FP64 pipe, where a warp instruction holds an SM for about 19 cycles, so
-// the work is laid out to issue few of them. Rows 0-9 of df/dw are constant (the rates and the
-// inputs), so only rows 10 and 11 are stored and every sum over the 12 rows takes the terms
-// that are not zero; the quotients by rho and 2N are formed once per entry; the block factor
-// carries the right-hand sides as further rows on the lanes that a 16-row factor leaves idle.
+// What bounds it: the FP64 units. A warp instruction holds its scheduler's unit for 64 cycles
+// whatever lanes are active, and a dependent one waits as long, so the work is laid out to issue
+// few of them and to spread them over all schedulers of the cluster. Rows 0-9 of df/dw are
+// constant (the rates and the inputs), so only rows 10 and 11 are stored and every sum over the 12
+// rows takes the terms that are not zero; a warp of the Jacobian takes one variable, so that the
+// terms that do not depend on it are left out; quotients are formed once; the block factor
+// carries the right-hand sides as further rows on the lanes that a 16-row factor leaves idle;
+// warps are numbered across the CTAs; the back substitution reads its blocks from shared memory,
+// staged before the barrier. 64 trajectories of 100 intervals (two CTAs each): 164.2 ms with none of
+// this, 105.0 ms with the first two and the factor, 75.6 ms with all of it, with the same bits. Of
+// an LM step's 1.15 M cycles then the levels' factors take 55%, their updates 30%, the Jacobian 6%.
 #include <cmath>
 #include <new>
+#include <type_traits>
 
 #include <cooperative_groups.h>
 #include <nvtx3/nvToolsExt.h>
@@ -50,7 +57,8 @@ constexpr int kSumCtas = 2;       // CTAs of a cluster that take the team sums (
 constexpr int kRedDoubles = 64;   // block reductions: [0, 32) and [32, 64) (one slot per warp)
 constexpr int NX = 12, NU = 4, NW = 16;
 constexpr int NF = 2;             // dense rows of df/dw (rows NX - NF .. NX - 1)
-constexpr int kWarpScratch = 3 * NW * NW;   // doubles of shared memory per warp (three blocks)
+constexpr int kWarpScratch = 3 * NW * NW + 2 * NW;   // doubles of shared memory per warp (three
+                                                     // blocks, two of them with padded rows)
 constexpr double kGravity = 9.81;
 
 // A value and one derivative (forward mode).
@@ -69,6 +77,56 @@ __device__ __forceinline__ Dual operator/(Dual a, Dual b)
 template <typename T> __device__ __forceinline__ T lift(double v);
 template <> __device__ __forceinline__ double lift<double>(double v) { return v; }
 template <> __device__ __forceinline__ Dual lift<Dual>(double v) { return {v, 0.0}; }
+
+// The same where the seed is known when this is compiled: an operand that does not depend on it is
+// a plain double, and its products and quotients leave out the terms that a zero derivative would
+// make. What is left is rounded as the full pairs are, each operation by name, so that no fusion
+// is left to the compiler: fma(0, x, y) is y and fma(x, y, 0) the rounded product.
+struct Part {
+    double v, d;
+};
+__device__ __forceinline__ Part operator+(Part a, Part b) { return {a.v + b.v, __dadd_rn(a.d, b.d)}; }
+__device__ __forceinline__ Part operator+(Part a, double b) { return {a.v + b, a.d}; }
+__device__ __forceinline__ Part operator+(double a, Part b) { return {a + b.v, b.d}; }
+__device__ __forceinline__ Part operator-(Part a, Part b) { return {a.v - b.v, __dadd_rn(a.d, -b.d)}; }
+__device__ __forceinline__ Part operator-(Part a, double b) { return {a.v - b, a.d}; }
+__device__ __forceinline__ Part operator-(double a, Part b) { return {a - b.v, -b.d}; }
+__device__ __forceinline__ Part operator*(Part a, Part b) { return {a.v * b.v, fma(a.v, b.d, __dmul_rn(a.d, b.v))}; }
+__device__ __forceinline__ Part operator*(double a, Part b) { return {a * b.v, __dmul_rn(a, b.d)}; }
+__device__ __forceinline__ Part operator*(Part a, double b) { return {a.v * b, __dmul_rn(a.d, b)}; }
+__device__ __forceinline__ Part operator/(Part a, double b) { return {a.v / b, a.d / b}; }
+__device__ __forceinline__ double value(double a) { return a; }
+__device__ __forceinline__ double value(Part a) { return a.v; }
+
+// x with the value v
+__device__ __forceinline__ double with_value(double, double v) { return v; }
+__device__ __forceinline__ Part with_value(Part x, double v) { return {v, x.d}; }
+
+// z + x y and z - x y with the values fused
+template <typename X, typename Y, typename Z>
+__device__ __forceinline__ auto madd(X x, Y y, Z z)
+{
+    return with_value(z + x * y, fma(value(x), value(y), value(z)));
+}
+template <typename X, typename Y, typename Z>
+__device__ __forceinline__ auto msub(X x, Y y, Z z)
+{
+    return with_value(z - x * y, fma(-value(x), value(y), value(z)));
+}
+
+// s x + y for a constant s, fused
+__device__ __forceinline__ double axpy(double s, double x, double y) { return fma(s, x, y); }
+__device__ __forceinline__ Part axpy(double s, Part x, double y) { return {fma(s, x.v, y), __dmul_rn(s, x.d)}; }
+__device__ __forceinline__ Part axpy(double s, double x, Part y) { return {fma(s, x, y.v), y.d}; }
+__device__ __forceinline__ Part axpy(double s, Part x, Part y) { return {fma(s, x.v, y.v), fma(s, x.d, y.d)}; }
+
+// Variable I of the grid point's 16 (states, then inputs).
+template <int SEED, int I>
+__device__ __forceinline__ auto seeded(const double *w)
+{
+    if constexpr (SEED == I) return Part{w[I], 1.0};
+    else return w[I];
+}
 
 // Cosine and sine of an angle of the dynamics. The primal values depend on the grid point
 // only, so a cache (c, s pairs written by the value pass at that point) serves the 16
@@ -101,13 +159,29 @@ __device__ __forceinline__ void trig_of(Dual a, const double *cache, double *cw,
     s = {sv, cv * a.d};
 }
 
+__device__ __forceinline__ void trig_of(Part a, const double *cache, double *, int idx, Part &c, Part &s)
+{
+    const double cv = cache[2 * idx], sv = cache[2 * idx + 1];
+    c = {cv, __dmul_rn(-sv, a.d)};
+    s = {sv, __dmul_rn(cv, a.d)};
+}
+
 struct TrajDev {
     double base_z, boom_len, jib_len, ell;
     double omega_s, omega_t, R[4];
     double x_min[NX], x_max[NX];
     double rho, rho_b, mu0;
     int N, outer, inner;
+    double inv_N, inv_2N;   // reciprocals rounded to nearest
 };
+
+// a / b correctly rounded from b's correctly rounded reciprocal (Markstein's theorem, IBM J. Res.
+// Dev. 34, 1990), three FP64 instructions where a division takes some thirty.
+__device__ __forceinline__ double quotient(double a, double b, double inv_b)
+{
+    const double q = a * inv_b;
+    return fma(fma(-q, b, a), inv_b, q);
+}
 
 // x' = f(x, u): the actuated joints' rates and accelerations, and the swing accelerations from
 // the tip acceleration T'' (cylindrical coordinates of the tip) by
@@ -151,6 +225,108 @@ __device__ void traj_f(const TrajDev &td, const T *x, const T *u, T *out, const 
     out[6] = u1; out[7] = u2; out[8] = u3; out[9] = u4;
     out[10] = lift<T>(0.0) - ra_v / lift<T>(td.ell);
     out[11] = lift<T>(0.0) - rb_v / (td.ell * ca * ca);
+}
+
+// The derivatives of outputs 10 and 11 of traj_f with respect to variable SEED, with the bits of
+// traj_f<Dual>: the same expressions over the operands that depend on the seed, the products that a
+// sum takes in fused as there (the solver's path follows every bit). Not for the slew angle and the
+// swing angles (0, 4, 5), whose derivatives take the accelerations' values.
+template <int SEED>
+__device__ __noinline__ void swing_deriv(const TrajDev &td, const double *w, const double *cache, double *F10,
+                                         double *F11)
+{
+    static_assert(SEED != 0 && SEED != 4 && SEED != 5);
+    double *const cw = nullptr;
+    const auto q1 = seeded<SEED, 0>(w);
+    const auto q2 = seeded<SEED, 1>(w);
+    const auto q3 = seeded<SEED, 2>(w);
+    const auto q4 = seeded<SEED, 3>(w);
+    const auto a = seeded<SEED, 4>(w);
+    const auto b = seeded<SEED, 5>(w);
+    const auto d1 = seeded<SEED, 6>(w);
+    const auto d2 = seeded<SEED, 7>(w);
+    const auto d3 = seeded<SEED, 8>(w);
+    const auto d4 = seeded<SEED, 9>(w);
+    const auto da = seeded<SEED, 10>(w);
+    const auto db = seeded<SEED, 11>(w);
+    const auto u1 = seeded<SEED, 12>(w);
+    const auto u2 = seeded<SEED, 13>(w);
+    const auto u3 = seeded<SEED, 14>(w);
+    const auto u4 = seeded<SEED, 15>(w);
+    const auto lam = td.jib_len + q4;
+    const auto A = q2;
+    const auto B = q2 + q3;
+    const auto dB = d2 + d3;
+    const auto ddB = u2 + u3;
+    std::decay_t<decltype(A)> cA, sA;
+    std::decay_t<decltype(B)> cB, sB;
+    trig_of(A, cache, cw, 0, cA, sA);
+    trig_of(B, cache, cw, 1, cB, sB);
+    const auto h = with_value(axpy(td.boom_len, cA, lam * cB),
+                              fma(value(lam), value(cB), __dmul_rn(td.boom_len, value(cA))));
+    const auto dh = msub(lam * sB, dB, madd(d4, cB, 0.0 - td.boom_len * sA * d2));
+    const auto bend = madd(sB, ddB, cB * dB * dB);
+    const auto rise = madd(cB, ddB, 0.0 - sB * dB * dB);
+    const auto ddh = 0.0 - td.boom_len * (cA * d2 * d2 + sA * u2) + u4 * cB - 2.0 * d4 * sB * dB - lam * bend;
+    const auto ddz = axpy(td.boom_len, cA * u2 - sA * d2 * d2, u4 * sB) + 2.0 * d4 * cB * dB + lam * rise;
+    const auto a_r = ddh - h * d1 * d1;
+    const auto a_t = h * u1 + 2.0 * dh * d1;
+    std::decay_t<decltype(q1)> c1, s1;
+    trig_of(q1, cache, cw, 2, c1, s1);
+    const auto ax = a_r * c1 - a_t * s1;
+    const auto ay = a_r * s1 + a_t * c1;
+    std::decay_t<decltype(a)> ca, sa;
+    std::decay_t<decltype(b)> cb, sb;
+    trig_of(a, cache, cw, 3, ca, sa);
+    trig_of(b, cache, cw, 4, cb, sb);
+    // w = r_aa da^2 + 2 r_ab da db + r_bb db^2
+    const auto wx = 0.0 - sa * da * da;
+    const auto wy = 0.0 - ca * sb * da * da - 2.0 * sa * cb * da * db - ca * sb * db * db;
+    const auto wz = ca * cb * da * da - 2.0 * sa * sb * da * db + ca * cb * db * db;
+    const auto vx = axpy(td.ell, wx, ax);
+    const auto vy = axpy(td.ell, wy, ay);
+    const auto vz = axpy(td.ell, wz, ddz) + kGravity;
+    const auto ra_v = ca * vx - sa * sb * vy + sa * cb * vz;
+    const auto rb_v = ca * cb * vy + ca * sb * vz;
+    const auto o10 = 0.0 - ra_v / td.ell;
+    const auto o11 = 0.0 - rb_v / (td.ell * ca * ca);
+    *F10 = o10.d;
+    *F11 = o11.d;
+}
+
+__device__ __noinline__ void swing_deriv_any(const TrajDev &td, const double *w, int seed, const double *cache,
+                                             double *F10, double *F11)
+{
+    Dual x[NX], u[NU], out[NX];
+#pragma unroll
+    for (int i = 0; i < NX; ++i) x[i] = {w[i], i == seed ? 1.0 : 0.0};
+#pragma unroll
+    for (int i = 0; i < NU; ++i) u[i] = {w[NX + i], NX + i == seed ? 1.0 : 0.0};
+    traj_f<Dual>(td, x, u, out, cache);
+    *F10 = out[10].d;
+    *F11 = out[11].d;
+}
+
+// Column `seed` (uniform over the warp) of the dense rows of df/dw at one grid point.
+__device__ __forceinline__ void swing_column(const TrajDev &td, const double *w, const double *trig, int seed,
+                                             double *F10, double *F11)
+{
+    switch (seed) {
+    case 1: swing_deriv<1>(td, w, trig, F10, F11); break;
+    case 2: swing_deriv<2>(td, w, trig, F10, F11); break;
+    case 3: swing_deriv<3>(td, w, trig, F10, F11); break;
+    case 6: swing_deriv<6>(td, w, trig, F10, F11); break;
+    case 7: swing_deriv<7>(td, w, trig, F10, F11); break;
+    case 8: swing_deriv<8>(td, w, trig, F10, F11); break;
+    case 9: swing_deriv<9>(td, w, trig, F10, F11); break;
+    case 10: swing_deriv<10>(td, w, trig, F10, F11); break;
+    case 11: swing_deriv<11>(td, w, trig, F10, F11); break;
+    case 12: swing_deriv<12>(td, w, trig, F10, F11); break;
+    case 13: swing_deriv<13>(td, w, trig, F10, F11); break;
+    case 14: swing_deriv<14>(td, w, trig, F10, F11); break;
+    case 15: swing_deriv<15>(td, w, trig, F10, F11); break;
+    default: swing_deriv_any(td, w, seed, trig, F10, F11); break;
+    }
 }
 
 // Per-trajectory device workspace (doubles), laid out by the launcher.
@@ -199,12 +375,13 @@ __device__ __forceinline__ TrajWs ws_of(double *base, int N)
 struct Team {
     int rank;   // this CTA's rank in the cluster
     int ctas;   // CTAs in the cluster
-    __device__ int tid() const { return rank * (int)blockDim.x + (int)threadIdx.x; }
+    // warps are numbered across the CTAs, so that a level of few blocks has them on all SMs
+    __device__ int warp() const { return ((int)threadIdx.x >> 5) * ctas + rank; }
+    __device__ int nwarps() const { return ctas * (int)blockDim.x >> 5; }
+    __device__ int tid() const { return warp() * 32 + ((int)threadIdx.x & 31); }
     __device__ int nthreads() const { return ctas * (int)blockDim.x; }
-    __device__ int warp() const { return tid() >> 5; }
-    __device__ int nwarps() const { return nthreads() >> 5; }
     // this thread's first term and the stride of a team sum (no term on the other CTAs)
-    __device__ int sum_first(int n) const { return rank < kSumCtas ? tid() : n; }
+    __device__ int sum_first(int n) const { return rank < kSumCtas ? rank * (int)blockDim.x + (int)threadIdx.x : n; }
     __device__ int sum_stride() const { return kSumCtas * (int)blockDim.x; }
 };
 
@@ -271,7 +448,7 @@ __device__ double merit(const Team &tm, const TrajDev &td, const double *z, cons
                         const double *f, const double *x_S, const double *x_T, double *s_red)
 {
     const int N = td.N;
-    const double h = z[0] / N;
+    const double h = quotient(z[0], N, td.inv_N);
     double acc = 0.0;
     // defects and end states: rho/2 (c + lam/rho)^2
     for (int e = tm.sum_first(NX * (N + 2)); e < NX * (N + 2); e += tm.sum_stride()) {
@@ -368,40 +545,61 @@ __device__ __noinline__ void warp_eliminate16(double *A, const double *Tl_rows, 
     __syncwarp();
 }
 
+// A block of the back substitution in the warp's shared memory: L_k as it is, P_k and Q_k with rows
+// of 17 doubles, so that lanes of different rows read different banks. Coalesced loads, all in
+// flight together; issued before the barrier that the neighbours' solutions wait for.
+constexpr int kPadRow = NW + 1, kPadBlock = NW * kPadRow;
+
+__device__ __forceinline__ void stage_back(double *sm, const double *Lk, const double *P, const double *Q, int lane)
+{
+    double *sP = sm + NW * NW, *sQ = sP + kPadBlock;
+#pragma unroll
+    for (int q = 0; q < NW * NW / 32; ++q) {
+        const int e = q * 32 + lane, at = (e >> 4) * kPadRow + (e & (NW - 1));
+        sm[e] = Lk[e];
+        if (P != nullptr) sP[at] = P[e];
+        if (Q != nullptr) sQ[at] = Q[e];
+    }
+    __syncwarp();
+}
+
 // x_k = L_k^-T (w_k - P_k x_l - Q_k x_r) for both vectors (lanes 0-15 y, 16-31 v, one row
-// each; P or Q absent when null): the products, then L^T x = rhs from the last row up,
-// column by column with the solved entry shuffled to the rows above it.
-__device__ __noinline__ void warp_back16(const double *Lk, const double *P, const double *xl_y, const double *xl_v,
-                            const double *Q, const double *xr_y, const double *xr_v, double *out_y, double *out_v,
-                            int lane)
+// each; P or Q absent when has_p or has_q is false), the block staged by stage_back: the products,
+// then L^T x = rhs from the last row up, column by column with the solved entry shuffled to the
+// rows above it.
+__device__ __noinline__ void warp_back16(const double *sm, bool has_p, const double *xl_y, const double *xl_v,
+                                         bool has_q, const double *xr_y, const double *xr_v, double *out_y,
+                                         double *out_v, int lane)
 {
     const unsigned full = 0xffffffffu;
-    const int r = lane & (NW - 1), which = lane >> 4;
+    const int r = lane & (NW - 1), which = lane >> 4, first = NW * which;
+    const double *sP = sm + NW * NW, *sQ = sP + kPadBlock;
     double *out = which ? out_v : out_y;
+    const double xl = has_p ? (which ? xl_v : xl_y)[r] : 0.0, xq = has_q ? (which ? xr_v : xr_y)[r] : 0.0;
     double x = out[r];   // w_k
-    if (P != nullptr) {
-        const double *xl = which ? xl_v : xl_y;
+    if (has_p) {
         double s0 = 0.0, s1 = 0.0;
+#pragma unroll
         for (int c = 0; c < NW; c += 2) {
-            s0 = fma(P[r * NW + c], xl[c], s0);
-            s1 = fma(P[r * NW + c + 1], xl[c + 1], s1);
+            s0 = fma(sP[r * kPadRow + c], __shfl_sync(full, xl, first + c), s0);
+            s1 = fma(sP[r * kPadRow + c + 1], __shfl_sync(full, xl, first + c + 1), s1);
         }
         x -= s0 + s1;
     }
-    if (Q != nullptr) {
-        const double *xr = which ? xr_v : xr_y;
+    if (has_q) {
         double s0 = 0.0, s1 = 0.0;
+#pragma unroll
         for (int c = 0; c < NW; c += 2) {
-            s0 = fma(Q[r * NW + c], xr[c], s0);
-            s1 = fma(Q[r * NW + c + 1], xr[c + 1], s1);
+            s0 = fma(sQ[r * kPadRow + c], __shfl_sync(full, xq, first + c), s0);
+            s1 = fma(sQ[r * kPadRow + c + 1], __shfl_sync(full, xq, first + c + 1), s1);
         }
         x -= s0 + s1;
     }
 #pragma unroll
     for (int rr = NW - 1; rr >= 0; --rr) {
-        const double lrr = Lk[rr * NW + rr];     // 1 / L_rr
-        const double lrq = Lk[rr * NW + r];      // L[rr][r] (r < rr)
-        const double xr = __shfl_sync(full, x * lrr, rr + NW * which);
+        const double lrr = sm[rr * NW + rr];     // 1 / L_rr
+        const double lrq = sm[rr * NW + r];      // L[rr][r] (r < rr)
+        const double xr = __shfl_sync(full, x * lrr, rr + first);
         if (r == rr) x = xr;
         else if (r < rr) x = fma(-lrq, xr, x);
     }
@@ -418,25 +616,30 @@ __device__ void lm_step(const Team &tm, const TrajDev &td, const double *z, cons
                         double *s_red, double *s_blk)
 {
     const int N = td.N, t = tm.tid(), nt = tm.nthreads();
-    const double h = z[0] / N, rho = td.rho;
-    // 1. f and df/dw at every grid point (16 forward-mode passes each)
+    const double h = quotient(z[0], N, td.inv_N), rho = td.rho;
+    // 1. f and df/dw at every grid point
     eval_f(tm, td, z, ws.f, ws.trig);
     team_sync();
-    for (int e = t; e < (N + 1) * NW; e += nt) {
-        const int k = e / NW, j = e - k * NW;
-        const double *w = z + 1 + (size_t)k * NW;
-        Dual x[NX], u[NU], out[NX];
-        for (int i = 0; i < NX; ++i) x[i] = {w[i], i == j ? 1.0 : 0.0};
-        for (int i = 0; i < NU; ++i) u[i] = {w[NX + i], NX + i == j ? 1.0 : 0.0};
-        traj_f<Dual>(td, x, u, out, ws.trig + (size_t)k * 10);
-        for (int i = 0; i < NF; ++i) ws.Fj[((size_t)k * NF + i) * NW + j] = out[NX - NF + i].d;
+    // a warp takes one seed at 32 grid points; the dear seeds (slew and swing angles, angles and
+    // rates of the arm) come first and the cheap ones in the reverse order, so that a warp that
+    // takes two has one of each
+    {
+        const unsigned long long order = 0xFCED6BA938721540ull;   // seed of place i: bits 4 i ..
+        const int groups = (N + 32) / 32, lane = threadIdx.x & 31;
+        for (int m = tm.warp(); m < NW * groups; m += tm.nwarps()) {
+            const int seed = (int)(order >> (4 * (m / groups))) & 15, k = 32 * (m % groups) + lane;
+            if (k <= N) {
+                double *F = ws.Fj + (size_t)k * NF * NW + seed;
+                swing_column(td, z + 1 + (size_t)k * NW, ws.trig + (size_t)k * 10, seed, F, F + NW);
+            }
+        }
     }
     // defect k: e_k = dd_k/dt_F = -(f_k + f_{k+1}) / (2N) and d_k + lam_k / rho
     for (int e = t; e < N * NX; e += nt) {
         const int k = e / NX, r = e - k * NX;
         const double *w0 = z + 1 + (size_t)k * NW;
         const double fs = ws.f[e] + ws.f[e + NX];
-        ws.er[e] = -fs / (2.0 * N);
+        ws.er[e] = quotient(-fs, 2.0 * N, td.inv_2N);
         ws.dr[e] = w0[NW + r] - w0[r] - 0.5 * h * fs + ws.lr[e];
     }
     team_sync();
@@ -449,7 +652,7 @@ __device__ void lm_step(const Team &tm, const TrajDev &td, const double *z, cons
     //   B_{k-1}^T B_{k-1} = I'^T I' - c (I'^T F_k + F_k^T I') + c^2 F_k^T F_k
     // (interior points take both, whose first-order terms cancel) and
     //   A_k^T B_k = -(I'^T I' - c I'^T F_{k+1} + c F_k^T I' - c^2 F_k^T F_{k+1}).
-    const double c = 0.5 * h;
+    const double c = 0.5 * h, cc = c * c;
     // one warp per grid point k: rows 10 and 11 of F_k and F_{k+1} staged in the warp's shared
     // memory, then the 136 lower entries of D_k and the 256 of E_k. Row r < 10 of F adds 1 to a
     // product's entry (r + 6, r + 6) and nothing elsewhere.
@@ -465,43 +668,49 @@ __device__ void lm_step(const Team &tm, const TrajDev &td, const double *z, cons
             for (int q = lane; q < 2 * NF * NW; q += 32)
                 sF[q] = (q < NF * NW || k < N) ? ws.Fj[(size_t)k * NF * NW + q] : 0.0;
             __syncwarp();
+            const bool end = k == 0 || k == N;
+            const double ck = k == 0 ? c : -c, s = end ? cc : 2.0 * cc;
             for (int e = lane; e < NW * (NW + 1) / 2; e += 32) {
                 int i, j;
                 tri_index(e, i, j);
                 const bool one = i == j && i >= 6;
-                const double f0 = fma(F0[i], F0[j], one && (i & 1) == 0 ? 1.0 : 0.0);        // even rows
-                const double f1 = fma(F0[NW + i], F0[NW + j], one && (i & 1) != 0 ? 1.0 : 0.0);   // odd rows
-                const double ff = f0 + f1;
-                const double cross = (i < NX ? Fent(F0, i, j) : 0.0) + (j < NX ? Fent(F0, j, i) : 0.0);
-                const double id = (i == j && i < NX) ? 1.0 : 0.0;
-                double v;
-                if (k == 0) v = id + c * cross + c * c * ff;
-                else if (k == N) v = id - c * cross + c * c * ff;
-                else v = 2.0 * id + 2.0 * c * c * ff;
-                v *= rho;
-                if (i == j) {
-                    if ((k == 0 || k == N) && i < NX) v += rho;                      // end states
-                    if (i < NX) {
-                        const double x = z[1 + (size_t)k * NW + i];
-                        if (x > td.x_max[i] || x < td.x_min[i]) v += td.rho_b;        // active bound
-                        if (i < 4 && k >= 1) v += 2.0 * td.omega_t;                   // tracking
-                    } else if (k >= 1) {
-                        v += 2.0 * td.omega_s * td.R[i - NX];                         // effort
-                    }
-                    v += mu * (v + 1e-9);                                             // damping
+                const double ff = fma(F0[i], F0[j], one && (i & 1) == 0 ? 1.0 : 0.0) +             // even rows
+                                  fma(F0[NW + i], F0[NW + j], one && (i & 1) != 0 ? 1.0 : 0.0);    // odd rows
+                double v = i == j && i < NX ? (end ? 1.0 : 2.0) : 0.0;
+                if (end) v = fma(ck, (i < NX ? Fent(F0, i, j) : 0.0) + (j < NX ? Fent(F0, j, i) : 0.0), v);
+                ws.D[(size_t)k * NW * NW + i * NW + j] = fma(s, ff, v) * rho;
+            }
+            __syncwarp();
+            if (lane < NW) {   // what only the diagonal has
+                const int i = lane;
+                double *d = &ws.D[(size_t)k * NW * NW + i * (NW + 1)], v = *d;
+                if (end && i < NX) v += rho;                                          // end states
+                if (i < NX) {
+                    const double x = z[1 + (size_t)k * NW + i];
+                    if (x > td.x_max[i] || x < td.x_min[i]) v += td.rho_b;        // active bound
+                    if (i < 4 && k >= 1) v += 2.0 * td.omega_t;                   // tracking
+                } else if (k >= 1) {
+                    v += 2.0 * td.omega_s * td.R[i - NX];                         // effort
                 }
-                ws.D[(size_t)k * NW * NW + i * NW + j] = v;
+                *d = v + mu * (v + 1e-9);                                         // damping
             }
             if (k < N)
-                for (int e = lane; e < NW * NW; e += 32) {
-                    const int i = e >> 4, j = e & (NW - 1);
-                    const bool one = i == j && i >= 6;
-                    const double p0 = fma(F0[i], F1[j], one && (i & 1) == 0 ? 1.0 : 0.0);
-                    const double p1 = fma(F0[NW + i], F1[NW + j], one && (i & 1) != 0 ? 1.0 : 0.0);
-                    const double id = (i == j && i < NX) ? 1.0 : 0.0;
-                    const double v = id - c * (i < NX ? Fent(F1, i, j) : 0.0) + c * (j < NX ? Fent(F0, j, i) : 0.0) -
-                                     c * c * (p0 + p1);
-                    ws.E[(size_t)k * NW * NW + e] = -rho * v;
+#pragma unroll
+                for (int q = 0; q < NW * NW / 32; ++q) {
+                    const int e = q * 32 + lane, i = e >> 4, j = e & (NW - 1);
+                    const bool one = i == j && i >= 6, dense = q == (NX - NF) / 2;   // rows 10 and 11
+                    const double p = fma(F0[i], F1[j], one && (i & 1) == 0 ? 1.0 : 0.0) +
+                                     fma(F0[NW + i], F1[NW + j], one && (i & 1) != 0 ? 1.0 : 0.0);
+                    // I'^T I' - c I'^T F_(k+1) + c F_k^T I': ones of the constant rows by selection
+                    const bool below = i == j + 6 && j < NX - NF;
+                    double v = i == j && i < NX ? 1.0 : (j == i + 6 && i < NX - NF ? -c : (below ? c : 0.0));
+                    if (dense) {
+                        v = fma(-c, F1[(lane >> 4) * NW + j], i == j ? 1.0 : 0.0);
+                        if (below) v += c;
+                    }
+                    if (j == NX - 2 || j == NX - 1) v = fma(c, F0[(j - (NX - NF)) * NW + i], v);
+                    v = -rho * fma(-cc, p, v);
+                    ws.E[(size_t)k * NW * NW + e] = v;
                 }
         }
     }
@@ -546,18 +755,18 @@ __device__ void lm_step(const Team &tm, const TrajDev &td, const double *z, cons
         ws.g[e] = -gv;
     }
     // the t_F corner and gradient
-    double cc = 0.0, gt = 0.0;
+    double ct = 0.0, gt = 0.0;
     for (int e = tm.sum_first(N * NX); e < N * NX; e += tm.sum_stride()) {
         const double ev = ws.er[e];
-        cc += ev * ev;
+        ct += ev * ev;
         gt += ev * ws.dr[e];
     }
     {
-        const double2 sums = team_sum2(cc, gt, s_red);   // also orders D, E, bb, g before the solve
-        cc = rho * sums.x;
+        const double2 sums = team_sum2(ct, gt, s_red);   // also orders D, E, bb, g before the solve
+        ct = rho * sums.x;
         gt = 1.0 + rho * sums.y;
     }
-    cc += mu * (cc + 1e-9);
+    ct += mu * (ct + 1e-9);
     // 3. the tridiagonal part T (diagonal blocks D_k, couplings T[k][k+1] = E_k) solved for the
     //    two right-hand sides b (into y, ws.bb) and -g (into v, ws.g) by block cyclic reduction.
     //    Level s = 1, 2, 4, ... eliminates the blocks k = s, 3s, 5s, ... <= N, each between
@@ -647,23 +856,33 @@ __device__ void lm_step(const Team &tm, const TrajDev &td, const double *z, cons
         }
         team_sync();
     }
-    // block 0: D_0 x_0 = f_0
+    // block 0: D_0 x_0 = f_0; then the eliminated blocks, from the last level to the first. Each
+    // warp stages its first block of the next level before the barrier.
+    auto stage_level = [&](int s, int m) {
+        const int n_odd = (N / s + 1) / 2;
+        if (m >= n_odd) return;
+        const int k = (2 * m + 1) * s;
+        stage_back(Fw, ws.D + (size_t)k * NW * NW, ws.P + (size_t)k * NW * NW,
+                   k + s <= N ? ws.E + (size_t)k * NW * NW : nullptr, lane);
+    };
     if (warp == 0) {
         warp_eliminate16(ws.D, nullptr, nullptr, nullptr, ws.bb, ws.g, lane);
-        warp_back16(ws.D, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, ws.bb, ws.g, lane);
+        stage_back(Fw, ws.D, nullptr, nullptr, lane);
+        warp_back16(Fw, false, nullptr, nullptr, false, nullptr, nullptr, ws.bb, ws.g, lane);
     }
+    stage_level(s_top, warp);
     team_sync();
-    // the eliminated blocks, from the last level to the first
     for (int s = s_top; s >= 1; s >>= 1) {
         const int n_odd = (N / s + 1) / 2;
         for (int m = warp; m < n_odd; m += n_warps) {
             const int k = (2 * m + 1) * s, l = k - s, r = k + s;
             const bool has_r = r <= N;
-            warp_back16(ws.D + (size_t)k * NW * NW, ws.P + (size_t)k * NW * NW, ws.bb + (size_t)l * NW,
-                        ws.g + (size_t)l * NW, has_r ? ws.E + (size_t)k * NW * NW : nullptr,
-                        has_r ? ws.bb + (size_t)r * NW : nullptr, has_r ? ws.g + (size_t)r * NW : nullptr,
+            if (m != warp) stage_level(s, m);
+            warp_back16(Fw, true, ws.bb + (size_t)l * NW, ws.g + (size_t)l * NW, has_r,
+                        ws.bb + (size_t)(has_r ? r : 0) * NW, ws.g + (size_t)(has_r ? r : 0) * NW,
                         ws.bb + (size_t)k * NW, ws.g + (size_t)k * NW, lane);
         }
+        if (s > 1) stage_level(s >> 1, warp);
         team_sync();
     }
     // 4. the border: dt = (-g_t - b^T v) / (c - b^T y), dw = v - y dt, with y = T^-1 b and
@@ -677,7 +896,7 @@ __device__ void lm_step(const Team &tm, const TrajDev &td, const double *z, cons
     const double2 sums = team_sum2(by, bv, s_red);
     by = sums.x;
     bv = sums.y;
-    const double dt = (-gt - bv) / (cc - by);
+    const double dt = (-gt - bv) / (ct - by);
     const int d0 = dz_local ? (int)threadIdx.x : t, dn = dz_local ? (int)blockDim.x : nt;
     if (d0 == 0) dz[0] = dt;
     for (int e = d0; e < (N + 1) * NW; e += dn) dz[1 + e] = ws.g[e] - ws.bb[e] * dt;
@@ -756,7 +975,7 @@ k_traj_solve(const TrajDev td, const double *q_star, double *z_io, double *ws_ba
             if (Fn < F) {
                 for (int i = t; i < n_var; i += blockDim.x) z[i] = zn[i];
                 F = Fn;
-                mu = fmax(mu / 3.0, 1e-12);
+                mu = fmax(quotient(mu, 3.0, 1.0 / 3.0), 1e-12);
             } else {
                 mu = fmin(mu * 4.0, 1e12);
             }
@@ -765,7 +984,7 @@ k_traj_solve(const TrajDev td, const double *q_star, double *z_io, double *ws_ba
         // multipliers: lam += rho c(z)
         eval_f(tm, td, z, ws.f);
         team_sync();
-        const double h = z[0] / N;
+        const double h = quotient(z[0], N, td.inv_N);
         for (int e = tm.tid(); e < n_eq; e += tm.nthreads()) {
             const int k = e / NX, i = e - k * NX;
             double c;
@@ -785,7 +1004,7 @@ k_traj_solve(const TrajDev td, const double *q_star, double *z_io, double *ws_ba
     eval_f(tm, td, z, ws.f);
     team_sync();
     double cmax = 0.0, vmax = 0.0;
-    const double h = z[0] / N;
+    const double h = quotient(z[0], N, td.inv_N);
     for (int e = t; e < n_eq; e += blockDim.x) {
         const int k = e / NX, i = e - k * NX;
         double c;
@@ -977,6 +1196,8 @@ int cp_traj_init(const cp_model *model, const cp_traj_params *tp, int32_t max_pa
     d.N = tp->N;
     d.outer = tp->outer;
     d.inner = tp->inner;
+    d.inv_N = 1.0 / tp->N;
+    d.inv_2N = 1.0 / (2.0 * tp->N);
     t->max_paths = max_paths;
     t->ws_stride = (traj_ws_doubles(tp->N) + 31) & ~(size_t)31;
     const size_t n_eq = (size_t)NX * (tp->N + 2);
