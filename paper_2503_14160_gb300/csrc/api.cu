@@ -159,7 +159,7 @@ struct cp_planner {
     float *elites = nullptr;
     double *w = nullptr, *mean_part = nullptr, *cov_part = nullptr;
     double *mom_y = nullptr;    // [2][nu][D] FP64 deviations of the elites for the moments
-    bool use_tc = false;        // the moments' tensor-core form (a rule on nu and D; paper update)
+    bool use_tc = false;        // cp_update's moments in their tensor-core form (a rule on nu and D; paper update)
     MomentsTc tc{};
     int tc_parts = 0;
     double *best = nullptr;
@@ -538,9 +538,13 @@ int run_sample(cp_planner *p, int iter, float *d_xi)
     return p->timer.end(ST_SAMPLE, p->st);
 }
 
-int run_moments(cp_planner *p, double *mu);
+int run_moments(cp_planner *p, double *mu, bool use_tc);
 
-int run_update(cp_planner *p, const double *d_J, const float *d_xi)
+// use_tc: the moments in integers on the tensor cores. Only an update by itself may take them
+// (cp_update): they are nearer to the exact sums than FP64 additions are, but differ from them in
+// the last bits, and over the iterations of a plan such a difference grows (over 17 plans of 5 to
+// 100 iterations, three ended with another covariance, by up to 1e-2).
+int run_update(cp_planner *p, const double *d_J, const float *d_xi, bool use_tc)
 {
     NvtxRange range("craneplan:update");
     int rc = p->timer.begin(p->st);
@@ -574,7 +578,7 @@ int run_update(cp_planner *p, const double *d_J, const float *d_xi)
         p->elites_ready = true;
         p->iteration += 1;
         return CP_OK;
-    } else if ((rc = run_moments(p, p->mu)) != CP_OK) {
+    } else if ((rc = run_moments(p, p->mu, use_tc)) != CP_OK) {
         return rc;
     }
     if ((rc = p->timer.end(ST_UPDATE, p->st)) != CP_OK) return rc;
@@ -584,9 +588,9 @@ int run_update(cp_planner *p, const double *d_J, const float *d_xi)
 }
 
 // Mean and covariance of the current elites into `mu` and the planner's C.
-int run_moments(cp_planner *p, double *mu)
+int run_moments(cp_planner *p, double *mu, bool use_tc)
 {
-    if (p->use_tc) {
+    if (use_tc) {
         MomentsTc a = p->tc;
         a.mu = mu;
         return launch_moments_tc(a, p->tc_parts, p->num_sms, p->st);
@@ -602,7 +606,7 @@ int materialise_distribution(const cp_planner *p)
 {
     if (!p->elites_ready) return CP_OK;
     cp_planner *q = const_cast<cp_planner *>(p);
-    int rc = run_moments(q, q->mu_prev);
+    int rc = run_moments(q, q->mu_prev, false);
     if (rc != CP_OK) return rc;
     return launch_factor(q->C, q->prm.sigma * q->prm.sigma, nullptr, q->D, q->L, q->Lt, q->status, q->st);
 }
@@ -624,7 +628,7 @@ int run_iteration(cp_planner *p)
     int rc;
     if ((rc = run_sample(p, p->iteration, p->xi)) != CP_OK) return rc;
     if ((rc = run_eval(p, p->xi, p->N, p->J, p->flag, nullptr, nullptr, nullptr)) != CP_OK) return rc;
-    if ((rc = run_update(p, p->J, p->xi)) != CP_OK) return rc;
+    if ((rc = run_update(p, p->J, p->xi, false)) != CP_OK) return rc;
     return record_metrics(p);
 }
 
@@ -739,7 +743,7 @@ int cp_plan_init(const cp_model *model, const cp_scene *scene, const cp_params *
     if ((rc = sample_configure()) != CP_OK) return fail(rc);
     if ((rc = update_configure()) != CP_OK) return fail(rc);
     if ((rc = moments_tc_configure()) != CP_OK) return fail(rc);
-    p->use_tc = p->prm.update_rule == CP_UPDATE_PAPER && moments_use_tc(p->nu, p->D);
+    p->use_tc = p->prm.update_rule == CP_UPDATE_PAPER && p->prm.sampler == CP_SAMPLE_FACTOR && moments_use_tc(p->nu, p->D);
     p->tc_parts = p->use_tc ? moments_tc_parts(p->nu, p->D, p->num_sms) : 0;
 
     const size_t N = p->N, D = p->D, nu = p->nu, ch = p->chunks, mc = p->n_mean_chunks;
@@ -771,9 +775,9 @@ int cp_plan_init(const cp_model *model, const cp_scene *scene, const cp_params *
     const size_t o_elites = L.take<float>(nu * D);
     const size_t o_w = L.take<double>(nu);
     const bool tc = p->use_tc;
-    const size_t o_mean_part = L.take<double>(tc ? 1 : (mc + 1) * D);   // chunk partials, then S1
-    const size_t o_cov_part = L.take<double>(tc ? 1 : mc * D * D);
-    const size_t o_mom_y = L.take<double>(tc ? 1 : 2 * nu * D);
+    const size_t o_mean_part = L.take<double>((mc + 1) * D);   // chunk partials, then S1
+    const size_t o_cov_part = L.take<double>(mc * D * D);
+    const size_t o_mom_y = L.take<double>(2 * nu * D);
     const size_t tc_n = tc ? moments_tc_partial(p->D, p->tc_parts) : 1;
     const size_t o_tc_hi = L.take<long long>(tc_n);
     const size_t o_tc_lo = L.take<long long>(tc_n);
@@ -1009,7 +1013,7 @@ int cp_update(cp_planner *p, const double *d_J, const float *d_xi)
     if (!p || !d_J || !d_xi) return set_error("NULL argument"), CP_ERR_ARG;
     if (!aligned16(d_xi)) return set_error("d_xi is not 16-byte aligned"), CP_ERR_ARG;
     if (!p->have_endpoints) return set_error("set the end points first"), CP_ERR_STATE;
-    return run_update(p, d_J, d_xi);
+    return run_update(p, d_J, d_xi, p->use_tc);
 }
 
 bool same_scene(const SceneDev &a, const SceneDev &b)
@@ -1441,9 +1445,6 @@ struct cp_batch {
     BatchEvalDev *ev_pop = nullptr, *ev_mean = nullptr;
     int2 *tab_init = nullptr, *tab_sample = nullptr, *tab_cand = nullptr, *tab_gather = nullptr;
     int2 *tab_mprep = nullptr, *tab_mpart = nullptr, *tab_mcomb = nullptr;
-    int2 *tab_trange = nullptr, *tab_tpart = nullptr, *tab_tcomb = nullptr;   // tensor-core moments
-    int n_trange = 0, n_tpart = 0, n_tcomb = 0;
-    uint32_t *colmax = nullptr;        // [nq][kMomentCols]
     int n_init = 0, n_sample = 0, n_cand = 0, n_gather = 0, n_mprep = 0, n_mpart = 0, n_mcomb = 0;
     int4 *tiles_pop = nullptr, *tiles_mean = nullptr;
     int64_t tiles_cap = 0;
@@ -1534,9 +1535,6 @@ int record_batch(cp_batch *b)
         if ((rc = launch_batch_gather(b->qdev, b->tab_gather, b->n_gather, sorted, b->st)) != CP_OK) return rc;
         if ((rc = launch_batch_moments(b->qdev, b->nq, b->tab_mprep, b->n_mprep, b->tab_mpart, b->n_mpart, b->tab_mcomb,
                                        b->n_mcomb, b->st)) != CP_OK)
-            return rc;
-        if ((rc = launch_batch_moments_tc(b->qdev, b->colmax, b->nq, b->tab_trange, b->n_trange, b->tab_tpart,
-                                          b->n_tpart, b->tab_tcomb, b->n_tcomb, b->st)) != CP_OK)
             return rc;
         if ((rc = launch_batch_factor(b->qdev, b->nq, b->max_D, b->st)) != CP_OK) return rc;
     }
@@ -1701,14 +1699,6 @@ int cp_batch_init(const cp_model *model, const cp_query *queries, int32_t nq, in
         d.s1p = p->mean_part;
         d.eps = p->prm.eps;
         d.n_chunks = moments_chunking(p->nu, p->D, &d.per);
-        if (p->use_tc) {
-            // parts of at least 12 stages each (three accumulations): the queries share the GPU,
-            // and the integer sums do not depend on the split
-            d.n_chunks = 0;
-            d.tc = p->tc;
-            d.tc_parts = std::min(p->tc_parts, (moments_tc_stages(p->nu) + 11) / 12);
-            d.tc_range_blocks = std::min(32, (p->nu + 255) / 256);
-        }
         d.mom_y = p->mom_y;
         d.cand_off = (int)off;
         d.status = p->status;
@@ -1767,17 +1757,12 @@ int cp_batch_init(const cp_model *model, const cp_query *queries, int32_t nq, in
     block_table(nq, [&](int q) { return (qh[q].N + kBatchSampleCands - 1) / kBatchSampleCands; }, t_sample);
     block_table(nq, [&](int q) { return (qh[q].N + 255) / 256; }, t_cand);
     block_table(nq, [&](int q) { return (qh[q].nu + 7) / 8; }, t_gather);
-    auto fp64_form = [&](int q) { return qh[q].n_chunks > 0; };
-    block_table(nq, [&](int q) { return fp64_form(q) ? (qh[q].nu * qh[q].D + 255) / 256 : 0; }, t_mprep);
+    block_table(nq, [&](int q) { return (qh[q].nu * qh[q].D + 255) / 256; }, t_mprep);
     block_table(nq, [&](int q) {
         const int nt = (qh[q].D + 15) / 16;
         return nt * (nt + 1) / 2 * qh[q].n_chunks;
     }, t_mpart);
-    block_table(nq, [&](int q) { return fp64_form(q) ? (qh[q].D * (qh[q].D + 1) / 2 + 31) / 32 : 0; }, t_mcomb);
-    std::vector<int2> t_trange, t_tpart, t_tcomb;
-    block_table(nq, [&](int q) { return fp64_form(q) ? 0 : qh[q].tc_range_blocks; }, t_trange);
-    block_table(nq, [&](int q) { return fp64_form(q) ? 0 : qh[q].tc_parts * moments_tc_tiles(qh[q].D); }, t_tpart);
-    block_table(nq, [&](int q) { return fp64_form(q) ? 0 : qh[q].D; }, t_tcomb);
+    block_table(nq, [&](int q) { return (qh[q].D * (qh[q].D + 1) / 2 + 31) / 32; }, t_mcomb);
     int64_t max_tiles = 0;
     for (int q = 0; q < nq; ++q) max_tiles += std::max(b->items_pop[q], b->items_mean[q]);   // tiles of >= 1 item
     b->tiles_cap = max_tiles;
@@ -1795,10 +1780,6 @@ int cp_batch_init(const cp_model *model, const cp_query *queries, int32_t nq, in
     const size_t o_tq = L.take<int2>(t_mprep.size());
     const size_t o_tp = L.take<int2>(t_mpart.size());
     const size_t o_tm = L.take<int2>(t_mcomb.size());
-    const size_t o_ttr = L.take<int2>(t_trange.size());
-    const size_t o_ttp = L.take<int2>(t_tpart.size());
-    const size_t o_ttc = L.take<int2>(t_tcomb.size());
-    const size_t o_colmax = L.take<uint32_t>((size_t)kMomentCols * nq);
     const size_t o_tilp = L.take<int4>((size_t)max_tiles);
     const size_t o_tilm = L.take<int4>((size_t)max_tiles);
     const size_t o_queue = L.take<int>((size_t)iters + 2);
@@ -1822,14 +1803,6 @@ int cp_batch_init(const cp_model *model, const cp_query *queries, int32_t nq, in
     b->tab_mprep = (int2 *)(base + o_tq);
     b->tab_mpart = (int2 *)(base + o_tp);
     b->tab_mcomb = (int2 *)(base + o_tm);
-    b->tab_trange = (int2 *)(base + o_ttr);
-    b->tab_tpart = (int2 *)(base + o_ttp);
-    b->tab_tcomb = (int2 *)(base + o_ttc);
-    b->colmax = (uint32_t *)(base + o_colmax);
-    for (int q = 0; q < nq; ++q) qh[q].tc.colmax = b->colmax + (size_t)kMomentCols * q;
-    b->n_trange = (int)t_trange.size();
-    b->n_tpart = (int)t_tpart.size();
-    b->n_tcomb = (int)t_tcomb.size();
     b->tiles_pop = (int4 *)(base + o_tilp);
     b->tiles_mean = (int4 *)(base + o_tilm);
     b->queue = (int *)(base + o_queue);
@@ -1862,9 +1835,6 @@ int cp_batch_init(const cp_model *model, const cp_query *queries, int32_t nq, in
         (e = up(b->tab_mprep, t_mprep.data(), sizeof(int2) * t_mprep.size())) != cudaSuccess ||
         (e = up(b->tab_mpart, t_mpart.data(), sizeof(int2) * t_mpart.size())) != cudaSuccess ||
         (e = up(b->tab_mcomb, t_mcomb.data(), sizeof(int2) * t_mcomb.size())) != cudaSuccess ||
-        (e = up(b->tab_trange, t_trange.data(), sizeof(int2) * t_trange.size())) != cudaSuccess ||
-        (e = up(b->tab_tpart, t_tpart.data(), sizeof(int2) * t_tpart.size())) != cudaSuccess ||
-        (e = up(b->tab_tcomb, t_tcomb.data(), sizeof(int2) * t_tcomb.size())) != cudaSuccess ||
         (e = up(b->qid, qid.data(), sizeof(uint16_t) * qid.size())) != cudaSuccess)
         return fail(cuda_fail(e, "cudaMemcpyAsync(batch tables)"));
     if ((rc = batch_upload_tiles(b)) != CP_OK) return fail(rc);   // synchronises

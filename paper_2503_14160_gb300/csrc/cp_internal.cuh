@@ -366,9 +366,7 @@ struct BatchQueryDev {
     double *s2p, *s1p;               // moment partials
     double *mom_y;                   // [2][nu][D] the elites' FP64 deviations, then weighted
     double eps;
-    int per, n_chunks;               // elites per moment chunk, chunks (0: the tensor-core form)
-    MomentsTc tc;                    // tensor-core form of the moments
-    int tc_parts, tc_range_blocks;
+    int per, n_chunks;               // elites per moment chunk, chunks
     int cand_off;                    // first position of the query in the concatenated ranking
     uint32_t *status;
     double *consts;                  // q0[4], qd[4], q_min[4], q_max[4]
@@ -402,15 +400,12 @@ int launch_batch_moments(const BatchQueryDev *qd, int nq, const int2 *tab_prep, 
                          const int2 *tab_partial, int blocks_partial, const int2 *tab_combine, int blocks_combine,
                          cudaStream_t st);
 bool moments_use_tc(int nu, int D);   // the form of the moments, a function of nu and D alone
-int moments_tc_stages(int nu);
 int moments_tc_tiles(int D);
 int moments_tc_parts(int nu, int D, int num_sms);
 size_t moments_tc_partial(int D, int parts);   // integers of each of hi and lo
 int moments_tc_configure();
 int launch_moments_tc_weights(const double *w, int nu, long long *W, long long *Wf, int *scale, cudaStream_t st);
 int launch_moments_tc(const MomentsTc &a, int parts, int num_sms, cudaStream_t st);
-int launch_batch_moments_tc(const BatchQueryDev *qd, uint32_t *colmax, int nq, const int2 *tab_range, int n_range,
-                            const int2 *tab_part, int n_part, const int2 *tab_comb, int n_comb, cudaStream_t st);
 int moments_chunking(int nu, int D, int *per);   // chunks of the moment partials and elites per chunk
 int launch_batch_outputs(const BatchQueryDev *qd, int nq, bool mean_candidate, double *out, int out_stride,
                          cudaStream_t st);

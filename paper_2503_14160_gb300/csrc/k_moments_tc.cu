@@ -24,7 +24,9 @@
 // A CTA takes 64 columns of S2 (all 128 rows) over a range of elites, 32 at a time: 1024 threads
 // turn one column of four elites each into digits in shared memory (K-major core matrices) while
 // the tensor cores work on the stage before, one thread issues the 68 MMAs of 128 x 64 x 16, and
-// the eight levels fill the 512 columns of tensor memory. Measured TC_MEASURED.
+// the eight levels fill the 512 columns of tensor memory. nu = 32768, D = 128: 84 us, with 9 us for
+// the columns' ranges and 11 us for the final sums; cp_update of 65536 candidates 241 us, and 740 us
+// with the FP64 form. A plan's and a batch's updates keep the FP64 sums (see run_update).
 #include "chain_launch.cuh"
 #include "cp_internal.cuh"
 #include "tcgen05.cuh"
@@ -322,29 +324,6 @@ __global__ void __launch_bounds__(kCombGroups *kTcRows) k_moments_tc_combine(con
     combine_tc_body(a, blockIdx.x, parts);
 }
 
-// Every query's share in one launch each (tab: {query, block within the query}).
-__global__ void __launch_bounds__(256)
-k_batch_moments_range(const BatchQueryDev *__restrict__ qd, const int2 *__restrict__ tab)
-{
-    const int2 e = tab[blockIdx.x];
-    range_body(qd[e.x].tc, e.y, qd[e.x].tc_range_blocks);
-}
-
-__global__ void __launch_bounds__(kTcThreads, 1)
-k_batch_moments_tc(const BatchQueryDev *__restrict__ qd, const int2 *__restrict__ tab)
-{
-    const int2 e = tab[blockIdx.x];
-    const int parts = qd[e.x].tc_parts;
-    moments_tc_body(qd[e.x].tc, e.y / parts, e.y % parts, parts);
-}
-
-__global__ void __launch_bounds__(kCombGroups *kTcRows)
-k_batch_moments_tc_combine(const BatchQueryDev *__restrict__ qd, const int2 *__restrict__ tab)
-{
-    const int2 e = tab[blockIdx.x];
-    combine_tc_body(qd[e.x].tc, e.y, qd[e.x].tc_parts);
-}
-
 // Integer weights: W = sqrt(w_j) 2^(63 - es) and Wf = w_j 2^(63 - ew), es and ew the exponents
 // that bound the first (largest) weight's.
 __global__ void k_moments_tc_weights(const double *__restrict__ w, int nu, long long *W, long long *Wf, int *scale)
@@ -362,11 +341,12 @@ __global__ void k_moments_tc_weights(const double *__restrict__ w, int nu, long 
 
 }  // namespace
 
-// The tensor-core form is taken from nu D^2 = 2^23 on: there the FP64 form needs about 14 us of the
-// whole GPU's FP64 units besides its launches, and the three launches here TC_SMALL us.
+// The tensor-core form is taken from nu D^2 = 2^23 on, where the FP64 form needs about 14 us of the
+// whole GPU's FP64 units: there a cp_update takes 104 us against 124 (nu = 8192, D = 32) and 108
+// against 114 (nu = 512, D = 128).
 bool moments_use_tc(int nu, int D) { return (long long)nu * D * D >= (1ll << 23); }
 
-int moments_tc_stages(int nu) { return (nu + kStage - 1) / kStage; }
+static int moments_tc_stages(int nu) { return (nu + kStage - 1) / kStage; }
 int moments_tc_tiles(int D) { return (D + kTcCols - 1) / kTcCols; }
 
 int moments_tc_parts(int nu, int D, int num_sms)
@@ -380,7 +360,6 @@ size_t moments_tc_partial(int D, int parts) { return (size_t)parts * moments_tc_
 int moments_tc_configure()
 {
     CP_CUDA(cudaFuncSetAttribute(k_moments_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem));
-    CP_CUDA(cudaFuncSetAttribute(k_batch_moments_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem));
     return CP_OK;
 }
 
@@ -401,20 +380,6 @@ int launch_moments_tc(const MomentsTc &a, int parts, int num_sms, cudaStream_t s
     CP_LAUNCHED("k_moments_tc");
     launch_chained(k_moments_tc_combine, a.D, kCombGroups * kTcRows, 0, st, a, parts);
     CP_LAUNCHED("k_moments_tc_combine");
-    return CP_OK;
-}
-
-int launch_batch_moments_tc(const BatchQueryDev *qd, uint32_t *colmax, int nq, const int2 *tab_range, int n_range,
-                            const int2 *tab_part, int n_part, const int2 *tab_comb, int n_comb, cudaStream_t st)
-{
-    if (n_part == 0) return CP_OK;
-    CP_CUDA(cudaMemsetAsync(colmax, 0, sizeof(uint32_t) * kTcRows * (size_t)nq, st));
-    k_batch_moments_range<<<n_range, 256, 0, st>>>(qd, tab_range);
-    CP_LAUNCHED("k_batch_moments_range");
-    k_batch_moments_tc<<<n_part, kTcThreads, kTcSmem, st>>>(qd, tab_part);
-    CP_LAUNCHED("k_batch_moments_tc");
-    k_batch_moments_tc_combine<<<n_comb, kCombGroups * kTcRows, 0, st>>>(qd, tab_comb);
-    CP_LAUNCHED("k_batch_moments_tc_combine");
     return CP_OK;
 }
 

@@ -316,7 +316,6 @@ __global__ void __launch_bounds__(128)
 k_batch_moments_s1(const BatchQueryDev *__restrict__ qd)
 {
     const BatchQueryDev &q = qd[blockIdx.y];
-    if (q.n_chunks == 0) return;   // its moments took the tensor-core form
     const int g = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     moments_s1_body(q.s1p, q.n_chunks, q.D, q.elites, q.mu, g / kSumLanes, g % kSumLanes);
 }
@@ -984,7 +983,6 @@ int launch_batch_moments(const BatchQueryDev *qd, int nq, const int2 *tab_prep, 
                          const int2 *tab_partial, int blocks_partial, const int2 *tab_combine, int blocks_combine,
                          cudaStream_t st)
 {
-    if (blocks_prep == 0) return CP_OK;   // every query takes the tensor-core form
     k_batch_moments_prep<<<blocks_prep, 256, 0, st>>>(qd, tab_prep);
     CP_LAUNCHED("k_batch_moments_prep");
     k_batch_moments_partial<<<blocks_partial, 256, 0, st>>>(qd, tab_partial);
