@@ -112,19 +112,48 @@ constexpr int kSampleThreads = 32 * kSampleWarps;
 constexpr int kSampleCands = 8;   // candidates a warp draws at a time
 
 // Shared memory of the sampler: L^T (FP32, column-major, D x D, plus a pad of 32 floats read
-// by the lanes past the last row) and per warp the normals of its kSampleCands candidates
-// ([D][kSampleCands], candidate fastest).
+// by the lanes past the last row), the mean's rows as MeanRow and per warp the normals of its
+// kSampleCands candidates ([D][kSampleCands], candidate fastest).
 size_t sample_smem(int K)
 {
     const size_t D = 4 * (size_t)K;
-    return sizeof(float) * (D * D + 32 + (size_t)kSampleWarps * kSampleCands * D);
+    return sizeof(float) * (D * D + 32 + 4 * D + (size_t)kSampleWarps * kSampleCands * D);
 }
+
+// A row of the mean for sum_rounded: m = hi + lo + r, |r| <= 2^-48 |m| + 2^-150 < slack / 2.
+struct __align__(16) MeanRow {
+    float hi, lo, slack, pad;
+};
+
+__device__ __forceinline__ MeanRow mean_row(double m)
+{
+    const float hi = (float)m;
+    return {hi, (float)(m - (double)hi), fmaxf(fabsf(hi) * 0x1p-46f, 0x1p-140f), 0.f};
+}
+
+// float(m + a), the sum rounded to FP64 and then to FP32, in FP32: s + e = hi + a exactly (Knuth's
+// two-sum), t = e + lo, and the true sum lies in s + t -+ d, d covering the roundings of t, lo, the
+// bracket's own and the FP64 sum's (2^-53 |sum|, below 2^-22 |t| wherever t reaches half an FP32
+// step). Rounding is monotone, so where both ends round to one float that is the result; else
+// (a sum within 2^-22 of a tie, infinities, NaN) false.
+__device__ __forceinline__ bool sum_rounded(const MeanRow &m, float a, float &x)
+{
+    const float s = __fadd_rn(m.hi, a), b = __fadd_rn(s, -m.hi);
+    const float e = __fadd_rn(__fadd_rn(m.hi, -__fadd_rn(s, -b)), __fadd_rn(a, -b));
+    const float t = __fadd_rn(e, m.lo), d = __fmaf_rn(fabsf(t), 0x1p-22f, m.slack);
+    x = __fadd_rn(s, __fadd_rn(t, d));
+    return x == __fadd_rn(s, __fadd_rn(t, -d));
+}
+
+__device__ __noinline__ float sum_fp64(const double *mu, int r, float a) { return (float)(mu[r] + (double)a); }
 
 // Warp w draws the candidates g .. g + 7 of the groups g = g0 + 8 w, g0 + 8 w + g_stride, ...
 // below i_end: their normals (Philox counter (j, i, iter, query) for z[4j..4j+3], spread over
 // the lanes) go to the warp's buffer; then, 32 rows at a time, lane l holds row r = r0 + l of
 // all eight and forms acc = sum_c L[r][c] z[c] over ascending c with one FMA per term (L read
-// once for the eight), and writes xi_r = mu_r + acc (added in FP64, rounded once to FP32).
+// once for the eight), and writes xi_r = mu_r + acc (added in FP64, rounded once to FP32: by
+// sum_rounded, as the conversion, the addition and the conversion back hold the scheduler's FP64
+// unit for 205 cycles per 32 entries, 46 of the kernel's 104 us at N = 65536, D = 128; now 90).
 // Columns past the block's last row hold zeros of L for every row of the block and are
 // skipped; adding 0 z leaves a nonzero sum unchanged, so each row equals the full D-term sum.
 __device__ __forceinline__ void sample_body(const double *__restrict__ mu, const float *__restrict__ Lt, int K,
@@ -134,9 +163,11 @@ __device__ __forceinline__ void sample_body(const double *__restrict__ mu, const
     const int D = 4 * K;
     float *sL = sm;
     const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float *sZ = sm + D * D + 32 + wib * kSampleCands * D;
+    MeanRow *sM = reinterpret_cast<MeanRow *>(sm + D * D + 32);
+    float *sZ = sm + D * D + 32 + 4 * D + wib * kSampleCands * D;
     for (int idx = threadIdx.x; idx < D * D; idx += blockDim.x) sL[idx] = Lt[idx];
     if (threadIdx.x < 32) sL[D * D + threadIdx.x] = 0.f;
+    for (int r = threadIdx.x; r < D; r += blockDim.x) sM[r] = mean_row(mu[r]);
     __syncthreads();
     for (int g = g0 + kSampleCands * wib; g < i_end; g += g_stride) {
         for (int pq = lane; pq < kSampleCands * K; pq += 32) {
@@ -174,10 +205,17 @@ __device__ __forceinline__ void sample_body(const double *__restrict__ mu, const
                 acc[7] = fmaf(l, zb.w, acc[7]);
             }
             if (r < D) {
-                const double m = mu[r];
+                const MeanRow m = sM[r];
+                bool ok = true;
+                float x[kSampleCands];
+#pragma unroll
+                for (int q = 0; q < kSampleCands; ++q) ok = sum_rounded(m, acc[q], x[q]) && ok;
+                if (!ok)
+#pragma unroll
+                    for (int q = 0; q < kSampleCands; ++q) x[q] = sum_fp64(mu, r, acc[q]);
 #pragma unroll
                 for (int q = 0; q < kSampleCands; ++q)
-                    if (g + q < i_end) xi[(size_t)(g + q) * D + r] = (float)(m + (double)acc[q]);
+                    if (g + q < i_end) xi[(size_t)(g + q) * D + r] = x[q];
             }
         }
         __syncwarp();

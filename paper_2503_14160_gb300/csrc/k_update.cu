@@ -120,7 +120,10 @@ __device__ __forceinline__ void moments_partial_body(const double *__restrict__ 
     const int tc = t;
     const bool diag = tr == tc;
     // the thread's entry (a, b) of the tile: all 256 of an off-diagonal tile; the 136 with
-    // b <= a of a diagonal tile (warps 5-7 idle there)
+    // b <= a of a diagonal tile, where half a further warp sums the first moments of the 16 rows.
+    // (On the lanes with b = 0 those sums took an FP64 instruction of four warps per elite, after
+    // the products: at nu = 32768, D = 128 the launch took 544 us, and takes 489.)
+    constexpr int kS1Thread = 160;
     int a = threadIdx.x >> 4, b = threadIdx.x & 15;
     const bool active = !diag || threadIdx.x < 136;
     if (diag && active) tri_index(threadIdx.x, a, b);
@@ -148,13 +151,16 @@ __device__ __forceinline__ void moments_partial_body(const double *__restrict__ 
                 a3 = fma(wyr[j + 3][a], yc[j + 3][b], a3);
             }
             for (; j < cnt; ++j) a0 = fma(wyr[j][a], yc[j][b], a0);
-            if (diag && b == 0)
-                for (int j = 0; j < cnt; ++j) acc1 += wyr[j][a];
+        } else if (threadIdx.x >= kS1Thread && threadIdx.x < kS1Thread + 16) {
+            for (int j = 0; j < cnt; ++j) acc1 += wyr[j][threadIdx.x - kS1Thread];
         }
     }
     const int r = tr * 16 + a, c = tc * 16 + b;
     if (active && r < D && c <= r) s2p[(size_t)p * D * D + (size_t)r * D + c] = (a0 + a1) + (a2 + a3);
-    if (active && diag && b == 0 && r < D) s1p[(size_t)p * D + r] = acc1;
+    if (!active && threadIdx.x >= kS1Thread && threadIdx.x < kS1Thread + 16) {
+        const int row = tr * 16 + (int)threadIdx.x - kS1Thread;
+        if (row < D) s1p[(size_t)p * D + row] = acc1;
+    }
 }
 
 // The elites' deviations from the best elite in FP64, y_j = x_(j) - x_(1) (exact: both are

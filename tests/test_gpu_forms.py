@@ -249,3 +249,28 @@ def test_batch_factor_cluster_sizes(lib, crane, K):
             assert np.array_equal(res[q][0], ctrl)
     finally:
         lib.cp_batch_destroy(b)
+
+
+@pytest.mark.parametrize("K", [1, 7, 32])
+def test_sample_adds_the_mean_in_fp64(lib, crane, K):
+    """xi = float(mu + acc) with the sum in FP64, for means of all sizes, on ties of the rounding to
+    FP32 and beside draws too small to leave them: acc is the draw about a zero mean."""
+    import torch
+    from paper_2503_14160_gb300 import workloads
+    g = np.random.default_rng(K)
+    D, N = 4 * K, 3001
+    mu = g.normal(size=D) * 10.0 ** g.uniform(-42, 6, D)
+    mu[0::4] = g.normal(size=K).astype(np.float32) * (1.0 + 2.0 ** -24)
+    mu[1::4] = 1.0 + 2.0 ** -24
+    std = np.where(np.arange(D) % 4 == 1, 1e-13, 10.0 ** g.uniform(-3, 1, D))
+    C = torch.from_numpy(np.diag(std ** 2)).cuda()
+    out = []
+    with lib.Planner(crane, workloads.empty_scene(), lib.make_params(N, K, 2, sigma=1.0)) as pl:
+        lib.cp_set_endpoints(pl.handle, *ENDS[0])
+        for m in (np.zeros(D), mu):
+            lib.cp_set_distribution(pl.handle, torch.from_numpy(m).cuda(), C, 1)
+            xi = torch.zeros(N, K, 4, device="cuda")
+            lib.cp_sample(pl.handle, 1, xi)
+            lib.cp_synchronize(pl.handle)
+            out.append(xi.cpu().numpy().reshape(N, D))
+    assert np.array_equal(out[1], (mu + out[0].astype(np.float64)).astype(np.float32))
