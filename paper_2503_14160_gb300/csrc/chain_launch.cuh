@@ -1,7 +1,7 @@
 // Launches of a chain of dependent kernels (programmatic dependent launch). A plan's iteration is
 // some ten short kernels, each needing all of the one before, so the gap between them counts: with
 // the attribute below a kernel's blocks may be placed while the kernel before still runs, and
-// after_previous(), the first statement of every such kernel, waits until that one has completed
+// after_previous(), called before such a kernel touches anything of the others, waits until that one has completed
 // and its writes are visible. Every kernel of a chain waits, so completion is transitive: whatever
 // follows a kernel on the stream sees everything before it. The wait has no limit of its own: it
 // ends when the kernel before ends, as an ordinary launch would begin.
@@ -21,8 +21,8 @@ static __device__ __forceinline__ void after_previous()
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// kern<<<grid, block, smem, st>>>(args...) with the attribute. The kernel's first statement is
-// after_previous().
+// kern<<<grid, block, smem, st>>>(args...) with the attribute. The kernel calls
+// after_previous() before it reads or writes global memory.
 template <typename... P, typename... A>
 inline void launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args)
 {

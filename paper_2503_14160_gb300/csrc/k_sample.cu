@@ -4,6 +4,8 @@
 //   k_sample  z_i from Philox4x32-10 (Salmon et al., SC'11) + Box-Muller, xi_i = mu + L z_i
 // The counter of candidate i, block j, iteration t, query q is (j, i, t, q); the key is
 // the 64-bit seed split into two words. Block j gives the normals z[4j..4j+3].
+#include <algorithm>
+
 #include "chain_launch.cuh"
 #include "cp_internal.cuh"
 #include "fp64_chain.cuh"
@@ -107,17 +109,30 @@ __global__ void __launch_bounds__(kFactorThreads) k_batch_factor(const BatchQuer
     factor_body(q.C, q.sigma2, q.D, q.L, q.Lt, q.status, A);
 }
 
+// The sampler's tile: a warp draws 2 Q candidates, its lower half the first Q and its upper half
+// the others; lane l of a half holds rows l, l + 16, .. of L z for all of its Q. Both operands of
+// an FMA come from shared memory, which delivers 128 bytes per cycle to the SM, a word broadcast to
+// 32 lanes like 32 words: with one row and eight candidates per lane, nine words per eight FMAs,
+// that bounded the kernel. With eight rows and eight candidates it is 16 per 64.
+// N = 65536, D = 128: 104 us in the former shape, 90 with the mean added in FP32, 54 now.
 constexpr int kSampleWarps = 8;
 constexpr int kSampleThreads = 32 * kSampleWarps;
-constexpr int kSampleCands = 8;   // candidates a warp draws at a time
+constexpr int kRowBlock = 16;                              // rows of a block, columns of a segment
+constexpr int kMaxBlocks = 4 * CP_MAX_WAYPOINTS / kRowBlock;   // 8
 
-// Shared memory of the sampler: L^T (FP32, column-major, D x D, plus a pad of 32 floats read
-// by the lanes past the last row), the mean's rows as MeanRow and per warp the normals of its
-// kSampleCands candidates ([D][kSampleCands], candidate fastest).
-size_t sample_smem(int K)
+// Row blocks that the sampler computes for dimension D: an even number (the forms compiled).
+__host__ __device__ constexpr int sample_blocks(int D) { return (D + 2 * kRowBlock - 1) / (2 * kRowBlock) * 2; }
+
+// Floats of the staged factor: column c of segment k = c / 16 from row 16 k on (the rows above
+// hold zeros of L).
+__host__ __device__ constexpr int staged_floats(int nb) { return kRowBlock * kRowBlock * nb * (nb + 1) / 2; }
+
+// Shared memory of the sampler: the staged L^T (FP32), the mean's rows as MeanRow and per warp the
+// normals of its 2 Q candidates ([D][2 Q], candidate fastest).
+size_t sample_smem(int K, int Q)
 {
-    const size_t D = 4 * (size_t)K;
-    return sizeof(float) * (D * D + 32 + 4 * D + (size_t)kSampleWarps * kSampleCands * D);
+    const int D = 4 * K, nb = sample_blocks(D);
+    return sizeof(float) * ((size_t)staged_floats(nb) + 4 * D + (size_t)kSampleWarps * 2 * Q * D);
 }
 
 // A row of the mean for sum_rounded: m = hi + lo + r, |r| <= 2^-48 |m| + 2^-150 < slack / 2.
@@ -147,105 +162,156 @@ __device__ __forceinline__ bool sum_rounded(const MeanRow &m, float a, float &x)
 
 __device__ __noinline__ float sum_fp64(const double *mu, int r, float a) { return (float)(mu[r] + (double)a); }
 
-// Warp w draws the candidates g .. g + 7 of the groups g = g0 + 8 w, g0 + 8 w + g_stride, ...
-// below i_end: their normals (Philox counter (j, i, iter, query) for z[4j..4j+3], spread over
-// the lanes) go to the warp's buffer; then, 32 rows at a time, lane l holds row r = r0 + l of
-// all eight and forms acc = sum_c L[r][c] z[c] over ascending c with one FMA per term (L read
-// once for the eight), and writes xi_r = mu_r + acc (added in FP64, rounded once to FP32: by
-// sum_rounded, as the conversion, the addition and the conversion back hold the scheduler's FP64
-// unit for 205 cycles per 32 entries, 46 of the kernel's 104 us at N = 65536, D = 128; now 90).
-// Columns past the block's last row hold zeros of L for every row of the block and are
+// The normals of candidates g .. g + 2 Q - 1 (Philox counter (j, i, iter, query) for z[4j..4j+3],
+// spread over the lanes) into the warp's buffer.
+template <int Q>
+__device__ __forceinline__ void draw_normals(float *sZ, int K, uint32_t k0, uint32_t k1, uint32_t iter, uint32_t query,
+                                             int g, int i_end, int lane)
+{
+    for (int pq = lane; pq < 2 * Q * K; pq += 32) {
+        const int cnd = pq % (2 * Q), j = pq / (2 * Q);
+        const int i = g + cnd;
+        float z0 = 0.f, z1 = 0.f, z2 = 0.f, z3 = 0.f;
+        if (i < i_end) {
+            const uint4 x = philox4x32_10(make_uint4((uint32_t)j, (uint32_t)i, iter, query), k0, k1);
+            box_muller(x.x, x.y, z0, z1);
+            box_muller(x.z, x.w, z2, z3);
+        }
+        sZ[(4 * j + 0) * 2 * Q + cnd] = z0;
+        sZ[(4 * j + 1) * 2 * Q + cnd] = z1;
+        sZ[(4 * j + 2) * 2 * Q + cnd] = z2;
+        sZ[(4 * j + 3) * 2 * Q + cnd] = z3;
+    }
+    __syncwarp();
+}
+
+// xi of the warp's candidates: acc = sum_c L[r][c] z[c] over ascending c with one FMA per term, then
+// xi_r = mu_r + acc (added in FP64, rounded once to FP32: by sum_rounded, as the conversion, the
+// addition and the conversion back hold the scheduler's FP64 unit for 205 cycles per 32 entries).
+// Columns past the last one of a row's block hold zeros of L for every row of the block and are
 // skipped; adding 0 z leaves a nonzero sum unchanged, so each row equals the full D-term sum.
+template <int Q, int NB>
+__device__ __forceinline__ void multiply_rows(const double *__restrict__ mu, const float *sL, const MeanRow *sM,
+                                              const float *sZ, int D, float *xi, int g, int i_end, int lane)
+{
+    const int row = lane & (kRowBlock - 1), half = lane >> 4;
+    float acc[NB][Q];
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+#pragma unroll
+        for (int q = 0; q < Q; ++q) acc[b][q] = 0.f;
+    const float *l = sL + row, *zc = sZ + Q * half;
+#pragma unroll
+    for (int k = 0; k < NB; ++k) {
+        const int n = min(D - kRowBlock * k, kRowBlock);   // columns of the segment (none: <= 0)
+#pragma unroll 2
+        for (int c = 0; c < n; ++c) {
+            float z[Q];
+#pragma unroll
+            for (int q = 0; q < Q; q += 2) {
+                const float2 v = *reinterpret_cast<const float2 *>(zc + q);
+                z[q] = v.x;
+                z[q + 1] = v.y;
+            }
+#pragma unroll
+            for (int b = k; b < NB; ++b) {
+                const float lv = l[kRowBlock * (b - k)];
+#pragma unroll
+                for (int q = 0; q < Q; ++q) acc[b][q] = fmaf(lv, z[q], acc[b][q]);
+            }
+            l += kRowBlock * (NB - k);
+            zc += 2 * Q;
+        }
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+        const int r = kRowBlock * b + row;
+        if (r < D) {
+            const MeanRow m = sM[r];
+            bool ok = true;
+            float x[Q];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) ok = sum_rounded(m, acc[b][q], x[q]) && ok;
+            if (!ok)
+#pragma unroll
+                for (int q = 0; q < Q; ++q) x[q] = sum_fp64(mu, r, acc[b][q]);
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const int i = g + Q * half + q;
+                if (i < i_end) xi[(size_t)i * D + r] = x[q];
+            }
+        }
+    }
+    __syncwarp();
+}
+
+// Warp w draws the groups of 2 Q candidates from g0 + 2 Q w on, g_stride apart, below i_end.
+// kWait: the mean and the factor come from the launch before (its end is awaited after
+// the first group's normals, which need neither).
+template <int Q, bool kWait>
 __device__ __forceinline__ void sample_body(const double *__restrict__ mu, const float *__restrict__ Lt, int K,
                                             uint32_t k0, uint32_t k1, uint32_t iter, uint32_t query,
                                             float *xi, int g0, int g_stride, int i_end, float *sm)
 {
-    const int D = 4 * K;
-    float *sL = sm;
+    const int D = 4 * K, nb = sample_blocks(D), rows = kRowBlock * nb;
     const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    MeanRow *sM = reinterpret_cast<MeanRow *>(sm + D * D + 32);
-    float *sZ = sm + D * D + 32 + 4 * D + wib * kSampleCands * D;
-    for (int idx = threadIdx.x; idx < D * D; idx += blockDim.x) sL[idx] = Lt[idx];
-    if (threadIdx.x < 32) sL[D * D + threadIdx.x] = 0.f;
+    float *sL = sm;
+    MeanRow *sM = reinterpret_cast<MeanRow *>(sm + staged_floats(nb));
+    float *sZ = sm + staged_floats(nb) + 4 * D + wib * 2 * Q * D;
+    const int first = g0 + 2 * Q * wib;
+    draw_normals<Q>(sZ, K, k0, k1, iter, query, first, i_end, lane);
+    if (kWait) after_previous();
+    // 16-byte pieces of the columns, all in flight together (rows past D: zeros)
+    for (int k = 0, at = 0; k < nb; ++k) {
+        const int top = kRowBlock * k, pieces = (rows - top) / 4;
+        for (int e = threadIdx.x; e < min(kRowBlock, D - top) * pieces; e += kSampleThreads) {
+            const int c = top + e / pieces, r = top + 4 * (e % pieces);
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::
+                         "r"((uint32_t)__cvta_generic_to_shared(sL + at + 4 * e)),
+                         "l"(Lt + (r < D ? c * D + r : 0)), "r"(r < D ? 16 : 0) : "memory");
+        }
+        at += kRowBlock * 4 * pieces;
+    }
     for (int r = threadIdx.x; r < D; r += blockDim.x) sM[r] = mean_row(mu[r]);
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    for (int g = g0 + kSampleCands * wib; g < i_end; g += g_stride) {
-        for (int pq = lane; pq < kSampleCands * K; pq += 32) {
-            const int cnd = pq % kSampleCands, j = pq / kSampleCands;
-            const int i = g + cnd;
-            float z0 = 0.f, z1 = 0.f, z2 = 0.f, z3 = 0.f;
-            if (i < i_end) {
-                const uint4 x = philox4x32_10(make_uint4((uint32_t)j, (uint32_t)i, iter, query), k0, k1);
-                box_muller(x.x, x.y, z0, z1);
-                box_muller(x.z, x.w, z2, z3);
-            }
-            sZ[(4 * j + 0) * kSampleCands + cnd] = z0;
-            sZ[(4 * j + 1) * kSampleCands + cnd] = z1;
-            sZ[(4 * j + 2) * kSampleCands + cnd] = z2;
-            sZ[(4 * j + 3) * kSampleCands + cnd] = z3;
+    for (int g = first; g < i_end; g += g_stride) {
+        if (g != first) draw_normals<Q>(sZ, K, k0, k1, iter, query, g, i_end, lane);
+        switch (nb) {
+        case 2: multiply_rows<Q, 2>(mu, sL, sM, sZ, D, xi, g, i_end, lane); break;
+        case 4: multiply_rows<Q, 4>(mu, sL, sM, sZ, D, xi, g, i_end, lane); break;
+        case 6: multiply_rows<Q, 6>(mu, sL, sM, sZ, D, xi, g, i_end, lane); break;
+        default: multiply_rows<Q, kMaxBlocks>(mu, sL, sM, sZ, D, xi, g, i_end, lane); break;
         }
-        __syncwarp();
-        for (int r0 = 0; r0 < D; r0 += 32) {
-            const int r = r0 + lane;
-            float acc[kSampleCands];
-#pragma unroll
-            for (int q = 0; q < kSampleCands; ++q) acc[q] = 0.f;
-            const int c_last = min(D, r0 + 32);
-            for (int c = 0; c < c_last; ++c) {
-                const float l = sL[c * D + r];
-                const float4 za = *reinterpret_cast<const float4 *>(sZ + c * kSampleCands);
-                const float4 zb = *reinterpret_cast<const float4 *>(sZ + c * kSampleCands + 4);
-                acc[0] = fmaf(l, za.x, acc[0]);
-                acc[1] = fmaf(l, za.y, acc[1]);
-                acc[2] = fmaf(l, za.z, acc[2]);
-                acc[3] = fmaf(l, za.w, acc[3]);
-                acc[4] = fmaf(l, zb.x, acc[4]);
-                acc[5] = fmaf(l, zb.y, acc[5]);
-                acc[6] = fmaf(l, zb.z, acc[6]);
-                acc[7] = fmaf(l, zb.w, acc[7]);
-            }
-            if (r < D) {
-                const MeanRow m = sM[r];
-                bool ok = true;
-                float x[kSampleCands];
-#pragma unroll
-                for (int q = 0; q < kSampleCands; ++q) ok = sum_rounded(m, acc[q], x[q]) && ok;
-                if (!ok)
-#pragma unroll
-                    for (int q = 0; q < kSampleCands; ++q) x[q] = sum_fp64(mu, r, acc[q]);
-#pragma unroll
-                for (int q = 0; q < kSampleCands; ++q)
-                    if (g + q < i_end) xi[(size_t)(g + q) * D + r] = x[q];
-            }
-        }
-        __syncwarp();
     }
 }
 
-__global__ void __launch_bounds__(kSampleThreads)
+template <int Q>
+__global__ void __launch_bounds__(kSampleThreads, 2)
 k_sample(const double *__restrict__ mu, const float *__restrict__ Lt, int N, int K,
          uint32_t k0, uint32_t k1, uint32_t iter, uint32_t query, float *xi)
 {
-    after_previous();
     extern __shared__ __align__(16) float sm[];
-    const int per_block = kSampleWarps * kSampleCands;
-    sample_body(mu, Lt, K, k0, k1, iter, query, xi, blockIdx.x * per_block, gridDim.x * per_block, N, sm);
+    const int per_block = kSampleWarps * 2 * Q;
+    sample_body<Q, true>(mu, Lt, K, k0, k1, iter, query, xi, blockIdx.x * per_block, gridDim.x * per_block, N, sm);
 }
 
+constexpr int kBatchQ = 8;
+
 // Every query's draw in one launch: block b of query q takes the kBatchSampleCands
-// candidates from b kBatchSampleCands, each warp several groups of kSampleCands in turn (the
+// candidates from b kBatchSampleCands, each warp several groups in turn (the
 // block stages the query's factor once for all of them). A candidate's normals and
 // arithmetic do not depend on which warp draws it, so each query's xi equals its plain draw.
-__global__ void __launch_bounds__(kSampleThreads)
+__global__ void __launch_bounds__(kSampleThreads, 2)
 k_batch_sample(const BatchQueryDev *__restrict__ qd, const int2 *__restrict__ tab, uint32_t iter)
 {
     extern __shared__ __align__(16) float sm[];
     const int2 e = tab[blockIdx.x];
     const BatchQueryDev &q = qd[e.x];
     const int b = e.y * kBatchSampleCands;
-    static_assert(kBatchSampleCands % (kSampleWarps * kSampleCands) == 0, "whole groups of candidates per warp");
-    sample_body(q.mu, q.Lt, q.K, q.seed_lo, q.seed_hi, iter, q.query, q.xi, b, kSampleWarps * kSampleCands,
-                min(q.N, b + kBatchSampleCands), sm);
+    static_assert(kBatchSampleCands % (kSampleWarps * 2 * kBatchQ) == 0, "whole groups of candidates per warp");
+    sample_body<kBatchQ, false>(q.mu, q.Lt, q.K, q.seed_lo, q.seed_hi, iter, q.query, q.xi, b,
+                                kSampleWarps * 2 * kBatchQ, min(q.N, b + kBatchSampleCands), sm);
 }
 
 }  // namespace
@@ -263,10 +329,11 @@ int launch_philox(const uint32_t *ctr, uint32_t k0, uint32_t k1, int64_t n, uint
 
 int sample_configure()
 {
-    CP_CUDA(cudaFuncSetAttribute(k_sample, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sample_smem(CP_MAX_WAYPOINTS)));
-    CP_CUDA(cudaFuncSetAttribute(k_batch_sample, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sample_smem(CP_MAX_WAYPOINTS)));
+    const int smem = (int)sample_smem(CP_MAX_WAYPOINTS, 8);
+    CP_CUDA(cudaFuncSetAttribute(k_sample<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    CP_CUDA(cudaFuncSetAttribute(k_sample<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    CP_CUDA(cudaFuncSetAttribute(k_sample<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    CP_CUDA(cudaFuncSetAttribute(k_batch_sample, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     const int Dm = 4 * CP_MAX_WAYPOINTS;
     CP_CUDA(cudaFuncSetAttribute(k_batch_factor, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(sizeof(double) * Dm * (Dm + 1))));
@@ -294,25 +361,40 @@ int launch_batch_sample(const BatchQueryDev *qd, const int2 *tab, int blocks, in
                         cudaStream_t st)
 {
     if (blocks == 0) return CP_OK;
-    k_batch_sample<<<blocks, kSampleThreads, sample_smem(max_K), st>>>(qd, tab, iter);
+    k_batch_sample<<<blocks, kSampleThreads, sample_smem(max_K, kBatchQ), st>>>(qd, tab, iter);
     CP_LAUNCHED("k_batch_sample");
+    return CP_OK;
+}
+
+// Candidates per warp: the fewest of 4, 8 and 16 whose blocks of eight warps all have an SM to
+// themselves, else 16. More per warp take fewer shared-memory words per FMA, fewer make more warps
+// and a shorter chain of one draw and one product. us with 4, 8 and 16 (former kernel):
+//   N = 4096, D = 128: 8.0, 9.2, 14.4 (23.6);   N = 8192, D = 128: 11.3, 10.0, 14.6 (23.6);
+//   N = 16384, D = 128: 20.0, 16.2, 15.6 (31.2);   N = 256, D = 32: 2.9, 3.1, 3.6 (4.1).
+template <int Q>
+int launch_sample_form(int sms, const double *mu, const float *Lt_f, int N, int K, uint64_t seed, uint32_t iter,
+                       uint32_t query, float *xi, cudaStream_t st)
+{
+    int per_sm = 0;
+    const size_t smem = sample_smem(K, Q);
+    CP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample<Q>, kSampleThreads, smem));
+    if (per_sm < 1) per_sm = 1;
+    const int per_block = kSampleWarps * 2 * Q, blocks = std::min((N + per_block - 1) / per_block, sms * per_sm);
+    launch_chained(k_sample<Q>, blocks, kSampleThreads, smem, st, mu, Lt_f, N, K, (uint32_t)seed,
+                   (uint32_t)(seed >> 32), iter, query, xi);
+    CP_LAUNCHED("k_sample");
     return CP_OK;
 }
 
 int launch_sample(const double *mu, const float *Lt_f, int N, int K, uint64_t seed,
                   uint32_t iter, uint32_t query, float *xi, cudaStream_t st)
 {
-    int dev = 0, sms = 0, per_sm = 0;
+    int dev = 0, sms = 0;
     CP_CUDA(cudaGetDevice(&dev));
     CP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const size_t smem = sample_smem(K);
-    CP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sample, kSampleThreads, smem));
-    if (per_sm < 1) per_sm = 1;
-    int blocks = (N + kSampleWarps * kSampleCands - 1) / (kSampleWarps * kSampleCands);
-    if (blocks > sms * per_sm) blocks = sms * per_sm;
-    launch_chained(k_sample, blocks, kSampleThreads, smem, st, mu, Lt_f, N, K, (uint32_t)seed, (uint32_t)(seed >> 32), iter, query, xi);
-    CP_LAUNCHED("k_sample");
-    return CP_OK;
+    if (N <= sms * kSampleWarps * 4) return launch_sample_form<2>(sms, mu, Lt_f, N, K, seed, iter, query, xi, st);
+    if (N <= sms * kSampleWarps * 8) return launch_sample_form<4>(sms, mu, Lt_f, N, K, seed, iter, query, xi, st);
+    return launch_sample_form<8>(sms, mu, Lt_f, N, K, seed, iter, query, xi, st);
 }
 
 }  // namespace cp

@@ -274,3 +274,31 @@ def test_sample_adds_the_mean_in_fp64(lib, crane, K):
             lib.cp_synchronize(pl.handle)
             out.append(xi.cpu().numpy().reshape(N, D))
     assert np.array_equal(out[1], (mu + out[0].astype(np.float64)).astype(np.float32))
+
+
+@pytest.mark.parametrize("K", [1, 4, 7, 12, 17, 20, 25, 32])
+def test_sample_forms(lib, crane, K):
+    """The sampler's row blocks (2, 4, 6 or 8 of 16 rows, ragged) and candidates per warp (4, 8 and
+    16, by N): a candidate's draw is the same in every form, and is mu + L z to the sampler's bound."""
+    import torch
+    import oracle
+    from helpers import factor_sample_bound
+    from paper_2503_14160_gb300 import workloads
+    g = np.random.default_rng(40 + K)
+    D = 4 * K
+    A, mu = g.normal(size=(D, D)), g.normal(size=D)
+    C = A @ A.T / D + 0.1 * np.eye(D)
+    out = []
+    for N in (61, 7001, 20003):
+        with lib.Planner(crane, workloads.empty_scene(), lib.make_params(N, K, 2, sigma=0.7, seed=11, query=3)) as pl:
+            lib.cp_set_endpoints(pl.handle, *ENDS[0])
+            lib.cp_set_distribution(pl.handle, torch.from_numpy(mu).cuda(), torch.from_numpy(C).cuda(), 5)
+            xi = torch.full((N, K, 4), np.nan, device="cuda")
+            lib.cp_sample(pl.handle, 5, xi)
+            lib.cp_synchronize(pl.handle)
+            out.append(xi.cpu().numpy().reshape(N, D))
+    assert np.array_equal(out[0], out[1][:61]) and np.array_equal(out[1], out[2][:7001])
+    assert np.all(np.isfinite(out[2]))
+    L = oracle.factor(C, 0.7)
+    want = oracle.sample(mu, L, 11, 5, 3, 61, K).reshape(61, D)
+    assert np.all(np.abs(out[0] - want) <= factor_sample_bound(want, oracle.normals(11, 5, 3, 61, K), L))
