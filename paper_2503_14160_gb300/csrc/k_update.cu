@@ -1,5 +1,5 @@
 // Algorithm 1 steps (3)-(6) (arXiv 2503.14160, Sec. 4.1):
-//   k_weights        w_j = (ln(nu + 1/2) - ln j) / sum_k (ln(nu + 1/2) - ln k), FP64, once
+//   k_weight_*       w_j = (ln(nu + 1/2) - ln j) / sum_k (ln(nu + 1/2) - ln k), FP64, once
 //   k_rank_count     rank of every candidate = number of candidates before it in the order
 //                    (J ascending, NaN as +inf, ties by index): an all-pairs count, split
 //                    over the grid's y dimension and summed with integer atomics
@@ -32,20 +32,32 @@ __device__ __forceinline__ unsigned long long order_key(double v)
     return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
 }
 
-__global__ void k_weights(int nu, double *w)
+// The weights in three launches: the terms over the grid, their sum by one block, the quotients over
+// the grid (nu = 32768: 664 us in one block, 25 us).
+__global__ void k_weight_terms(int nu, double *w)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < nu) w[j] = log((double)nu + 0.5) - log((double)(j + 1));
+}
+
+__global__ void __launch_bounds__(1024) k_weight_sum(int nu, const double *__restrict__ w, double *total)
 {
     __shared__ double part[1024];
-    const double top = log((double)nu + 0.5);
     double acc = 0.0;
-    for (int j = threadIdx.x; j < nu; j += blockDim.x) acc += top - log((double)(j + 1));
+    for (int j = threadIdx.x; j < nu; j += 1024) acc += w[j];
     part[threadIdx.x] = acc;
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
+    for (int s = 512; s > 0; s >>= 1) {
         if (threadIdx.x < s) part[threadIdx.x] += part[threadIdx.x + s];
         __syncthreads();
     }
-    const double total = part[0];
-    for (int j = threadIdx.x; j < nu; j += blockDim.x) w[j] = (top - log((double)(j + 1))) / total;
+    if (threadIdx.x == 0) *total = part[0];
+}
+
+__global__ void k_weight_quotients(int nu, double *w, const double *__restrict__ total)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < nu) w[j] /= *total;
 }
 
 // Block (x, y): candidates i of block x against the candidates j of the y-th range of
@@ -106,7 +118,11 @@ __global__ void k_scatter(int *__restrict__ rank, const double *__restrict__ J,
 // chunk-major ([chunk][row][col] and [chunk][row]): a tile's writes are rows of 16
 // consecutive entries, and the combine (one thread per entry) reads one chunk of
 // consecutive entries per load.
+// kRaw: the deviations are formed from the elites where they are staged (elites, w; Y and WY unused)
+// instead of by a launch before.
+template <bool kRaw>
 __device__ __forceinline__ void moments_partial_body(const double *__restrict__ Y, const double *__restrict__ WY,
+                                                    const float *__restrict__ elites, const double *__restrict__ w,
                                                     int nu, int D, int per, int n_chunks, double *s2p, double *s1p,
                                                     int t, int p)
 {
@@ -138,8 +154,14 @@ __device__ __forceinline__ void moments_partial_body(const double *__restrict__ 
             const int j = idx >> 4, k = idx & 15;
             const int r = tr * 16 + k, c = tc * 16 + k;
             const size_t row = (size_t)(j0 + j) * D;
-            wyr[j][k] = r < D ? WY[row + r] : 0.0;
-            yc[j][k] = c < D ? Y[row + c] : 0.0;
+            if (kRaw) {
+                const double y = r < D ? (double)elites[row + r] - (double)elites[r] : 0.0;
+                wyr[j][k] = w[j0 + j] * y;
+                yc[j][k] = diag ? y : (c < D ? (double)elites[row + c] - (double)elites[c] : 0.0);
+            } else {
+                wyr[j][k] = r < D ? WY[row + r] : 0.0;
+                yc[j][k] = c < D ? Y[row + c] : 0.0;
+            }
         }
         __syncthreads();
         if (active) {
@@ -187,7 +209,15 @@ k_moments_partial(const double *__restrict__ Y, const double *__restrict__ WY, i
                   int per, int n_chunks, double *s2p, double *s1p)
 {
     after_previous();
-    moments_partial_body(Y, WY, nu, D, per, n_chunks, s2p, s1p, blockIdx.x, blockIdx.y);
+    moments_partial_body<false>(Y, WY, nullptr, nullptr, nu, D, per, n_chunks, s2p, s1p, blockIdx.x, blockIdx.y);
+}
+
+__global__ void __launch_bounds__(256)
+k_moments_partial_raw(const float *__restrict__ elites, const double *__restrict__ w, int nu, int D,
+                      int per, int n_chunks, double *s2p, double *s1p)
+{
+    after_previous();
+    moments_partial_body<true>(nullptr, nullptr, elites, w, nu, D, per, n_chunks, s2p, s1p, blockIdx.x, blockIdx.y);
 }
 
 // Every query's deviations in one launch (block b of query q: entries 256 b ..).
@@ -207,7 +237,7 @@ k_batch_moments_partial(const BatchQueryDev *__restrict__ qd, const int2 *__rest
     const int2 e = tab[blockIdx.x];
     const BatchQueryDev &q = qd[e.x];
     const int nt = (q.D + 15) / 16, tiles = nt * (nt + 1) / 2;
-    moments_partial_body(q.mom_y, q.mom_y + (size_t)q.nu * q.D, q.nu, q.D, q.per, q.n_chunks, q.s2p, q.s1p,
+    moments_partial_body<false>(q.mom_y, q.mom_y + (size_t)q.nu * q.D, nullptr, nullptr, q.nu, q.D, q.per, q.n_chunks, q.s2p, q.s1p,
                          e.y % tiles, e.y / tiles);
 }
 
@@ -315,6 +345,23 @@ k_moments_combine(const double *__restrict__ s2p, const double *__restrict__ s1,
     after_previous();
     const int g = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     moments_combine_body(s2p, s1, n_chunks, D, eps, C, g / kSumLanes, g % kSumLanes);
+}
+
+// S1, the mean (by block 0) and the entries in one launch: every block sums S1 of the rows up to its
+// last entry's itself.
+__global__ void __launch_bounds__(128)
+k_moments_final(const double *__restrict__ s2p, const double *__restrict__ s1p, int n_chunks, int D, double eps,
+                const float *__restrict__ elites, double *mu, double *C)
+{
+    after_previous();
+    __shared__ double s_s1[4 * CP_MAX_WAYPOINTS];
+    const int g = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    int r_last, c_last;
+    tri_index(min((int)(blockIdx.x + 1) * 32, D * (D + 1) / 2) - 1, r_last, c_last);
+    stage_s1(s1p, n_chunks, D, blockIdx.x == 0 ? D - 1 : r_last, s_s1);
+    if (blockIdx.x == 0)
+        for (int r = threadIdx.x; r < D; r += blockDim.x) mu[r] = (double)elites[r] + s_s1[r];
+    moments_combine_body(s2p, s_s1, n_chunks, D, eps, C, g / kSumLanes, g % kSumLanes);
 }
 
 // Block (x, q): S1 and the mean of rows 32 x .. 32 x + 31 of query q.
@@ -848,10 +895,15 @@ int update_configure()
     return CP_OK;
 }
 
-int launch_weights(int nu, double *w, cudaStream_t st)
+int launch_weights(int nu, double *w, double *total, cudaStream_t st)
 {
-    k_weights<<<1, 1024, 0, st>>>(nu, w);
-    CP_LAUNCHED("k_weights");
+    const int blocks = (nu + 255) / 256;
+    k_weight_terms<<<blocks, 256, 0, st>>>(nu, w);
+    CP_LAUNCHED("k_weight_terms");
+    k_weight_sum<<<1, 1024, 0, st>>>(nu, w, total);
+    CP_LAUNCHED("k_weight_sum");
+    k_weight_quotients<<<blocks, 256, 0, st>>>(nu, w, total);
+    CP_LAUNCHED("k_weight_quotients");
     return CP_OK;
 }
 
@@ -891,11 +943,24 @@ static int launch_moments_partial(const float *elites, const double *w, int nu, 
     const int n_chunks = (nu + per - 1) / per;
     const int tiles = (D + 15) / 16;
     double *Y = yw, *WY = yw + (size_t)nu * D;
-    launch_chained(k_moments_prep, (nu * D + 255) / 256, 256, 0, st, elites, w, nu, D, Y, WY);
-    CP_LAUNCHED("k_moments_prep");
     dim3 grid(tiles * (tiles + 1) / 2, n_chunks);
-    launch_chained(k_moments_partial, grid, 256, 0, st, Y, WY, nu, D, per, n_chunks, s2p, s1p);
-    CP_LAUNCHED("k_moments_partial");
+    int dev = 0, sms = 0;
+    CP_CUDA(cudaGetDevice(&dev));
+    CP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    // The deviations by a launch of their own, once for all tiles, unless the blocks are few: then
+    // the time is that of one block and the launches, and forming them in the blocks is shorter.
+    // An iteration of a plan with it and with kShortS1's rule, against neither: nu = 128, D = 32
+    // 43.1 against 44.1 us, nu = 300, D = 32 47.9 against 49.0; beyond both rules (nu = 750, D = 48,
+    // 144 blocks) 90.8 against 77.9.
+    if ((int)(4 * grid.x * grid.y) <= sms) {
+        launch_chained(k_moments_partial_raw, grid, 256, 0, st, elites, w, nu, D, per, n_chunks, s2p, s1p);
+        CP_LAUNCHED("k_moments_partial_raw");
+    } else {
+        launch_chained(k_moments_prep, (nu * D + 255) / 256, 256, 0, st, elites, w, nu, D, Y, WY);
+        CP_LAUNCHED("k_moments_prep");
+        launch_chained(k_moments_partial, grid, 256, 0, st, Y, WY, nu, D, per, n_chunks, s2p, s1p);
+        CP_LAUNCHED("k_moments_partial");
+    }
     *n_chunks_out = n_chunks;
     return CP_OK;
 }
@@ -1000,6 +1065,10 @@ int launch_batch_moments(const BatchQueryDev *qd, int nq, const int2 *tab_prep, 
     return CP_OK;
 }
 
+// Chunk sums of the first moments up to which every block of the combine adds them itself (128 at
+// nu = 128, D = 32; figures at launch_moments_partial).
+constexpr int kShortS1 = 512;
+
 int launch_moments(const float *elites, const double *w, int nu, int D, double eps, double *yw,
                    double *s2p, double *s1p, double *mu, double *C, cudaStream_t st)
 {
@@ -1007,6 +1076,12 @@ int launch_moments(const float *elites, const double *w, int nu, int D, double e
     int rc = launch_moments_partial(elites, w, nu, D, yw, s2p, s1p, &n_chunks, st);
     if (rc != CP_OK) return rc;
     const int entries = D * (D + 1) / 2;
+    // One launch where S1 is short (its sums are repeated by every block), else two.
+    if (D * n_chunks <= kShortS1) {
+        launch_chained(k_moments_final, (entries + 31) / 32, 128, 0, st, s2p, s1p, n_chunks, D, eps, elites, mu, C);
+        CP_LAUNCHED("k_moments_final");
+        return CP_OK;
+    }
     launch_chained(k_moments_s1, (D + 31) / 32, 128, 0, st, s1p, n_chunks, D, elites, mu);
     CP_LAUNCHED("k_moments_s1");
     launch_chained(k_moments_combine, (entries + 31) / 32, 128, 0, st, s2p, s1p + (size_t)n_chunks * D, n_chunks, D, eps, C);

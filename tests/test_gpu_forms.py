@@ -302,3 +302,35 @@ def test_sample_forms(lib, crane, K):
     L = oracle.factor(C, 0.7)
     want = oracle.sample(mu, L, 11, 5, 3, 61, K).reshape(61, D)
     assert np.all(np.abs(out[0] - want) <= factor_sample_bound(want, oracle.normals(11, 5, 3, 61, K), L))
+
+
+@pytest.mark.parametrize("N,K", [(2, 1), (37, 3), (130, 8), (600, 8), (4000, 8), (4400, 8), (600, 32), (1000, 5),
+                                 (2200, 4)])
+def test_moment_forms(lib, crane, N, K):
+    """Deviations formed in the partial sums' blocks or by a launch before, first moments summed in the
+    combine's blocks or by a launch before: mean and covariance of one update against long double,
+    each sum within nu + 16 FP64 roundings of its absolute terms."""
+    import torch
+    from paper_2503_14160_gb300 import workloads
+    g = np.random.default_rng(N * K)
+    D = 4 * K
+    xi = g.normal(size=(N, D)).astype(np.float32)
+    J = workloads.random_costs(N, seed=N)
+    with lib.Planner(crane, workloads.empty_scene(), lib.make_params(N, K, 2, eps=0.125)) as pl:
+        nu = pl.nu
+        lib.cp_set_endpoints(pl.handle, *ENDS[0])
+        lib.cp_update(pl.handle, torch.from_numpy(J).cuda(), torch.from_numpy(xi).cuda())
+        mu = torch.empty(D, dtype=torch.float64, device="cuda")
+        C = torch.empty(D, D, dtype=torch.float64, device="cuda")
+        lib.cp_get_distribution(pl.handle, mu, C)
+        torch.cuda.synchronize()
+    w = np.log(nu + 0.5) - np.log(np.arange(1, nu + 1))
+    w = w / w.sum()
+    x = xi[np.argsort(J, kind="stable")[:nu]].astype(np.float64)
+    mu_ref, C_ref, s2, s1 = _moments_reference(x, w)
+    y = np.abs(x - x[0])
+    a1, a2 = (w[:, None] * y).sum(0), (w[:, None] * y).T @ y
+    u = (nu + 16) * 2.0 ** -53
+    assert np.all(np.abs(mu.cpu().numpy() - mu_ref) <= u * (a1 + np.abs(x[0])))
+    C_ref = C_ref + 0.125 * np.eye(D)
+    assert np.all(np.abs(C.cpu().numpy() - C_ref) <= u * (a2 + 3 * np.outer(a1, a1) + 0.125 * np.eye(D)))
