@@ -180,10 +180,8 @@ KERNEL_SOURCES = {
 # kernel's sources at the time of the capture: reported only while the sources still hash
 # to it, None once the kernel has changed.
 PROFILED_TRAFFIC = {
-    # captured at b833554f...; the file changed since only in the batched kernel's call of the
-    # item body, which leaves k_eval_polar as it was
-    ("k_eval_polar", "dense_forest"): {"sha1": "8484a179acebfd8666a344e6c3f694ae59bae607", "bytes": 34001408.0},
-    ("k_eval_polar", "single_large"): {"sha1": "8484a179acebfd8666a344e6c3f694ae59bae607", "bytes": 1160192.0},
+    ("k_eval_polar", "dense_forest"): {"sha1": "8b9ac833ee19a97554bfbac69af387f533f42f47", "bytes": 33655040.0},
+    ("k_eval_polar", "single_large"): {"sha1": "8b9ac833ee19a97554bfbac69af387f533f42f47", "bytes": 1133312.0},
 }
 
 
