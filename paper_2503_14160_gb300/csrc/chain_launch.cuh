@@ -5,6 +5,10 @@
 // and its writes are visible. Every kernel of a chain waits, so completion is transitive: whatever
 // follows a kernel on the stream sees everything before it. The wait has no limit of its own: it
 // ends when the kernel before ends, as an ordinary launch would begin.
+// A chained kernel begins before that wait ends, so what the others write is not read-only for its
+// whole life: it and the functions it calls read global memory by plain loads, never through
+// `const T *__restrict__` or __ldg, which would allow non-coherent loads and let the compiler move
+// them over the wait (a host test looks through the sources for it).
 // Measured with the node that cleared the evaluation's counter gone too: an iteration of the 20-tree
 // query 59 -> 48.5 us, update and sample of 65536 candidates 382 -> 356 us.
 #pragma once

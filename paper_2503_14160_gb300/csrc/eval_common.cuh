@@ -486,10 +486,10 @@ struct Checkpoint {
 static __device__ __forceinline__ void stage_controls(float4 *s_ctrl, const EvalArgs &a, int cand, int lane)
 {
     __syncwarp();
-    const float4 q0 = a.ends != nullptr ? __ldg(a.ends) : a.q0;
-    const float4 qd = a.ends != nullptr ? __ldg(a.ends + 1) : a.qd;
+    const float4 q0 = a.ends != nullptr ? *a.ends : a.q0;
+    const float4 qd = a.ends != nullptr ? a.ends[1] : a.qd;
     const float4 *xi = a.xi + (size_t)cand * a.K;
-    for (int i = lane; i < a.K + 8; i += 32) s_ctrl[i] = i < 4 ? q0 : (i >= a.K + 4 ? qd : __ldg(xi + (i - 4)));
+    for (int i = lane; i < a.K + 8; i += 32) s_ctrl[i] = i < 4 ? q0 : (i >= a.K + 4 ? qd : xi[i - 4]);
     __syncwarp();
 }
 

@@ -90,7 +90,7 @@ __host__ __device__ inline size_t factor_smem(int n_ctas)
 
 // Called by every thread of every CTA of the cluster (`n_ctas` CTAs; those past the last row
 // only take part in the barriers).
-__device__ __forceinline__ void factor_cluster(const double *__restrict__ C, double sigma2, int D, int n_ctas,
+__device__ __forceinline__ void factor_cluster(const double *C, double sigma2, int D, int n_ctas,
                                                double *L, float *Lt, uint32_t *status, double *smem)
 {
     const int b = (int)cooperative_groups::this_cluster().block_rank();
@@ -205,7 +205,7 @@ __device__ __forceinline__ void factor_cluster(const double *__restrict__ C, dou
 }
 
 __global__ void __launch_bounds__(kFactorThreads)
-k_factor(const double *__restrict__ C, double sigma2, const double *__restrict__ sigma_dev, int D, double *L,
+k_factor(const double *C, double sigma2, const double *sigma_dev, int D, double *L,
          float *Lt, uint32_t *status)
 {
     after_previous();

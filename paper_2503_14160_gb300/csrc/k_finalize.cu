@@ -20,8 +20,8 @@ constexpr int kFinalAhead = 8;    // items loaded ahead
 
 // Candidate i on the kFinalLanes aligned lanes that share it (sub = lane within the group).
 // Called by whole warps.
-__device__ __forceinline__ void finalize_body(const double *__restrict__ item_sum,
-                                              const uint32_t *__restrict__ item_count, int n, int P, double w_c,
+__device__ __forceinline__ void finalize_body(const double *item_sum,
+                                              const uint32_t *item_count, int n, int P, double w_c,
                                               double w_l, double lambda_c, double *J, uint8_t *flag, double *terms,
                                               const uint32_t *status, int i, int sub)
 {
@@ -72,7 +72,7 @@ __device__ __forceinline__ void finalize_body(const double *__restrict__ item_su
 }
 
 __global__ void __launch_bounds__(256)
-k_eval_finalize(const double *__restrict__ item_sum, const uint32_t *__restrict__ item_count, int n, int P,
+k_eval_finalize(const double *item_sum, const uint32_t *item_count, int n, int P,
                 double w_c, double w_l, double lambda_c, double *J, uint8_t *flag, double *terms,
                 const uint32_t *status, int *queue)
 {

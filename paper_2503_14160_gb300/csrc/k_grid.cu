@@ -189,11 +189,11 @@ static __device__ __forceinline__ void polar_item(const ModelDev &m, const Scene
                 const int r0 = min(max(round_index(fmaf(r_lo - reach, g.inv_dr, -0.5f)), 0), g.n_ring - 1);
                 const int r1 = min(max(round_index(fmaf(r_hi + reach, g.inv_dr, -0.5f)), 0), g.n_ring - 1);
                 const int cell = bin * g.n_ring;
-                const int beg = __ldg(g.cell_start + cell + r0);
-                const int end = min(__ldg(g.cell_start + cell + r1 + 1), g.capacity);
+                const int beg = g.cell_start[cell + r0];
+                const int end = min(g.cell_start[cell + r1 + 1], g.capacity);
                 if (kExtras) tests += (uint32_t)max(end - beg, 0);
                 for (int e = beg; e < end; ++e) {
-                    const float4 rec = __ldg(g.items + e);   // {cx, cy, bound, id}
+                    const float4 rec = g.items[e];   // {cx, cy, bound, id}
                     const float p = fmaf(c1, rec.x, s1 * rec.y);
                     const float q = fmaf(c1, rec.y, -(s1 * rec.x));
                     const float rhs = fmaf(-q, q, rec.z);
@@ -210,10 +210,10 @@ static __device__ __forceinline__ void polar_item(const ModelDev &m, const Scene
                         const uint32_t in = sign_mask<NSPH>(t);
                         dmin = fminf(dmin, id < sc.n_cyl
                                                ? walk_cylinder<NSPH>(tab, tr, m.base_z, c.q.w, m.r_max, in, rec.x, rec.y,
-                                                                     __ldg(sc.cyl_exact + id))
+                                                                     sc.cyl_exact[id])
                                                : walk_box<NSPH>(tab, tr, m.base_z, c.q.w, in,
-                                                                __ldg(sc.box_c + id - sc.n_cyl),
-                                                                __ldg(sc.box_h + id - sc.n_cyl)));
+                                                                sc.box_c[id - sc.n_cyl],
+                                                                sc.box_h[id - sc.n_cyl]));
                     }
                 }
             }

@@ -233,7 +233,7 @@ __device__ __forceinline__ Obb load_box(const float *r)
 __device__ __forceinline__ float pair_depth(const SceneDev &sc, const float *boxes, int ob, float pen)
 {
     if (ob < sc.n_cyl) {
-        const float4 f = __ldg(sc.cyl_filt + ob), e = __ldg(sc.cyl_exact + ob);
+        const float4 f = sc.cyl_filt[ob], e = sc.cyl_exact[ob];
         const float rc = e.x / kOctCos, hz = 0.5f * (e.z - e.y);
         const float3 pc = make_float3(f.x, f.y, 0.5f * (e.y + e.z));
         const float rbo = sqrtf(fmaf(rc, rc, hz * hz));
@@ -247,7 +247,7 @@ __device__ __forceinline__ float pair_depth(const SceneDev &sc, const float *box
         }
     } else {
         const int bi = ob - sc.n_cyl;
-        const float4 c = __ldg(sc.box_c + bi), h = __ldg(sc.box_h + bi);
+        const float4 c = sc.box_c[bi], h = sc.box_h[bi];
         const float rbo = sqrtf(fmaf(h.x, h.x, fmaf(h.y, h.y, h.z * h.z)));
 #pragma unroll 1
         for (int l = 0; l < 4; ++l) {
@@ -328,12 +328,12 @@ __device__ __forceinline__ float hull_pen_warp(const ModelDev &m, const SceneDev
     auto scan_one = [&](int o) {
         float cx, cy, reach;
         if (o < sc.n_cyl) {
-            const float4 f = __ldg(sc.cyl_filt + o);
+            const float4 f = sc.cyl_filt[o];
             cx = f.x;
             cy = f.y;
-            reach = __ldg(&sc.cyl_exact[o].x) / kOctCos;
+            reach = sc.cyl_exact[o].x / kOctCos;
         } else {
-            const float4 c = __ldg(sc.box_c + o - sc.n_cyl), h = __ldg(sc.box_h + o - sc.n_cyl);
+            const float4 c = sc.box_c[o - sc.n_cyl], h = sc.box_h[o - sc.n_cyl];
             cx = c.x;
             cy = c.y;
             reach = sqrtf(fmaf(h.x, h.x, h.y * h.y));
@@ -362,7 +362,7 @@ __device__ __forceinline__ float hull_pen_warp(const ModelDev &m, const SceneDev
         const int n_grp = n_groups(sc.n_cyl);
         for (int gbase = 0; gbase < n_grp; gbase += 32) {
             uint32_t gmask = __ballot_sync(0xffffffffu, gbase + lane < n_grp &&
-                                                            unit_near(fr, __ldg(sc.cyl_group + gbase + lane), extra));
+                                                            unit_near(fr, sc.cyl_group[gbase + lane], extra));
             while (gmask) {
                 // lane l takes member l % 8 of the (l / 8)-th remaining group
                 uint32_t g = gmask;
@@ -373,7 +373,7 @@ __device__ __forceinline__ float hull_pen_warp(const ModelDev &m, const SceneDev
                 const int o = g ? (gbase + __ffs(g) - 1) * kGroup + (lane & (kGroup - 1)) : sc.n_cyl;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) gmask &= gmask - 1;
-                uint32_t mmask = __ballot_sync(0xffffffffu, o < sc.n_cyl && unit_near(fr, __ldg(sc.cyl_filt + o), extra));
+                uint32_t mmask = __ballot_sync(0xffffffffu, o < sc.n_cyl && unit_near(fr, sc.cyl_filt[o], extra));
                 while (mmask) {
                     const int ob = __shfl_sync(0xffffffffu, o, __ffs(mmask) - 1);
                     mmask &= mmask - 1;

@@ -191,7 +191,7 @@ __device__ __forceinline__ void draw_normals(float *sZ, int K, uint32_t k0, uint
 // Columns past the last one of a row's block hold zeros of L for every row of the block and are
 // skipped; adding 0 z leaves a nonzero sum unchanged, so each row equals the full D-term sum.
 template <int Q, int NB>
-__device__ __forceinline__ void multiply_rows(const double *__restrict__ mu, const float *sL, const MeanRow *sM,
+__device__ __forceinline__ void multiply_rows(const double *mu, const float *sL, const MeanRow *sM,
                                               const float *sZ, int D, float *xi, int g, int i_end, int lane)
 {
     const int row = lane & (kRowBlock - 1), half = lane >> 4;
@@ -249,7 +249,7 @@ __device__ __forceinline__ void multiply_rows(const double *__restrict__ mu, con
 // kWait: the mean and the factor come from the launch before (its end is awaited after
 // the first group's normals, which need neither).
 template <int Q, bool kWait>
-__device__ __forceinline__ void sample_body(const double *__restrict__ mu, const float *__restrict__ Lt, int K,
+__device__ __forceinline__ void sample_body(const double *mu, const float *Lt, int K,
                                             uint32_t k0, uint32_t k1, uint32_t iter, uint32_t query,
                                             float *xi, int g0, int g_stride, int i_end, float *sm)
 {
@@ -288,7 +288,7 @@ __device__ __forceinline__ void sample_body(const double *__restrict__ mu, const
 
 template <int Q>
 __global__ void __launch_bounds__(kSampleThreads, 2)
-k_sample(const double *__restrict__ mu, const float *__restrict__ Lt, int N, int K,
+k_sample(const double *mu, const float *Lt, int N, int K,
          uint32_t k0, uint32_t k1, uint32_t iter, uint32_t query, float *xi)
 {
     extern __shared__ __align__(16) float sm[];

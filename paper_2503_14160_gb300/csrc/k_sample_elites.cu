@@ -224,7 +224,7 @@ k_elite_update(const float *__restrict__ elites, const double *__restrict__ w, c
 // (results are then meaningless) and still releases its tensor memory. `withhold` issues
 // no operand copy, so that the wait for it runs out on purpose (the test of this path).
 __global__ void __launch_bounds__(kTcThreads + 32)
-k_sample_elites(const float *__restrict__ Yp, int N, int D, int n_chunks, int slices, uint32_t tmem_cols,
+k_sample_elites(const float *Yp, int N, int D, int n_chunks, int slices, uint32_t tmem_cols,
                 const PhiloxKeys key, uint32_t iter, uint32_t query, float *P, uint32_t *status, int withhold)
 {
     after_previous();
@@ -378,7 +378,7 @@ k_sample_elites(const float *__restrict__ Yp, int N, int D, int n_chunks, int sl
 // xi[i][d] = mu_d + sum_s P[s][i][d] (slices in order) + sigma sqrt(eps) g'_id, four
 // coordinates per thread: their normals nu + d .. nu + d + 3 come from one Philox block, or
 // two when nu is not a multiple of four.
-__global__ void k_sample_reduce(const float *__restrict__ P, int slices, const float *__restrict__ mu_f, int N,
+__global__ void k_sample_reduce(const float *P, int slices, const float *mu_f, int N,
                                 int D, int nu, float eps_scale, const PhiloxKeys key, uint32_t iter,
                                 uint32_t query, float *xi)
 {

@@ -65,7 +65,7 @@ __global__ void k_weight_quotients(int nu, double *w, const double *__restrict__
 // is k_j < k_i + 1 (the key of a real cost stays below 2^64 - 1), for j >= i k_j < k_i, so
 // each comparison is one 64-bit compare against a threshold that changes once per range.
 __global__ void __launch_bounds__(kRankThreads)
-k_rank_count(const double *__restrict__ J, int N, int *rank)
+k_rank_count(const double *J, int N, int *rank)
 {
     after_previous();
     __shared__ unsigned long long s_key[kRankPer];
@@ -87,8 +87,8 @@ k_rank_count(const double *__restrict__ J, int N, int *rank)
 // One warp per candidate: a candidate of rank r < nu writes its index to elite[r] and its
 // row to elites[r][:]; rank 0 also records its cost. The rank counter goes back to zero for
 // the next ranking.
-__global__ void k_scatter(int *__restrict__ rank, const double *__restrict__ J,
-                          const float *__restrict__ xi, int N, int nu, int D, int *elite,
+__global__ void k_scatter(int *rank, const double *J,
+                          const float *xi, int N, int nu, int D, int *elite,
                           float *elites, double *best_J)
 {
     after_previous();
@@ -121,8 +121,8 @@ __global__ void k_scatter(int *__restrict__ rank, const double *__restrict__ J,
 // kRaw: the deviations are formed from the elites where they are staged (elites, w; Y and WY unused)
 // instead of by a launch before.
 template <bool kRaw>
-__device__ __forceinline__ void moments_partial_body(const double *__restrict__ Y, const double *__restrict__ WY,
-                                                    const float *__restrict__ elites, const double *__restrict__ w,
+__device__ __forceinline__ void moments_partial_body(const double *Y, const double *WY,
+                                                    const float *elites, const double *w,
                                                     int nu, int D, int per, int n_chunks, double *s2p, double *s1p,
                                                     int t, int p)
 {
@@ -187,7 +187,7 @@ __device__ __forceinline__ void moments_partial_body(const double *__restrict__ 
 
 // The elites' deviations from the best elite in FP64, y_j = x_(j) - x_(1) (exact: both are
 // FP32), and w_j y_j, once per update for every tile of the moments.
-__device__ __forceinline__ void moments_prep_body(const float *__restrict__ elites, const double *__restrict__ w,
+__device__ __forceinline__ void moments_prep_body(const float *elites, const double *w,
                                                  int nu, int D, double *Y, double *WY, int idx)
 {
     if (idx >= nu * D) return;
@@ -197,7 +197,7 @@ __device__ __forceinline__ void moments_prep_body(const float *__restrict__ elit
     WY[idx] = w[j] * y;
 }
 
-__global__ void k_moments_prep(const float *__restrict__ elites, const double *__restrict__ w, int nu, int D,
+__global__ void k_moments_prep(const float *elites, const double *w, int nu, int D,
                                double *Y, double *WY)
 {
     after_previous();
@@ -205,7 +205,7 @@ __global__ void k_moments_prep(const float *__restrict__ elites, const double *_
 }
 
 __global__ void __launch_bounds__(256)
-k_moments_partial(const double *__restrict__ Y, const double *__restrict__ WY, int nu, int D,
+k_moments_partial(const double *Y, const double *WY, int nu, int D,
                   int per, int n_chunks, double *s2p, double *s1p)
 {
     after_previous();
@@ -213,7 +213,7 @@ k_moments_partial(const double *__restrict__ Y, const double *__restrict__ WY, i
 }
 
 __global__ void __launch_bounds__(256)
-k_moments_partial_raw(const float *__restrict__ elites, const double *__restrict__ w, int nu, int D,
+k_moments_partial_raw(const float *elites, const double *w, int nu, int D,
                       int per, int n_chunks, double *s2p, double *s1p)
 {
     after_previous();
@@ -253,7 +253,7 @@ k_batch_moments_partial(const BatchQueryDev *__restrict__ qd, const int2 *__rest
 // are left out: the first term is taken as it is, and a level that pairs sums l < n with sums
 // l + off >= n does nothing (few chunks: the smallest query has four, and three additions).
 template <int G>
-__device__ __forceinline__ double tree_sum(const double *__restrict__ v, int n, size_t stride, int sub)
+__device__ __forceinline__ double tree_sum(const double *v, int n, size_t stride, int sub)
 {
     constexpr int P = 32 / G;
     double s[P];
@@ -288,7 +288,7 @@ constexpr int kSumLanes = 4;
 
 // S1 of rows 0 .. r_last into shared memory (kSumLanes lanes per row), for the entries of a block
 // of whole warps.
-__device__ __forceinline__ void stage_s1(const double *__restrict__ s1p, int n_chunks, int D, int r_last,
+__device__ __forceinline__ void stage_s1(const double *s1p, int n_chunks, int D, int r_last,
                                          double *s_s1)
 {
     const int per = (int)blockDim.x / kSumLanes, sub = (int)threadIdx.x % kSumLanes;
@@ -302,7 +302,7 @@ __device__ __forceinline__ void stage_s1(const double *__restrict__ s1p, int n_c
 
 // S1 of row r (its chunk partials summed in the fixed order above, kSumLanes lanes per row),
 // stored after the chunk partials of s1p, and mu_r = m0_r + S1_r. Called by whole warps.
-__device__ __forceinline__ void moments_s1_body(double *s1p, int n_chunks, int D, const float *__restrict__ elites,
+__device__ __forceinline__ void moments_s1_body(double *s1p, int n_chunks, int D, const float *elites,
                                                double *mu, int r, int sub)
 {
     const double s = tree_sum<kSumLanes>(s1p + min(r, D - 1), n_chunks, D, sub);
@@ -315,7 +315,7 @@ __device__ __forceinline__ void moments_s1_body(double *s1p, int n_chunks, int D
 // Lower-triangle entry e (r >= c), kSumLanes lanes per entry:
 // C[r][c] = C[c][r] = S2 - S1_r S1_c + eps [r = c], with S1 from moments_s1_body. Called by
 // whole warps.
-__device__ __forceinline__ void moments_combine_body(const double *__restrict__ s2p, const double *__restrict__ s1,
+__device__ __forceinline__ void moments_combine_body(const double *s2p, const double *s1,
                                                     int n_chunks, int D, double eps, double *C, int e, int sub)
 {
     const int entries = D * (D + 1) / 2;
@@ -331,7 +331,7 @@ __device__ __forceinline__ void moments_combine_body(const double *__restrict__ 
 
 // Blocks of 128 threads: 32 rows (entries) per block, kSumLanes lanes each.
 __global__ void __launch_bounds__(128)
-k_moments_s1(double *s1p, int n_chunks, int D, const float *__restrict__ elites, double *mu)
+k_moments_s1(double *s1p, int n_chunks, int D, const float *elites, double *mu)
 {
     after_previous();
     const int g = (int)(blockIdx.x * blockDim.x + threadIdx.x);
@@ -339,7 +339,7 @@ k_moments_s1(double *s1p, int n_chunks, int D, const float *__restrict__ elites,
 }
 
 __global__ void __launch_bounds__(128)
-k_moments_combine(const double *__restrict__ s2p, const double *__restrict__ s1, int n_chunks, int D, double eps,
+k_moments_combine(const double *s2p, const double *s1, int n_chunks, int D, double eps,
                   double *C)
 {
     after_previous();
@@ -350,8 +350,8 @@ k_moments_combine(const double *__restrict__ s2p, const double *__restrict__ s1,
 // S1, the mean (by block 0) and the entries in one launch: every block sums S1 of the rows up to its
 // last entry's itself.
 __global__ void __launch_bounds__(128)
-k_moments_final(const double *__restrict__ s2p, const double *__restrict__ s1p, int n_chunks, int D, double eps,
-                const float *__restrict__ elites, double *mu, double *C)
+k_moments_final(const double *s2p, const double *s1p, int n_chunks, int D, double eps,
+                const float *elites, double *mu, double *C)
 {
     after_previous();
     __shared__ double s_s1[4 * CP_MAX_WAYPOINTS];
@@ -407,7 +407,7 @@ __global__ void k_radix_init(const double *__restrict__ J, int N, unsigned long 
 // The digit of a pass: 8 bits of the key, or (kByQuery) 8 bits of the query of the element's
 // value (qid[value]), for the last passes of the batched ranking.
 template <bool kByQuery>
-__device__ __forceinline__ int radix_digit(unsigned long long k, int v, int shift, const uint16_t *__restrict__ qid)
+__device__ __forceinline__ int radix_digit(unsigned long long k, int v, int shift, const uint16_t *qid)
 {
     if (kByQuery) return (int)((qid[v] >> shift) & 255u);
     return (int)((k >> shift) & 255ull);
@@ -528,9 +528,9 @@ constexpr int kOnePasses = 10;   // histograms kept: eight key passes and two qu
 
 template <bool kByQuery, bool kNextByQuery>
 __global__ void __launch_bounds__(kRadixTile)
-k_radix_pass(const unsigned long long *__restrict__ key_in, const int *__restrict__ val_in, int N, int shift,
-             const int *__restrict__ hist, unsigned long long *key_out, int *val_out, int next_shift, int *hist_next,
-             const uint16_t *__restrict__ qid)
+k_radix_pass(const unsigned long long *key_in, const int *val_in, int N, int shift,
+             const int *hist, unsigned long long *key_out, int *val_out, int next_shift, int *hist_next,
+             const uint16_t *qid)
 {
     after_previous();
     __shared__ int s_before[4][256], s_total[4][256];
@@ -595,8 +595,8 @@ k_radix_pass(const unsigned long long *__restrict__ key_in, const int *__restric
 }
 
 // Elite list and rows from the sorted indices; rank 0 also records its cost.
-__device__ __forceinline__ void gather_body(const int *__restrict__ sorted, int base, const double *__restrict__ J,
-                                            const float *__restrict__ xi, int nu, int D, int *elite, float *elites,
+__device__ __forceinline__ void gather_body(const int *sorted, int base, const double *J,
+                                            const float *xi, int nu, int D, int *elite, float *elites,
                                             double *best_J, int r, int n_valid = 0x7FFFFFFF,
                                             uint32_t *status = nullptr)
 {
@@ -614,8 +614,8 @@ __device__ __forceinline__ void gather_body(const int *__restrict__ sorted, int 
     for (int c = lane; c < D; c += 32) elites[(size_t)r * D + c] = xi[(size_t)i * D + c];
 }
 
-__global__ void k_gather_elites(const int *__restrict__ sorted, const double *__restrict__ J,
-                                const float *__restrict__ xi, int nu, int D, int *elite,
+__global__ void k_gather_elites(const int *sorted, const double *J,
+                                const float *xi, int nu, int D, int *elite,
                                 float *elites, double *best_J)
 {
     after_previous();
@@ -679,8 +679,8 @@ __global__ void k_cma_reset(double sigma0, int D, double *cma, double *p_sigma, 
 // runs the substitution column by column, lane l holding rows l, l + 32, l + 64, l + 96,
 // each new z_j passed by a shuffle, so the dependent chain has no block barrier.
 __global__ void __launch_bounds__(kCmaThreads)
-k_cma_paths(const double *__restrict__ s1p, int n_chunks, int D, const float *__restrict__ elites,
-            double *__restrict__ mu_prev, const double *__restrict__ L, CmaConsts k, double path_len, double path_max,
+k_cma_paths(const double *s1p, int n_chunks, int D, const float *elites,
+            double *mu_prev, const double *L, CmaConsts k, double path_len, double path_max,
             double *mu, double *p_sigma, double *p_c, double *cma)
 {
     after_previous();
@@ -761,9 +761,9 @@ k_cma_paths(const double *__restrict__ s1p, int n_chunks, int D, const float *__
 // the moments about x_(1) (with d = x_(1) - m and weights summing to one:
 // S2 + S1 d^T + d S1^T + d d^T), then C' = a C + c_1 p_c p_c^T + c_mu scatter / sigma^2 with
 // a = 1 + c_1 (1 - h_sigma) c_c (2 - c_c) - c_1 - c_mu.
-__global__ void __launch_bounds__(128) k_cma_cov(const double *__restrict__ s2p, const double *__restrict__ s1p, int n_chunks,
-                          int D, const float *__restrict__ elites, const double *__restrict__ mu_prev,
-                          const double *__restrict__ p_c, const double *__restrict__ cma, CmaConsts k,
+__global__ void __launch_bounds__(128) k_cma_cov(const double *s2p, const double *s1p, int n_chunks,
+                          int D, const float *elites, const double *mu_prev,
+                          const double *p_c, const double *cma, CmaConsts k,
                           double *C)
 {
     after_previous();
