@@ -209,6 +209,7 @@ struct cp_planner {
     int plan_start = -1, plan_iters = -1;
     SceneDev plan_sdev{};
     PolarDev plan_gdev{};
+    float plan_reach_extra = 0.f;
     bool plan_ready_before = false, plan_ready_after = false;
     bool plan_metrics = false;
     int64_t plan_nodes = 0;   // kernels in the recorded graph
@@ -1031,14 +1032,16 @@ bool same_grid(const PolarDev &a, const PolarDev &b)
 }
 
 // The iterations of cp_plan from p->iteration as one CUDA graph launch, recorded on first
-// use and again whenever the start iteration, the count or the scene records (kernel
-// arguments of the recorded launches) differ from the recorded ones. Every evaluation form
+// use and again whenever the start iteration, the count, the scene records or the hull form's
+// reach over the scene's prisms (kernel arguments of the recorded launches) differ from the
+// recorded ones. Every evaluation form
 // takes the end points from the device copy that cp_set_endpoints writes in stream order.
 int run_plan_graph(cp_planner *p, int iters)
 {
     const bool same = p->plan_exec && p->plan_start == p->iteration && p->plan_iters == iters &&
                       p->plan_ready_before == p->elites_ready && p->plan_metrics == p->metrics_on &&
-                      same_scene(p->plan_sdev, p->sdev) && same_grid(p->plan_gdev, p->gdev);
+                      same_scene(p->plan_sdev, p->sdev) && same_grid(p->plan_gdev, p->gdev) &&
+                      p->plan_reach_extra == p->hull_reach_extra;
     const int start = p->iteration;
     const bool ready_before = p->elites_ready;
     if (!same) {
@@ -1078,6 +1081,7 @@ int run_plan_graph(cp_planner *p, int iters)
         p->plan_metrics = p->metrics_on;
         p->plan_sdev = p->sdev;
         p->plan_gdev = p->gdev;
+        p->plan_reach_extra = p->hull_reach_extra;
     }
     CP_CUDA(cudaGraphLaunch(p->plan_exec, p->st));
     g_launches.fetch_add(p->plan_nodes, std::memory_order_relaxed);
