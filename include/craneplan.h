@@ -268,9 +268,7 @@ int cp_evaluate(cp_planner *p, const float *d_xi, int32_t n, double *d_J, uint8_
 /* Algorithm 1 steps (3)-(6) for the N candidates d_xi with costs d_J (double[N], NaN
  * ranks last, ties go to the lower index): mu <- sum_j w_j xi_(j),
  * C <- sum_j w_j (xi_(j) - mu)(xi_(j) - mu)^T + eps I with the new mu, then factor
- * sigma^2 C for the next sample and advance the iteration counter. From nu D^2 = 2^23 on (paper
- * rule, factor sampler) mu and C come from integer sums, nearer to the exact values than FP64
- * additions: they agree with a cp_plan iteration's to rounding, not bit for bit.
+ * sigma^2 C for the next sample and advance the iteration counter.
  * Errors: CP_ERR_STATE, CP_ERR_ARG, CP_ERR_NUMERIC (reported by the next host-synchronising call). */
 int cp_update(cp_planner *p, const double *d_J, const float *d_xi);
 

@@ -159,9 +159,6 @@ struct cp_planner {
     float *elites = nullptr;
     double *w = nullptr, *mean_part = nullptr, *cov_part = nullptr;
     double *mom_y = nullptr;    // [2][nu][D] FP64 deviations of the elites for the moments
-    bool use_tc = false;        // cp_update's moments in their tensor-core form (a rule on nu and D; paper update)
-    MomentsTc tc{};
-    int tc_parts = 0;
     double *best = nullptr;
     uint32_t *status = nullptr;
     double *ctrl = nullptr;
@@ -539,13 +536,7 @@ int run_sample(cp_planner *p, int iter, float *d_xi)
     return p->timer.end(ST_SAMPLE, p->st);
 }
 
-int run_moments(cp_planner *p, double *mu, bool use_tc);
-
-// use_tc: the moments in integers on the tensor cores. Only an update by itself may take them
-// (cp_update): they are nearer to the exact sums than FP64 additions are, but differ from them in
-// the last bits, and over the iterations of a plan such a difference grows (over 17 plans of 5 to
-// 100 iterations, three ended with another covariance, by up to 1e-2).
-int run_update(cp_planner *p, const double *d_J, const float *d_xi, bool use_tc)
+int run_update(cp_planner *p, const double *d_J, const float *d_xi)
 {
     NvtxRange range("craneplan:update");
     int rc = p->timer.begin(p->st);
@@ -579,25 +570,14 @@ int run_update(cp_planner *p, const double *d_J, const float *d_xi, bool use_tc)
         p->elites_ready = true;
         p->iteration += 1;
         return CP_OK;
-    } else if ((rc = run_moments(p, p->mu, use_tc)) != CP_OK) {
+    } else if ((rc = launch_moments(p->elites, p->w, p->nu, p->D, p->prm.eps, p->mom_y, p->cov_part, p->mean_part,
+                                    p->mu, p->C, p->st)) != CP_OK) {
         return rc;
     }
     if ((rc = p->timer.end(ST_UPDATE, p->st)) != CP_OK) return rc;
     if ((rc = run_factor(p)) != CP_OK) return rc;
     p->iteration += 1;
     return CP_OK;
-}
-
-// Mean and covariance of the current elites into `mu` and the planner's C.
-int run_moments(cp_planner *p, double *mu, bool use_tc)
-{
-    if (use_tc) {
-        MomentsTc a = p->tc;
-        a.mu = mu;
-        return launch_moments_tc(a, p->tc_parts, p->num_sms, p->st);
-    }
-    return launch_moments(p->elites, p->w, p->nu, p->D, p->prm.eps, p->mom_y, p->cov_part, p->mean_part, mu, p->C,
-                          p->st);
 }
 
 // With the factor-free sampler after an update, C (and its factor) exist only on request:
@@ -607,7 +587,8 @@ int materialise_distribution(const cp_planner *p)
 {
     if (!p->elites_ready) return CP_OK;
     cp_planner *q = const_cast<cp_planner *>(p);
-    int rc = run_moments(q, q->mu_prev, false);
+    int rc = launch_moments(q->elites, q->w, q->nu, q->D, q->prm.eps, q->mom_y, q->cov_part, q->mean_part, q->mu_prev, q->C,
+                            q->st);
     if (rc != CP_OK) return rc;
     return launch_factor(q->C, q->prm.sigma * q->prm.sigma, nullptr, q->D, q->L, q->Lt, q->status, q->st);
 }
@@ -629,7 +610,7 @@ int run_iteration(cp_planner *p)
     int rc;
     if ((rc = run_sample(p, p->iteration, p->xi)) != CP_OK) return rc;
     if ((rc = run_eval(p, p->xi, p->N, p->J, p->flag, nullptr, nullptr, nullptr)) != CP_OK) return rc;
-    if ((rc = run_update(p, p->J, p->xi, false)) != CP_OK) return rc;
+    if ((rc = run_update(p, p->J, p->xi)) != CP_OK) return rc;
     return record_metrics(p);
 }
 
@@ -743,9 +724,6 @@ int cp_plan_init(const cp_model *model, const cp_scene *scene, const cp_params *
     if ((rc = factor_configure()) != CP_OK) return fail(rc);
     if ((rc = sample_configure()) != CP_OK) return fail(rc);
     if ((rc = update_configure()) != CP_OK) return fail(rc);
-    p->use_tc = p->prm.update_rule == CP_UPDATE_PAPER && p->prm.sampler == CP_SAMPLE_FACTOR && moments_use_tc(p->nu, p->D);
-    if (p->use_tc && (rc = moments_tc_configure()) != CP_OK) return fail(rc);
-    p->tc_parts = p->use_tc ? moments_tc_parts(p->nu, p->D, p->num_sms) : 0;
 
     const size_t N = p->N, D = p->D, nu = p->nu, ch = p->chunks, mc = p->n_mean_chunks;
     Layout L;
@@ -775,17 +753,9 @@ int cp_plan_init(const cp_model *model, const cp_scene *scene, const cp_params *
     const size_t o_elite = L.take<int>(nu);
     const size_t o_elites = L.take<float>(nu * D);
     const size_t o_w = L.take<double>(nu);
-    const bool tc = p->use_tc;
     const size_t o_mean_part = L.take<double>((mc + 1) * D);   // chunk partials, then S1
     const size_t o_cov_part = L.take<double>(mc * D * D);
     const size_t o_mom_y = L.take<double>(2 * nu * D);
-    const size_t tc_n = tc ? moments_tc_partial(p->D, p->tc_parts) : 1;
-    const size_t o_tc_hi = L.take<long long>(tc_n);
-    const size_t o_tc_lo = L.take<long long>(tc_n);
-    const size_t o_tc_s1 = L.take<long long>(tc ? (size_t)p->tc_parts * kMomentCols : 1);
-    const size_t o_tc_W = L.take<long long>(tc ? 2 * nu : 1);
-    const size_t o_tc_max = L.take<uint32_t>(kMomentCols);
-    const size_t o_tc_scale = L.take<int>(2);
     const size_t o_best = L.take<double>(1);
     const size_t o_status = L.take<uint32_t>(1);
     const size_t o_ctrl = L.take<double>(4 * ((size_t)p->K + 8));
@@ -859,24 +829,6 @@ int cp_plan_init(const cp_model *model, const cp_scene *scene, const cp_params *
     p->cov_part = (double *)(b + o_cov_part);
     p->mom_y = (double *)(b + o_mom_y);
     p->best = (double *)(b + o_best);
-    if (tc) {
-        MomentsTc &t = p->tc;
-        t.elites = p->elites;
-        t.w = p->w;
-        t.W = (long long *)(b + o_tc_W);
-        t.Wf = t.W + nu;
-        t.scale = (int *)(b + o_tc_scale);
-        t.nu = p->nu;
-        t.D = p->D;
-        t.colmax = (uint32_t *)(b + o_tc_max);
-        t.hi = (long long *)(b + o_tc_hi);
-        t.lo = (long long *)(b + o_tc_lo);
-        t.s1 = (long long *)(b + o_tc_s1);
-        t.mu = p->mu;
-        t.C = p->C;
-        t.eps = p->prm.eps;
-        t.status = (uint32_t *)(b + o_status);
-    }
     p->status = (uint32_t *)(b + o_status);
     p->ctrl = (double *)(b + o_ctrl);
     p->mean_xi = (float *)(b + o_mean_xi);
@@ -933,9 +885,6 @@ int cp_plan_init(const cp_model *model, const cp_scene *scene, const cp_params *
     if ((rc = stage_scene(p, scene)) != CP_OK) return fail(rc);
     if ((rc = launch_basis_table(p->S, p->basis, p->st)) != CP_OK) return fail(rc);
     if ((rc = launch_weights(p->nu, p->w, p->mean_part, p->st)) != CP_OK) return fail(rc);
-    if (p->use_tc && (rc = launch_moments_tc_weights(p->w, p->nu, (long long *)p->tc.W, (long long *)p->tc.Wf,
-                                                     (int *)p->tc.scale, p->st)) != CP_OK)
-        return fail(rc);
     if (p->prm.sampler == CP_SAMPLE_ELITES &&
         (rc = launch_elite_weights(p->w, p->nu, p->prm.sigma, p->elite_sw, p->st)) != CP_OK)
         return fail(rc);
@@ -1014,7 +963,7 @@ int cp_update(cp_planner *p, const double *d_J, const float *d_xi)
     if (!p || !d_J || !d_xi) return set_error("NULL argument"), CP_ERR_ARG;
     if (!aligned16(d_xi)) return set_error("d_xi is not 16-byte aligned"), CP_ERR_ARG;
     if (!p->have_endpoints) return set_error("set the end points first"), CP_ERR_STATE;
-    return run_update(p, d_J, d_xi, p->use_tc);
+    return run_update(p, d_J, d_xi);
 }
 
 bool same_scene(const SceneDev &a, const SceneDev &b)

@@ -331,21 +331,6 @@ struct BatchEvalDev {          // what the evaluation of one query reads (restag
     PolarDev g;
 };
 
-// Operands of the tensor-core form of the moments (k_moments_tc.cu).
-constexpr int kMomentCols = 128;   // columns of a colmax array, rows of the partials
-struct MomentsTc {
-    const float *elites;             // [nu][D] in rank order
-    const double *w;                 // [nu] weights, largest first
-    const long long *W, *Wf;         // [nu] integer sqrt(w_j) and w_j
-    const int *scale;                // [2] their exponents
-    int nu, D;
-    uint32_t *colmax;                // [128] bits of the largest |x_j - x_1| per column (zeroed before)
-    long long *hi, *lo, *s1;         // partial integer sums of the parts
-    double *mu, *C;
-    double eps;
-    uint32_t *status;
-};
-
 struct BatchQueryDev {
     int N, K, D, nu;
     double *J;                       // [N] costs of the population
@@ -399,13 +384,6 @@ int launch_batch_gather(const BatchQueryDev *qd, const int2 *tab, int blocks, co
 int launch_batch_moments(const BatchQueryDev *qd, int nq, const int2 *tab_prep, int blocks_prep,
                          const int2 *tab_partial, int blocks_partial, const int2 *tab_combine, int blocks_combine,
                          cudaStream_t st);
-bool moments_use_tc(int nu, int D);   // the form of the moments, a function of nu and D alone
-int moments_tc_tiles(int D);
-int moments_tc_parts(int nu, int D, int num_sms);
-size_t moments_tc_partial(int D, int parts);   // integers of each of hi and lo
-int moments_tc_configure();
-int launch_moments_tc_weights(const double *w, int nu, long long *W, long long *Wf, int *scale, cudaStream_t st);
-int launch_moments_tc(const MomentsTc &a, int parts, int num_sms, cudaStream_t st);
 int moments_chunking(int nu, int D, int *per);   // chunks of the moment partials and elites per chunk
 int launch_batch_outputs(const BatchQueryDev *qd, int nq, bool mean_candidate, double *out, int out_stride,
                          cudaStream_t st);

@@ -1,11 +1,10 @@
 // Thin inline-PTX wrappers for the fifth-generation tensor cores of sm_100-family parts
 // (tcgen05: accumulators in tensor memory, operands described by shared-memory matrix
 // descriptors), mbarriers and bulk copies. Only what the kernels of this library use:
-// kind::tf32 and kind::f16 (BF16) MMAs with M = 128 on one CTA, K-major operands without
-// swizzling.
+// kind::tf32 MMAs with M = 128 on one CTA, K-major operands without swizzling.
 //
-// Operand layout (K-major, no swizzle; BF16 the same with 8 elements of K per core matrix). A
-// tile of R rows (M or N) by C elements of K, with 4-byte elements, is stored as "core matrices" of 8 rows x 16 bytes (4 elements of K),
+// Operand layout (K-major, no swizzle). A tile of R rows (M or N) by C elements of K, with
+// 4-byte elements, is stored as "core matrices" of 8 rows x 16 bytes (4 elements of K),
 // each core matrix 128 contiguous bytes (row r of the core at byte 16 r). Core (g, kc),
 // g = row / 8 and kc = k / 4, starts at byte (g * (C / 4) + kc) * 128, so cores adjacent
 // along K are 128 bytes apart (the descriptor's leading-dimension offset) and cores
@@ -126,25 +125,6 @@ static __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v)
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// 8 consecutive columns of this thread's lane, as tmem_ld16, without the wait: the registers
-// hold the values only after tmem_ld_wait() (several loads can be in flight before it).
-static __device__ __forceinline__ void tmem_ld8_async(uint32_t taddr, uint32_t *r)
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr));
-}
-
-// Waits for this thread's tensor-memory loads; passing the registers through keeps their uses
-// behind the wait.
-template <int N>
-static __device__ __forceinline__ void tmem_ld_wait(uint32_t *r)
-{
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < N; ++i) asm volatile("" : "+r"(r[i]));
-}
-
 // ---------------------------------------------------------------- MMA
 
 // Shared-memory matrix descriptor, K-major, no swizzle: start address, leading-dimension
@@ -161,24 +141,6 @@ static __device__ __forceinline__ uint64_t desc_kmajor(uint32_t saddr, uint32_t 
 static __host__ __device__ constexpr uint32_t idesc_tf32(int M, int N)
 {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-// Instruction descriptor of kind::f16 with BF16 operands (bits 7-9 and 10-12 = 1), otherwise as
-// above.
-static __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N)
-{
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-// D[tmem] (+)= A B^T for one K step of 16 BF16 elements; issued by one thread.
-static __device__ __forceinline__ void mma_f16kind(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                                   bool accumulate)
-{
-    asm volatile("{\n\t.reg .pred p;\n\t"
-                 "setp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                 :: "r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate)
-                 : "memory");
 }
 
 // D[tmem] (+)= A B^T for one K step of 8 TF32 elements; issued by one thread.
