@@ -30,6 +30,7 @@ constexpr int kEvalBroadMinBlocks = CP_EVAL_BROAD_MIN_BLOCKS;
 constexpr int kObstaclesPerBranch = 2;   // obstacles tested between two branches
 constexpr long long kStagingWaitCycles = 2000000000ll;   // about one second at 2 GHz
 constexpr int kCtrlSlots = CP_MAX_WAYPOINTS + 8;         // control points per warp, float4
+constexpr size_t kRoomySmem = 224 * 1024;                // up to here the static shared memory fits beside it
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
 {
@@ -365,32 +366,50 @@ __global__ void k_signed_distance(const ModelDev m, const SceneDev sc, const flo
 }
 
 template <typename F>
-int eval_grid(F *kernel, size_t smem, int num_sms, int units, int ctas_per_sm)
+int eval_grid(F *kernel, int threads, size_t smem, int num_sms, int units, int ctas_per_sm)
 {
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kEvalThreads, smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
     if (e != cudaSuccess || per_sm < 1) per_sm = 1;
     if (ctas_per_sm > 0 && ctas_per_sm < per_sm) per_sm = ctas_per_sm;
-    const int warps_per_block = kEvalThreads / 32;
+    const int warps_per_block = threads / 32;
     const int needed = (units + warps_per_block - 1) / warps_per_block;
     int grid = num_sms * per_sm;
     if (grid > needed) grid = needed;
     return grid < 1 ? 1 : grid;
 }
 
-}  // namespace
-
-size_t eval_smem_bytes(int n_cyl, int n_box, int S)
+// Dynamic shared memory of a CTA of `threads` threads.
+size_t eval_cta_bytes(int n_cyl, int n_box, int S, int threads)
 {
     return sizeof(float4) * (2 * (size_t)n_cyl + 2 * (size_t)n_box + 2 * (size_t)S +
-                             (size_t)n_groups(n_cyl) + (size_t)(kEvalThreads / 32) * kCtrlSlots);
+                             (size_t)n_groups(n_cyl) + (size_t)(threads / 32) * kCtrlSlots);
 }
+
+// Dynamic shared memory that a block can have beside the kernel's own static shared memory.
+template <typename F>
+int dynamic_smem_limit(F *fn, cudaFuncAttributes &at, size_t *limit)
+{
+    int dev = 0, optin = 0;
+    CP_CUDA(cudaGetDevice(&dev));
+    CP_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    CP_CUDA(cudaFuncGetAttributes(&at, fn));
+    *limit = (size_t)optin - at.sharedSizeBytes;
+    return CP_OK;
+}
+
+}  // namespace
+
+size_t eval_smem_bytes(int n_cyl, int n_box, int S) { return eval_cta_bytes(n_cyl, n_box, S, kEvalThreads); }
 
 template <typename F>
 int raise_smem(F *fn, size_t smem_bytes)
 {
     cudaFuncAttributes at{};
-    CP_CUDA(cudaFuncGetAttributes(&at, fn));
+    size_t limit = 0;
+    const int rc = dynamic_smem_limit(fn, at, &limit);
+    if (rc != CP_OK) return rc;
+    if (smem_bytes > limit) smem_bytes = limit;   // launch_eval keeps within it
     if ((size_t)at.maxDynamicSharedSizeBytes < smem_bytes)
         CP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes));
     return CP_OK;
@@ -415,11 +434,27 @@ int launch_eval(const ModelDev &m, const SceneDev &sc, const EvalArgs &a, int nu
 {
     const int units = a.n * a.P;   // work items
     if (units == 0) return CP_OK;
-    const size_t smem = eval_smem_bytes(sc.n_cyl, sc.n_box, a.S);
+    size_t smem = eval_smem_bytes(sc.n_cyl, sc.n_box, a.S);
     const bool plain = a.words_out == nullptr && a.pen_out == nullptr && !a.want_len;
     auto kern = m.n_spheres == 12 ? (a.broadphase ? (plain ? k_eval_broad<12, true> : k_eval_broad<12, false>) : k_eval<12>)
                                   : (a.broadphase ? (plain ? k_eval_broad<16, true> : k_eval_broad<16, false>) : k_eval<16>);
-    launch_chained(kern, eval_grid(kern, smem, num_sms, units, a.ctas_per_sm), kEvalThreads, smem, st, m, sc, a);
+    // The bound on the scenes counts the dynamic shared memory of eight warps against all that a block
+    // can have. In its last few hundred bytes that leaves no room for the kernel's static shared
+    // memory (the sphere table and the barrier): such a scene runs with one warp fewer, whose
+    // control points take more than that.
+    int threads = kEvalThreads;
+    static_assert(kCtrlSlots * sizeof(float4) >= sizeof(SphereTable<16>) + 64, "a warp's share covers the static part");
+    if (smem > kRoomySmem) {
+        cudaFuncAttributes at{};
+        size_t limit = 0;
+        const int rc = dynamic_smem_limit(kern, at, &limit);
+        if (rc != CP_OK) return rc;
+        if (smem > limit) {
+            threads -= 32;
+            smem = eval_cta_bytes(sc.n_cyl, sc.n_box, a.S, threads);
+        }
+    }
+    launch_chained(kern, eval_grid(kern, threads, smem, num_sms, units, a.ctas_per_sm), threads, smem, st, m, sc, a);
     CP_LAUNCHED("k_eval");
     return CP_OK;
 }
