@@ -223,6 +223,11 @@ int64_t cp_launch_count(void);
  * CP_ERR_OOM after releasing what it holds. n = 0 turns it off; no other effect. */
 void cp_debug_fail_allocations(int32_t n);
 
+/* Test hook: the next n evaluations of a planner (cp_evaluate, each iteration of cp_plan and its
+ * final one) return CP_ERR_CUDA between their main kernel and the launch that sums its results, as
+ * if that launch had failed. n = 0 turns it off; no other effect. */
+void cp_debug_fail_evaluations(int32_t n);
+
 /* Create a planner on the current CUDA device: validates the model, scene and parameters,
  * allocates the device workspace for N candidates, stages the scene (host -> device) and
  * tabulates the spline basis. End points must be set with cp_set_endpoints before

@@ -21,6 +21,7 @@ namespace {
 thread_local char g_err[512] = "";
 std::atomic<int64_t> g_launches{0};
 std::atomic<int32_t> g_fail_allocs{0};   // test hook: workspace allocations still to fail
+std::atomic<int32_t> g_fail_evals{0};    // test hook: evaluations still to fail before their sums
 }  // namespace
 
 void set_error(const char *fmt, ...)
@@ -169,6 +170,7 @@ struct cp_planner {
     float4 *ends_f = nullptr;   // [2] {q0, qd} in float, written with the end points
     unsigned long long *work = nullptr;   // [2] broad-phase survivors and box tests while timing
     int *eval_queue = nullptr;            // [2] item counters of the evaluation and of the smooth cost
+    bool queue_stale = false;             // an evaluation failed before its sums, which clear the counter
     size_t item_cap = 0;                  // work items the item_sum / item_count buffers hold
     unsigned long long *rkey_a = nullptr, *rkey_b = nullptr;   // radix sort scratch
     int *rval_a = nullptr, *rval_b = nullptr, *rhist = nullptr;
@@ -492,6 +494,17 @@ int run_eval(cp_planner *p, const float *d_xi, int n, double *d_J, uint8_t *d_fl
     a.item_count = p->item_count;
     a.words_out = d_words;
     a.pen_out = d_pen;
+    // The counter is zero between evaluations, as the launch of the sums clears it. After an
+    // evaluation that returned before that launch it is cleared here; while a caller records, the
+    // record clears it when it is run, and the next call has to clear it again.
+    bool still_stale = false;
+    if (p->queue_stale) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        CP_CUDA(cudaStreamIsCapturing(p->st, &cap));
+        still_stale = cap != cudaStreamCaptureStatusNone;
+        CP_CUDA(cudaMemsetAsync(p->eval_queue, 0, sizeof(int), p->st));
+    }
+    p->queue_stale = true;
     int rc = p->timer.begin(p->st);
     if (rc != CP_OK) return rc;
     if (p->prm.collision_model == CP_COLLISION_HULLS) {
@@ -505,8 +518,14 @@ int run_eval(cp_planner *p, const float *d_xi, int n, double *d_J, uint8_t *d_fl
     if (rc != CP_OK) return rc;
     rc = p->timer.end(ST_EVAL, p->st);
     if (rc != CP_OK) return rc;
-    return launch_eval_finalize(p->item_sum, p->item_count, n, a.P, p->prm.w_c, p->prm.w_l, p->prm.lambda_c,
-                                d_J, d_flag, d_terms, p->st, nullptr, p->eval_queue);
+    int32_t fail = g_fail_evals.load();
+    while (fail > 0 && !g_fail_evals.compare_exchange_weak(fail, fail - 1)) {
+    }
+    if (fail > 0) return set_error("evaluation failed by cp_debug_fail_evaluations"), CP_ERR_CUDA;
+    rc = launch_eval_finalize(p->item_sum, p->item_count, n, a.P, p->prm.w_c, p->prm.w_l, p->prm.lambda_c,
+                              d_J, d_flag, d_terms, p->st, nullptr, p->eval_queue);
+    p->queue_stale = rc != CP_OK || still_stale;
+    return rc;
 }
 
 int run_factor(cp_planner *p)
@@ -645,6 +664,8 @@ int32_t cp_version(void) { return CP_VERSION; }
 int64_t cp_launch_count(void) { return g_launches.load(); }
 
 void cp_debug_fail_allocations(int32_t n) { g_fail_allocs.store(n > 0 ? n : 0); }
+
+void cp_debug_fail_evaluations(int32_t n) { g_fail_evals.store(n > 0 ? n : 0); }
 
 int cp_plan_init(const cp_model *model, const cp_scene *scene, const cp_params *params,
                  void *stream, cp_planner **out)

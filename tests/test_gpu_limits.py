@@ -74,3 +74,55 @@ def test_scene_at_the_shared_memory_limit(lib, crane, short, sixteen):
     with pytest.raises(lib.CranePlanError) as e:
         lib.Planner(crane, one_more, lib.make_params(n, K, S))
     assert e.value.status == -1 and "shared memory" in str(e.value)
+
+
+@pytest.mark.parametrize("form", ["polar", "broad", "exhaustive", "hulls"])
+@pytest.mark.parametrize("stream", [False, True])
+def test_calls_after_a_failed_evaluation(lib, crane, form, stream):
+    """An evaluation that fails between its main kernel and its sums (on the host: cp_evaluate, and
+    an iteration of a plan, recorded on a stream of its own) leaves nothing that a later call takes
+    for its own: the next evaluations and plans are right without new end points."""
+    import torch
+    from paper_2503_14160_gb300 import workloads
+    kw = {"polar": {"grid_cell": 0.5}, "exhaustive": {"eval_exhaustive": 1},
+          "hulls": {"collision_model": lib.CP_COLLISION_HULLS}}.get(form, {})
+    scene = workloads.make_scene(workloads.WORKLOADS["single_small"])
+    n, K, S = 300, 5, 9
+    st = torch.cuda.Stream() if stream else None
+    x = [torch.from_numpy(workloads.random_candidates(Q0, QD, K, n, seed=seed)).cuda() for seed in (1, 2)]
+    torch.cuda.synchronize()
+
+    def evaluate(pl, i):
+        J = torch.full((n,), -1.0, dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        lib.cp_evaluate(pl.handle, x[i], n, J)
+        lib.cp_synchronize(pl.handle)
+        return J.cpu().numpy()
+
+    with lib.Planner(crane, scene, lib.make_params(n, K, S, **kw), st) as fresh:
+        lib.cp_set_endpoints(fresh.handle, Q0, QD)
+        want = [evaluate(fresh, 0), evaluate(fresh, 1)]
+        lib.cp_set_endpoints(fresh.handle, Q0, QD)
+        want_plan = lib.cp_plan(fresh.handle, 3, K=K)
+    with lib.Planner(crane, scene, lib.make_params(n, K, S, **kw), st) as pl:
+        lib.cp_set_endpoints(pl.handle, Q0, QD)
+        try:
+            lib.cp_debug_fail_evaluations(1)
+            with pytest.raises(lib.CranePlanError) as e:
+                evaluate(pl, 0)
+            assert e.value.status == -2
+            assert np.array_equal(evaluate(pl, 1), want[1])
+            lib.cp_debug_fail_evaluations(2)
+            for _ in range(2):
+                with pytest.raises(lib.CranePlanError):
+                    lib.cp_plan(pl.handle, 3, K=K)
+        finally:
+            lib.cp_debug_fail_evaluations(0)
+        assert np.array_equal(evaluate(pl, 0), want[0])
+        assert np.array_equal(evaluate(pl, 1), want[1])
+        if stream:   # its recording failed, so no iteration has run: the plan from the start
+            ctrl, stats = lib.cp_plan(pl.handle, 3, K=K)
+            assert np.array_equal(ctrl, want_plan[0]) and stats == want_plan[1]
+        lib.cp_set_endpoints(pl.handle, Q0, QD)
+        ctrl, stats = lib.cp_plan(pl.handle, 3, K=K)
+        assert np.array_equal(ctrl, want_plan[0]) and stats == want_plan[1]
