@@ -121,6 +121,8 @@ __device__ __forceinline__ bool unit_axis(float3 &L)
 // Smallest overlap over the axes of (box a, prism at centre pc) or (box a, axis-aligned box
 // with half extents bh), or any overlap at most `floor` as soon as one is met: such a pair
 // cannot raise a running maximum that stands at floor >= 0, so the rest of its axes is left out.
+// An axis whose overlap is NaN separates nothing: a box without a place (a NaN configuration beside
+// an obstacle) has an infinite overlap and is reported.
 // r: the box's record in shared memory, whose axes the loops over the cross products take in
 // turn: rolled, because the unrolled code outgrew the instruction cache (a third of the cycles
 // were spent waiting for instructions).
@@ -134,7 +136,7 @@ __device__ __forceinline__ float sat_prism(const Obb &a, const float *r, float3 
     const float3 d = make_float3(pc.x - a.c.x, pc.y - a.c.y, pc.z - a.c.z);
     const float h = kSqrtHalf;
     // prism faces: z, then the four side normals at multiples of 45 degrees
-    float best = prism_overlap<kZx | kZy>(a, rc, hz, d, make_float3(0.f, 0.f, 1.f));
+    float best = fminf(CUDART_INF_F, prism_overlap<kZx | kZy>(a, rc, hz, d, make_float3(0.f, 0.f, 1.f)));
     best = fminf(best, prism_overlap<kZy | kZz>(a, rc, hz, d, make_float3(1.f, 0.f, 0.f)));
     best = fminf(best, prism_overlap<kZz>(a, rc, hz, d, make_float3(h, h, 0.f)));
     best = fminf(best, prism_overlap<kZx | kZz>(a, rc, hz, d, make_float3(0.f, 1.f, 0.f)));
@@ -166,7 +168,7 @@ __device__ __forceinline__ float sat_prism(const Obb &a, const float *r, float3 
 __device__ __forceinline__ float sat_box(const Obb &a, const float *r, float3 bc, float3 bh, float floor)
 {
     const float3 d = make_float3(bc.x - a.c.x, bc.y - a.c.y, bc.z - a.c.z);
-    float best = obb_support<kZy | kZz>(a, make_float3(1.f, 0.f, 0.f)) + bh.x - fabsf(d.x);
+    float best = fminf(CUDART_INF_F, obb_support<kZy | kZz>(a, make_float3(1.f, 0.f, 0.f)) + bh.x - fabsf(d.x));
     best = fminf(best, obb_support<kZx | kZz>(a, make_float3(0.f, 1.f, 0.f)) + bh.y - fabsf(d.y));
     best = fminf(best, obb_support<kZx | kZy>(a, make_float3(0.f, 0.f, 1.f)) + bh.z - fabsf(d.z));
     if (best <= floor) return best;

@@ -1,0 +1,71 @@
+"""Candidates and configurations with NaN or infinite entries: they are reported where they are, and
+change nothing else."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lib():
+    from paper_2503_14160_gb300 import build, craneplan
+    build.build()
+    craneplan.load()
+    return craneplan
+
+
+@pytest.fixture(scope="module")
+def crane():
+    from paper_2503_14160_gb300 import workloads
+    return workloads.forestry_crane()
+
+
+Q0, QD = np.array([-0.4, 0.4, -1.2, 0.5]), np.array([0.4, 0.6, -1.8, 1.5])
+
+
+def _beside(boxes):
+    """One obstacle in the crane's reach ahead of it: a trunk or a box."""
+    from paper_2503_14160_gb300 import workloads
+    if boxes:
+        return workloads.Scene(np.zeros((0, 5)), np.array([[3.0, -2.0, 0.0, 6.0, 2.0, 15.0]]))
+    return workloads.Scene(np.array([[4.0, 0.0, 0.5, 0.0, 15.0]]), np.zeros((0, 6)))
+
+
+@pytest.mark.parametrize("boxes", [False, True])
+@pytest.mark.parametrize("joint,value", [(2, np.nan), (3, np.nan)])
+def test_hulls_report_a_nan_configuration(lib, crane, boxes, joint, value):
+    """Hulls without a place beside an obstacle in the reach of the others have no separating axis:
+    the depth is infinite, not 0."""
+    import torch
+    q = np.array([[0.0, 0.4, -1.0, 0.5], [0.0, 0.4, -1.0, 0.5]], np.float32)
+    q[1, joint] = value
+    with lib.Planner(crane, _beside(boxes), lib.make_params(4, 2, 2)) as pl:
+        pen = torch.full((2,), -1.0, device="cuda")
+        lib.cp_hull_penetration(pl.handle, torch.from_numpy(q).cuda(), 2, pen)
+        torch.cuda.synchronize()
+        pen = pen.cpu().numpy()
+    assert np.isfinite(pen[0]) and pen[0] > 0.0
+    assert pen[1] == np.inf
+
+
+@pytest.mark.parametrize("boxes", [False, True])
+def test_hull_paths_report_nan_checkpoints(lib, crane, boxes):
+    import torch
+    K, S = 8, 8
+    f = (np.arange(1, K + 1) / (K + 1))[:, None]
+    xi = np.repeat((Q0 + f * (QD - Q0))[None], 2, 0).astype(np.float32)
+    xi[1, 3, 3] = np.nan
+    with lib.Planner(crane, _beside(boxes), lib.make_params(2, K, S, collision_model=lib.CP_COLLISION_HULLS)) as pl:
+        lib.cp_set_endpoints(pl.handle, Q0, QD)
+        J = torch.zeros(2, dtype=torch.float64, device="cuda")
+        flag = torch.zeros(2, dtype=torch.uint8, device="cuda")
+        pen = torch.zeros(2, pl.n_s, device="cuda")
+        lib.cp_evaluate(pl.handle, torch.from_numpy(xi).cuda(), 2, J, flag, None, None, pen)
+        lib.cp_synchronize(pl.handle)
+        J, flag, pen = J.cpu().numpy(), flag.cpu().numpy(), pen.cpu().numpy()
+    # control point 3 (the seventh in all) acts on spans 3 .. 6 of the path
+    near = pen[0, 3 * S:7 * S] > 0.0
+    assert near.any() and np.isfinite(J[0])
+    assert np.all(pen[1, 3 * S:7 * S][near] == np.inf)
+    assert np.array_equal(pen[1, :3 * S], pen[0, :3 * S]) and np.array_equal(pen[1, 7 * S:], pen[0, 7 * S:])
+    assert flag[1] == 1 and not np.isfinite(J[1])
