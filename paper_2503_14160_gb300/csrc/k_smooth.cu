@@ -350,20 +350,24 @@ k_smooth(const ModelDev m, const SceneDev sc, const SmoothArgs a)
                 const float4 r = make_float4(fmaf(a.wc_lc, sum.ht, a.w_l * lim2.x), fmaf(a.wc_lc, r1, a.w_l * lim2.y),
                                              fmaf(a.wc_lc, r2, a.w_l * lim2.z), fmaf(a.wc_lc, r3, a.w_l * lim2.w));
                 // contribution to control point span+1+i: 2 dq db_i + r b_i, summed over the lanes
-                // of each span the chunk covers (one or two when S >= 32)
+                // of each span the chunk covers (one or two when S >= 32). The other lanes' dq and r
+                // are taken as 0, not multiplied by it: a checkpoint without a finite gradient
+                // spoils its own control points only.
                 const float4 bw = s_basis[2 * (mstep - 1)], dbw = s_basis[2 * (mstep - 1) + 1];
                 const int sp_lo = __shfl_sync(0xffffffffu, span, 0), sp_hi = __shfl_sync(0xffffffffu, span, 31);
                 for (int sp = sp_lo; sp <= sp_hi; ++sp) {
                     const bool mine = valid && span == sp;
                     const float bi[4] = {bw.x, bw.y, bw.z, bw.w}, dbi[4] = {dbw.x, dbw.y, dbw.z, dbw.w};
+                    const float4 dm = make_float4(mine ? dq.x : 0.f, mine ? dq.y : 0.f, mine ? dq.z : 0.f, mine ? dq.w : 0.f);
+                    const float4 rm = make_float4(mine ? r.x : 0.f, mine ? r.y : 0.f, mine ? r.z : 0.f, mine ? r.w : 0.f);
                     float t[16];
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        const float wd = mine ? 2.f * dbi[i] : 0.f, wb = mine ? bi[i] : 0.f;
-                        t[4 * i + 0] = fmaf(wd, dq.x, wb * r.x);
-                        t[4 * i + 1] = fmaf(wd, dq.y, wb * r.y);
-                        t[4 * i + 2] = fmaf(wd, dq.z, wb * r.z);
-                        t[4 * i + 3] = fmaf(wd, dq.w, wb * r.w);
+                        const float wd = 2.f * dbi[i], wb = bi[i];
+                        t[4 * i + 0] = fmaf(wd, dm.x, wb * rm.x);
+                        t[4 * i + 1] = fmaf(wd, dm.y, wb * rm.y);
+                        t[4 * i + 2] = fmaf(wd, dm.z, wb * rm.z);
+                        t[4 * i + 3] = fmaf(wd, dm.w, wb * rm.w);
                     }
                     const float total = sum16(t, lane);
                     const int at = (sp - 3) * 4 + (lane >> 1);   // control point span + 1 + i, from the first free one

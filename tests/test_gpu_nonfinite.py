@@ -69,3 +69,35 @@ def test_hull_paths_report_nan_checkpoints(lib, crane, boxes):
     assert np.all(pen[1, 3 * S:7 * S][near] == np.inf)
     assert np.array_equal(pen[1, :3 * S], pen[0, :3 * S]) and np.array_equal(pen[1, 7 * S:], pen[0, 7 * S:])
     assert flag[1] == 1 and not np.isfinite(J[1])
+
+
+@pytest.mark.parametrize("S", [2, 8, 24, 64])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_smooth_gradient_keeps_a_bad_entry_to_its_own_control_points(lib, crane, S, bad):
+    """Control point 13 acts on four spans, and these on control points 10 .. 16: the others'
+    gradients are those of the candidate without it, bit for bit. With 8 and 24 substeps a
+    32-checkpoint chunk holds a bad span and a good one."""
+    import torch
+    from paper_2503_14160_gb300 import workloads
+    K, n = 24, 2
+    g = np.random.default_rng(S)
+    f = (np.arange(1, K + 1) / (K + 1))[:, None]
+    xi = ((Q0 + f * (QD - Q0))[None] + 0.02 * g.normal(size=(n, K, 4))).astype(np.float32)
+    scene = workloads.make_scene(workloads.WORKLOADS["single_small"])
+    out = []
+    with lib.Planner(crane, scene, lib.make_params(n, K, S)) as pl:
+        lib.cp_set_endpoints(pl.handle, Q0, QD)
+        for value in (xi[1, 13, 1], bad):
+            x = xi.copy()
+            x[1, 13, 1] = value
+            J = torch.zeros(n, dtype=torch.float64, device="cuda")
+            d = torch.zeros(n, K, 4, device="cuda")
+            lib.cp_smooth_cost_grad(pl.handle, torch.from_numpy(x).cuda(), n, None, J, d)
+            lib.cp_synchronize(pl.handle)
+            out.append((J.cpu().numpy(), d.cpu().numpy()))
+    (J0, d0), (J1, d1) = out
+    assert np.isfinite(d0).all() and np.isfinite(J0).all()
+    far = np.r_[0:10, 17:K]
+    np.testing.assert_array_equal(d1[0], d0[0])
+    np.testing.assert_array_equal(d1[1, far], d0[1, far])
+    assert J1[0] == J0[0] and not np.isfinite(J1[1]) and not np.isfinite(d1[1, 13]).all()
