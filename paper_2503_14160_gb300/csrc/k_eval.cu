@@ -228,7 +228,9 @@ k_eval_broad(const ModelDev m, const SceneDev sc, const EvalArgs a)
                     const int ob = base + __ffs(mask) - 1;
                     mask &= mask - 1;
                     const float4 cb = s_bc[ob];
-                    const uint32_t in = spheres_in_reach<NSPH>(H2, c1, s1, cb.x, cb.y, cb.w * cb.w);
+                    // a lane whose checkpoint is not finite takes every sphere, as the exhaustive form
+                    const uint32_t in = c.jp < CUDART_INF_F ? spheres_in_reach<NSPH>(H2, c1, s1, cb.x, cb.y, cb.w * cb.w)
+                                                            : (1u << NSPH) - 1u;
                     if (in) dmin = fminf(dmin, walk_box<NSPH>(s_tab, tr, m.base_z, c.q.w, in, cb, s_bh[ob]));
                 }
             }

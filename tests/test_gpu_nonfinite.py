@@ -101,3 +101,29 @@ def test_smooth_gradient_keeps_a_bad_entry_to_its_own_control_points(lib, crane,
     np.testing.assert_array_equal(d1[0], d0[0])
     np.testing.assert_array_equal(d1[1, far], d0[1, far])
     assert J1[0] == J0[0] and not np.isfinite(J1[1]) and not np.isfinite(d1[1, 13]).all()
+
+
+@pytest.mark.parametrize("joint,value", [(1, np.nan), (3, np.nan), (3, np.inf), (2, 1e30)])
+def test_broad_phase_equals_exhaustive_beside_a_box(lib, crane, joint, value):
+    """The default form and the exhaustive one give the same flags, penalties and costs for a
+    candidate with such an entry, whose checkpoints the box is close to."""
+    import torch
+    K, S, n = 8, 8, 3
+    f = (np.arange(1, K + 1) / (K + 1))[:, None]
+    xi = np.repeat((Q0 + f * (QD - Q0))[None], n, 0).astype(np.float32)
+    xi[1, 3, joint] = value
+    out = []
+    for exhaustive in (0, 1):
+        with lib.Planner(crane, _beside(True), lib.make_params(n, K, S, eval_exhaustive=exhaustive)) as pl:
+            lib.cp_set_endpoints(pl.handle, Q0, QD)
+            J = torch.zeros(n, dtype=torch.float64, device="cuda")
+            flag = torch.zeros(n, dtype=torch.uint8, device="cuda")
+            terms = torch.zeros(n, 5, dtype=torch.float64, device="cuda")
+            words = torch.zeros(n, (pl.n_s + 31) // 32, dtype=torch.int32, device="cuda")
+            pen = torch.zeros(n, pl.n_s, device="cuda")
+            lib.cp_evaluate(pl.handle, torch.from_numpy(xi).cuda(), n, J, flag, terms, words, pen)
+            lib.cp_synchronize(pl.handle)
+            out.append([t.cpu().numpy() for t in (J, flag, terms, words, pen)])
+    assert out[0][1][0] == 1
+    for a, b in zip(*out):
+        np.testing.assert_array_equal(a, b)
