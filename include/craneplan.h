@@ -223,6 +223,11 @@ int64_t cp_launch_count(void);
  * CP_ERR_OOM after releasing what it holds. n = 0 turns it off; no other effect. */
 void cp_debug_fail_allocations(int32_t n);
 
+/* Test hook: while on, a planner's factor kernel withholds one message between its thread blocks
+ * (from 20 rows on), so that a bounded wait runs out: the next host-synchronising call returns
+ * CP_ERR_TIMEOUT. No other effect. */
+void cp_debug_withhold_factor(int32_t on);
+
 /* Test hook: the next n evaluations of a planner (cp_evaluate, each iteration of cp_plan and its
  * final one) return CP_ERR_CUDA between their main kernel and the launch that sums its results, as
  * if that launch had failed. n = 0 turns it off; no other effect. */

@@ -151,6 +151,7 @@ _SIGS = {
     "cp_launch_count": (ctypes.c_int64, []),
     "cp_debug_fail_allocations": (None, [ctypes.c_int32]),
     "cp_debug_fail_evaluations": (None, [ctypes.c_int32]),
+    "cp_debug_withhold_factor": (None, [ctypes.c_int32]),
     "cp_debug_static_withhold_staging": (None, [ctypes.c_int32]),
     "cp_plan_init": (ctypes.c_int, [ctypes.POINTER(cp_model), ctypes.POINTER(cp_scene),
                                     ctypes.POINTER(cp_params), _P, ctypes.POINTER(_P)]),
@@ -335,6 +336,10 @@ def cp_debug_fail_allocations(n: int) -> None:
 
 def cp_debug_fail_evaluations(n: int) -> None:
     load().cp_debug_fail_evaluations(int(n))
+
+
+def cp_debug_withhold_factor(on: bool) -> None:
+    load().cp_debug_withhold_factor(1 if on else 0)
 
 
 def cp_debug_static_withhold_staging(on: bool) -> None:

@@ -23,6 +23,8 @@
 // Measured (factor and the two small copies of cp_set_distribution): 31.6 -> 24.8 us at D = 32,
 // 62.9 -> 41.4 at 64, 116.9 -> 62.9 at 96, 201.4 -> 87.9 at 128. An own column takes 870 cycles
 // (the pivot's chain); the last CTA's early columns, with up to 64 pairs, 1300 on average.
+#include <atomic>
+
 #include <cooperative_groups.h>
 
 #include "chain_launch.cuh"
@@ -54,9 +56,8 @@ __device__ __forceinline__ void send_double(const double *dst, uint64_t *bar, in
                  :: "r"(remote_addr(dst, rank)), "l"(__double_as_longlong(v)), "r"(remote_addr(bar, rank)) : "memory");
 }
 
-__device__ __forceinline__ bool wait_column(uint64_t *bar)
+__device__ __forceinline__ bool wait_column(uint64_t *bar, long long t0)
 {
-    const long long t0 = clock64();
     for (;;) {
         uint32_t ok;
         asm volatile("{\n\t.reg .pred p;\n\t"
@@ -89,9 +90,10 @@ __host__ __device__ inline size_t factor_smem(int n_ctas)
 }
 
 // Called by every thread of every CTA of the cluster (`n_ctas` CTAs; those past the last row
-// only take part in the barriers).
-__device__ __forceinline__ void factor_cluster(const double *C, double sigma2, int D, int n_ctas,
-                                               double *L, float *Lt, uint32_t *status, double *smem)
+// only take part in the barriers). withhold: the first CTA sends nothing of column 0, so that the
+// others' wait for it runs out on purpose (the test of this path).
+__device__ __forceinline__ void factor_cluster(const double *C, double sigma2, int D, int n_ctas, double *L,
+                                               float *Lt, uint32_t *status, double *smem, bool withhold)
 {
     const int b = (int)cooperative_groups::this_cluster().block_rank();
     const int n_used = (D + kRows - 1) / kRows, Dp = kRows * n_ctas;
@@ -138,11 +140,11 @@ __device__ __forceinline__ void factor_cluster(const double *C, double sigma2, i
                 if (j > k && !(k >= k0 && j == k + 1 && row == j)) *at = x;
             }
         };
-        publish(0, warp, kWarps);
+        if (!withhold) publish(0, warp, kWarps);
         __syncthreads();
         bool late = false;
         for (int k = 0; k < k0; ++k) {   // columns of the earlier CTAs
-            if (!late && !wait_column(bar + k)) {
+            if (!late && !wait_column(bar + k, clock64())) {
                 late = true;
                 atomicOr(status, DEV_ERR_TIMEOUT);
             }
@@ -178,7 +180,7 @@ __device__ __forceinline__ void factor_cluster(const double *C, double sigma2, i
                     const double u = U[(size_t)k * Dp + k + 1];
                     x = fma(-(u * dk), u, U[(size_t)(k + 1) * Dp + k + 1]);
                 }
-                if (lane > b && lane < n_used) {   // while the chain above runs
+                if (lane > b && lane < n_used && !(withhold && k == 0)) {   // while the chain above runs
                     send_double(s_d + k, bar + k, lane, dk);
                     send_double(s_v + k, bar + k, lane, vk);
                 }
@@ -199,19 +201,23 @@ __device__ __forceinline__ void factor_cluster(const double *C, double sigma2, i
             const double l = c < r ? U[(size_t)c * Dp + r] * s_s[c] : (c == r ? s_v[r] * s_s[r] : 0.0);
             Lt[(size_t)c * D + r] = (float)l;
         }
-        if (tid == 0 && s_bad) atomicOr(status, DEV_ERR_NOT_PD);
+        if (tid == 0 && s_bad && !late) atomicOr(status, DEV_ERR_NOT_PD);
+        if (late) {   // what the others still send arrives here: awaited too, with one limit for all
+            const long long t0 = clock64();
+            for (int k = 0; k < k0; ++k) wait_column(bar + k, t0);
+        }
     }
     cluster_barrier();   // no CTA leaves while a message to it or from it may be under way
 }
 
 __global__ void __launch_bounds__(kFactorThreads)
 k_factor(const double *C, double sigma2, const double *sigma_dev, int D, double *L,
-         float *Lt, uint32_t *status)
+         float *Lt, uint32_t *status, int withhold)
 {
     after_previous();
     extern __shared__ __align__(16) double sm[];
     if (sigma_dev != nullptr) sigma2 = sigma_dev[0] * sigma_dev[0];   // the step size kept on the device
-    factor_cluster(C, sigma2, D, (int)gridDim.x, L, Lt, status, sm);
+    factor_cluster(C, sigma2, D, (int)gridDim.x, L, Lt, status, sm, withhold != 0);
 }
 
 // The factors of every query of a batch, one cluster per query.
@@ -220,8 +226,10 @@ k_batch_factor_cluster(const BatchQueryDev *__restrict__ qd, int n_ctas)
 {
     extern __shared__ __align__(16) double sm[];
     const BatchQueryDev &q = qd[blockIdx.x / n_ctas];
-    factor_cluster(q.C, q.sigma2, q.D, n_ctas, q.L, q.Lt, q.status, sm);
+    factor_cluster(q.C, q.sigma2, q.D, n_ctas, q.L, q.Lt, q.status, sm, false);
 }
+
+std::atomic<int> g_withhold_factor{0};   // test hook
 
 struct ClusterLaunch {
     cudaLaunchAttribute attr[2] = {};
@@ -257,7 +265,7 @@ int launch_factor(const double *C, double sigma2, const double *sigma_dev, int D
 {
     const int n_ctas = (D + kRows - 1) / kRows;
     const ClusterLaunch l(n_ctas, n_ctas, st, true);
-    CP_CUDA(cudaLaunchKernelEx(&l.cfg, k_factor, C, sigma2, sigma_dev, D, L, Lt_f, status));
+    CP_CUDA(cudaLaunchKernelEx(&l.cfg, k_factor, C, sigma2, sigma_dev, D, L, Lt_f, status, g_withhold_factor.load()));
     CP_LAUNCHED("k_factor");
     return CP_OK;
 }
@@ -280,3 +288,5 @@ int launch_batch_factor_cluster(const BatchQueryDev *qd, int nq, int max_D, cuda
 }
 
 }  // namespace cp
+
+extern "C" void cp_debug_withhold_factor(int32_t on) { cp::g_withhold_factor.store(on != 0); }

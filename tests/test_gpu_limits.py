@@ -126,3 +126,33 @@ def test_calls_after_a_failed_evaluation(lib, crane, form, stream):
         lib.cp_set_endpoints(pl.handle, Q0, QD)
         ctrl, stats = lib.cp_plan(pl.handle, 3, K=K)
         assert np.array_equal(ctrl, want_plan[0]) and stats == want_plan[1]
+
+
+@pytest.mark.parametrize("K", [5, 8, 32])
+def test_factor_whose_message_is_missing(lib, crane, K):
+    """One message between the factor's blocks withheld: their wait ends by its limit, the call after
+    reports it, and the next factor is right."""
+    import torch
+    from paper_2503_14160_gb300 import workloads
+    D = 4 * K
+    g = np.random.default_rng(K)
+    A = g.normal(size=(D, D + 3))
+    mu, C = torch.zeros(D, dtype=torch.float64, device="cuda"), torch.from_numpy(A @ A.T).cuda()
+    L = [torch.empty(D, D, dtype=torch.float64, device="cuda") for _ in range(2)]
+    with lib.Planner(crane, workloads.empty_scene(), lib.make_params(64, K, 2)) as pl:
+        lib.cp_set_endpoints(pl.handle, Q0, QD)
+        lib.cp_set_distribution(pl.handle, mu, C, 1)
+        lib.cp_get_factor(pl.handle, L[0])
+        lib.cp_synchronize(pl.handle)
+        lib.cp_debug_withhold_factor(True)
+        try:
+            lib.cp_set_distribution(pl.handle, mu, C, 1)
+        finally:
+            lib.cp_debug_withhold_factor(False)
+        with pytest.raises(lib.CranePlanError) as e:
+            lib.cp_synchronize(pl.handle)
+        assert e.value.status == -3
+        lib.cp_set_distribution(pl.handle, mu, C, 1)
+        lib.cp_get_factor(pl.handle, L[1])
+        lib.cp_synchronize(pl.handle)
+        assert torch.equal(L[0], L[1])
