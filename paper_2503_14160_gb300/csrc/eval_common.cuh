@@ -89,8 +89,10 @@ static __device__ __forceinline__ float round_even(float v)
     return __fadd_rn(__fadd_rn(v, kRoundShift), -kRoundShift);
 }
 
-// The integer next to v (ties to even), saturating outwards: monotone in v for every v (the bits of
-// floats of one sign are), far values beyond any index either way.
+// The integer next to v (ties to even) for |v| < 2^22. From there up to any positive v the result only
+// grows (the bits of positive floats do), beyond any index; below -1.5 x 2^23 the sum turns negative
+// and the difference of the bits is no index, so callers pass no such v: a ring's distance less the
+// reach of one obstacle and an angle on [-pi, pi], in units of a cell, lie far above it.
 static __device__ __forceinline__ int round_index(float v)
 {
     return __float_as_int(__fadd_rn(v, kRoundShift)) - 0x4B400000;

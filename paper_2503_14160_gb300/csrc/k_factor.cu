@@ -12,17 +12,18 @@
 // each: the split below does not change a bit. CTA b of the cluster owns rows 16 b .. 16 b + 15
 // and keeps them in shared memory (a warp instruction holds 16 rows x 2 neighbouring columns, the
 // column pairs dealt to the warps; in registers the pairs that are finished cost their FP64
-// instruction all the same, as the compiler makes the choice by selects). Row i needs column k of rows j <= i only, so data flows one way, from a
-// CTA to the later ones: before step k a CTA sends its 16 entries of column k, and the owner of
-// pivot k also sends 1 / a_kk and a_kk, by st.async into the receivers' shared memory, which
+// instruction all the same, as the compiler makes the choice by selects). Row i needs column k of
+// rows j <= i only, so data flows one way, from a CTA to the later ones: before step k a CTA sends
+// its 16 entries of column k, and the owner of pivot k also sends 1 / a_kk and a_kk, by st.async into the receivers' shared memory, which
 // completes on the receivers' mbarrier of column k. Within its own 16 columns a CTA has the
 // pivots to itself: warp 0 works one column ahead on the reciprocal, on the scheduler that has
 // one worker warp instead of two, while the workers apply the current column; one block barrier
 // per column. Each wait for another CTA has a limit and ends in DEV_ERR_TIMEOUT.
 //
 // Measured (factor and the two small copies of cp_set_distribution): 31.6 -> 24.8 us at D = 32,
-// 62.9 -> 41.4 at 64, 116.9 -> 62.9 at 96, 201.4 -> 87.9 at 128. An own column takes 870 cycles
-// (the pivot's chain); the last CTA's early columns, with up to 64 pairs, 1300 on average.
+// 62.9 -> 41.4 at 64, 116.9 -> 62.9 at 96, 201.4 -> 87.9 at 128. An own column takes 870 cycles:
+// the pivot's chain of 550, the shared-memory round trips and the block barrier; the last CTA's early
+// columns, with up to 64 pairs, 1300 on average.
 #include <atomic>
 
 #include <cooperative_groups.h>

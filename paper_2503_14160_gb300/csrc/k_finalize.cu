@@ -110,14 +110,11 @@ int launch_eval_finalize(const double *item_sum, const uint32_t *item_count, int
 {
     if (n == 0) return CP_OK;
     const int threads = 256, per = threads / kFinalLanes;
-    launch_chained(k_eval_finalize, (unsigned)((n + per - 1) / per), threads, 0, st,  item_sum, item_count, n, P, w_c, w_l, lambda_c, J, flag, terms, status, queue);
+    launch_chained(k_eval_finalize, (unsigned)((n + per - 1) / per), threads, 0, st, item_sum, item_count, n, P, w_c,
+                   w_l, lambda_c, J, flag, terms, status, queue);
     CP_LAUNCHED("k_eval_finalize");
     return CP_OK;
 }
-
-}  // namespace cp
-
-namespace cp {
 
 int launch_batch_finalize(const BatchQueryDev *qd, const int2 *tab, int blocks, const BatchEvalDev *mean_ev,
                           cudaStream_t st)

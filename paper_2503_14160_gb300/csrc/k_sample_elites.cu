@@ -506,10 +506,12 @@ int launch_sample_elites(const float *Yp, const float *mu_f, int N, int K, int n
     if (slices > chunks) slices = chunks;
     const PhiloxKeys key = philox_keys((uint32_t)seed, (uint32_t)(seed >> 32));
     dim3 grid((N + kTcM - 1) / kTcM, slices);
-    launch_chained(k_sample_elites, grid, kTcThreads + 32, tc_smem_bytes(Dp), st, Yp, N, D, chunks, slices, tmem_columns(Dp), key, iter, query, P, status, withhold ? 1 : 0);
+    launch_chained(k_sample_elites, grid, kTcThreads + 32, tc_smem_bytes(Dp), st, Yp, N, D, chunks, slices,
+                   tmem_columns(Dp), key, iter, query, P, status, withhold ? 1 : 0);
     CP_LAUNCHED("k_sample_elites");
     const int64_t total = (int64_t)N * (D / 4);
-    launch_chained(k_sample_reduce, (unsigned)((total + 255) / 256), 256, 0, st, P, slices, mu_f, N, D, nu, (float)(sigma * sqrt(eps)), key, iter, query, xi);
+    launch_chained(k_sample_reduce, (unsigned)((total + 255) / 256), 256, 0, st, P, slices, mu_f, N, D, nu,
+                   (float)(sigma * sqrt(eps)), key, iter, query, xi);
     CP_LAUNCHED("k_sample_reduce");
     return CP_OK;
 }

@@ -75,8 +75,6 @@ struct ChainSums {
 // One lane's view of its checkpoint for the pair terms.
 struct PairCtx {
     float c1, s1, c2, s2, c23, s23, q4, base_z;
-    const float4 *sph;                // [NSPH] {alpha, beta, gamma, -delta} in shared memory
-    const float *radius;              // [NSPH]
 };
 
 // Softplus term of sphere s (its centre at (x, y, z), h from the axis) against an obstacle at
@@ -226,8 +224,6 @@ k_smooth(const ModelDev m, const SceneDev sc, const SmoothArgs a)
             sincosf(q.y + q.z, &ctx.s23, &ctx.c23);
             ctx.q4 = q.w;
             ctx.base_z = m.base_z;
-            ctx.sph = s_sph;
-            ctx.radius = s_rad;
             const float c1 = ctx.c1, s1 = ctx.s1;
             const float extra = a.margin + kSmoothCut * a.beta;
             const float zreach = m.r_max + extra + kZGate;

@@ -518,8 +518,10 @@ k_radix_scatter(const unsigned long long *__restrict__ key_in, const int *__rest
 // tile histograms of the pass are there already (tile-major, hist[tile][digit]): every block sums
 // the columns it needs, the counts of its digits in the tiles before it and in all tiles, so no
 // scan kernel stands between, and while it scatters it counts the next pass's histograms at the
-// elements' new places (integer atomics). The sums read 1 KB per earlier tile and block, 2 MB in
-// all at 64 tiles and 33 MB at 256; beyond that the scan kernel is the cheaper form. The order is
+// elements' new places (integer atomics). The sums read 1 KB per tile in every block, 4 MB in all at
+// 64 tiles and 67 MB at 256 (from L2). An update of 2 elites, ranking included, takes 67 us at 65536
+// candidates, 117 at 196608 and 138 at 262144, the last size of this form, and 160 at 262145 with
+// three launches per pass; the reads grow with the square of the tiles. The order is
 // that of k_radix_scatter: stable, by warp and lane within the tile.
 // The three launches per pass it replaces were bound by launch latency (3.3 + 3.6 + 7.6 us for
 // 65536 keys, 64 blocks taking four dependent rounds).
@@ -862,7 +864,8 @@ int launch_gather_elites(const int *sorted, const double *J, const float *xi, in
                          int *elite, float *elites, double *best_J, cudaStream_t st)
 {
     const int threads = 256;
-    launch_chained(k_gather_elites, (nu * 32 + threads - 1) / threads, threads, 0, st, sorted, J, xi, nu, D, elite, elites, best_J);
+    launch_chained(k_gather_elites, (nu * 32 + threads - 1) / threads, threads, 0, st, sorted, J, xi, nu, D, elite,
+                   elites, best_J);
     CP_LAUNCHED("k_gather_elites");
     return CP_OK;
 }
@@ -973,11 +976,13 @@ int launch_cma_update(const float *elites, const double *w, int nu, int D, doubl
     int rc = launch_moments_partial(elites, w, nu, D, yw, s2p, s1p, &n_chunks, st);
     if (rc != CP_OK) return rc;
     const size_t smem = sizeof(double) * (size_t)D * (D + 1);
-    launch_chained(k_cma_paths, 1, kCmaThreads, smem, st, s1p, n_chunks, D, elites, mu_prev, L, k, std::sqrt(1.0 - std::pow(1.0 - k.c_sigma, 2.0 * (t + 1))),
+    const double path_len = std::sqrt(1.0 - std::pow(1.0 - k.c_sigma, 2.0 * (t + 1)));
+    launch_chained(k_cma_paths, 1, kCmaThreads, smem, st, s1p, n_chunks, D, elites, mu_prev, L, k, path_len,
                    (1.4 + 2.0 / (D + 1)) * k.chi_n, mu, p_sigma, p_c, cma);
     CP_LAUNCHED("k_cma_paths");
     const int entries = D * (D + 1) / 2;
-    launch_chained(k_cma_cov, (entries * kSumLanes + 127) / 128, 128, 0, st, s2p, s1p, n_chunks, D, elites, mu_prev, p_c, cma, k, C);
+    launch_chained(k_cma_cov, (entries * kSumLanes + 127) / 128, 128, 0, st, s2p, s1p, n_chunks, D, elites, mu_prev,
+                   p_c, cma, k, C);
     CP_LAUNCHED("k_cma_cov");
     return CP_OK;
 }
