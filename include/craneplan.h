@@ -225,7 +225,7 @@ void cp_debug_fail_allocations(int32_t n);
 
 /* Test hook: while on, a planner's factor kernel withholds one message between its thread blocks
  * (from 20 rows on), so that a bounded wait runs out: the next host-synchronising call returns
- * CP_ERR_TIMEOUT. No other effect. */
+ * CP_ERR_TIMEOUT (launches recorded while it is on keep it). No other effect. */
 void cp_debug_withhold_factor(int32_t on);
 
 /* Test hook: the next n evaluations of a planner (cp_evaluate, each iteration of cp_plan and its
